@@ -320,6 +320,10 @@ static int gauge_upload(bridge_lattice L, const double* U, const bridge_op* op, 
   BR_CUDA(cudaStreamSynchronize(L->stream));
   for (int p = 0; p < 4; ++p) L->gauge[p].reset();
   {
+    std::lock_guard<std::mutex> lk(L->fx_mu);
+    L->gauge_fx = FxCopy{};
+  }
+  {
     std::lock_guard<std::mutex> lk(L->clover_mu);
     L->clovers.clear();
   }

@@ -65,6 +65,14 @@ struct HopArgs {
   // blocking); the other sites are neither read nor written.
   const uint32_t* site_map;
   uint32_t n_map;
+  // FP64 only, non-null when the fixed-point kernel may run (dslash_fx.cuh):
+  // the same links and clover blocks as 64-bit fixed-point numbers.
+  const char* gauge_fx;
+  const char* clovE_fx;
+  const char* clovM_fx;
+  int eE_fx, eM_fx;  // their exponents: entries below 2^e
+  const char* in_fx;  // `in` in fixed point
+  long in_fx_rs;
 };
 
 template <class R, int MU, bool FWD>
@@ -177,6 +185,89 @@ BR_D void hop_dir(const HopArgs& a, const char* in, const char* g_out, const cha
   hop_one<P, MU, false, ST>(in, g_in + MU * lbb, a.g.vh, b, b, wb, bc, acc);
 }
 
+// The hop term of one output site and its epilogue: v = the output spinor, s
+// = the self spinor (F_SELF).
+template <int P, int FL, bool ST>
+BR_D void hop_site(const HopArgs& a, int rhs, uint32_t ih, const int c[4], uint32_t xh, cx<typename Tr<P>::R> v[12],
+                   cx<typename Tr<P>::R> s[12]) {
+  using R = typename Tr<P>::R;
+  const R beta = pick<R>(a.beta, a.betaf), s1 = pick<R>(a.s1, a.s1f), ca = pick<R>(a.caux, a.cauxf);
+  const int p = a.out_parity;
+  const long vh = a.g.vh, lbb = link_block_bytes(P, vh), cbb = clover_block_bytes(P, vh);
+  const char* g_out = a.gauge + (long)p * 4 * lbb;
+  const char* g_in = a.gauge + (long)(1 - p) * 4 * lbb;
+  const char* in = a.in + rhs * a.in_rs;
+  cx<R> acc[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k) acc[k] = czero<R>();
+  hop_dir<P, 0, ST>(a, in, g_out, g_in, lbb, ih, c, xh, acc);
+  hop_dir<P, 1, ST>(a, in, g_out, g_in, lbb, ih, c, xh, acc);
+  hop_dir<P, 2, ST>(a, in, g_out, g_in, lbb, ih, c, xh, acc);
+  hop_dir<P, 3, ST>(a, in, g_out, g_in, lbb, ih, c, xh, acc);
+#pragma unroll
+  for (int k = 0; k < 12; ++k) acc[k] = beta * acc[k];
+  if (FL & F_AUX) {
+    cx<R> x[12];
+    load_spinor<P, true, ST>(a.aux + rhs * a.aux_rs, vh, ih, x);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) acc[k] = acc[k] + ca * x[k];
+  }
+  if (FL & F_G5) {
+#pragma unroll
+    for (int k = 6; k < 12; ++k) acc[k] = cx<R>{-acc[k].r, -acc[k].i};
+  }
+  if (FL & F_E_CLOV) {
+    clover_apply<P, ST>(a.clovE + p * cbb, vh, ih, acc, v);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 12; ++k) v[k] = acc[k];
+  }
+  if (FL & F_SELF) {
+    load_spinor<P, true, ST>(a.self + rhs * a.self_rs, vh, ih, s);
+    if (FL & F_SELF_CLOV) {
+      cx<R> ms[12];
+      clover_apply<P, ST>(a.clovM + p * cbb, vh, ih, s, ms);
+#pragma unroll
+      for (int k = 0; k < 12; ++k) v[k] = v[k] + s1 * ms[k];
+    } else {
+#pragma unroll
+      for (int k = 0; k < 12; ++k) v[k] = v[k] + s1 * s[k];
+    }
+  }
+}
+
+// One site's contribution to the fused reduction.
+template <int P, int RED, bool ST, class PS>
+BR_D void hop_reduce(const HopArgs& a, int rhs, uint32_t ih, const cx<typename Tr<P>::R> v[12],
+                     const cx<typename Tr<P>::R> s[12], PS* ps) {
+  using R = typename Tr<P>::R;
+  if (RED == R_NORM) {
+    R n = 0;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) n += v[k].r * v[k].r + v[k].i * v[k].i;
+    ps[0].add(n);
+  } else if (RED == R_DOT_A) {
+    cx<R> w[12];
+    load_spinor<P, true, ST>(a.avec + rhs * a.avec_rs, a.g.vh, ih, w);
+    cx<R> d = czero<R>();
+#pragma unroll
+    for (int k = 0; k < 12; ++k) d = d + cmul_conj(w[k], v[k]);
+    ps[0].add(d.r);
+    ps[1].add(d.i);
+  } else if (RED == R_TS) {
+    cx<R> d = czero<R>();
+    R n = 0;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      d = d + cmul_conj(v[k], s[k]);
+      n += v[k].r * v[k].r + v[k].i * v[k].i;
+    }
+    ps[0].add(d.r);
+    ps[1].add(d.i);
+    ps[2].add(n);
+  }
+}
+
 // MINB: minimum resident 256-thread blocks per SM the compiler must allow
 // (1 = no register cap, 3 = <= 80 registers, 4 = <= 64 registers); ST:
 // load the read-once operands around L1 (see ldg4).  The autotuner picks
@@ -190,14 +281,9 @@ __global__ void __launch_bounds__(256, MINB) hop_kernel(const HopArgs a) {
   const long vh = a.g.vh;
   constexpr int NV = RED == R_NORM ? 1 : RED == R_DOT_A ? 2 : 3;
   PartialSum<R> ps[NV];
-  const R beta = pick<R>(a.beta, a.betaf), s1 = pick<R>(a.s1, a.s1f), ca = pick<R>(a.caux, a.cauxf);
   const bool skip = rhs_finished(a.red, rhs);
   if (!skip) {
     const int p = a.out_parity;
-    const long lbb = link_block_bytes(P, vh), cbb = clover_block_bytes(P, vh);
-    const char* g_out = a.gauge + (long)p * 4 * lbb;
-    const char* g_in = a.gauge + (long)(1 - p) * 4 * lbb;
-    const char* in = a.in + rhs * a.in_rs;
     const uint32_t stride = (uint32_t)a.nblk * blockDim.x;
     const uint32_t nsite = a.site_map ? a.n_map : (uint32_t)vh;
     for (uint32_t k = sb * blockDim.x + threadIdx.x; k < nsite; k += stride) {
@@ -205,71 +291,10 @@ __global__ void __launch_bounds__(256, MINB) hop_kernel(const HopArgs a) {
       int c[4];
       uint32_t xh;
       site_coords(a.g, ih, p, c, xh);
-      cx<R> acc[12];
-#pragma unroll
-      for (int k = 0; k < 12; ++k) acc[k] = czero<R>();
-      hop_dir<P, 0, ST>(a, in, g_out, g_in, lbb, ih, c, xh, acc);
-      hop_dir<P, 1, ST>(a, in, g_out, g_in, lbb, ih, c, xh, acc);
-      hop_dir<P, 2, ST>(a, in, g_out, g_in, lbb, ih, c, xh, acc);
-      hop_dir<P, 3, ST>(a, in, g_out, g_in, lbb, ih, c, xh, acc);
-#pragma unroll
-      for (int k = 0; k < 12; ++k) acc[k] = beta * acc[k];
-      if (FL & F_AUX) {
-        cx<R> x[12];
-        load_spinor<P, true, ST>(a.aux + rhs * a.aux_rs, vh, ih, x);
-#pragma unroll
-        for (int k = 0; k < 12; ++k) acc[k] = acc[k] + ca * x[k];
-      }
-      if (FL & F_G5) {
-#pragma unroll
-        for (int k = 6; k < 12; ++k) acc[k] = cx<R>{-acc[k].r, -acc[k].i};
-      }
-      cx<R> v[12];
-      if (FL & F_E_CLOV) {
-        clover_apply<P, ST>(a.clovE + p * cbb, vh, ih, acc, v);
-      } else {
-#pragma unroll
-        for (int k = 0; k < 12; ++k) v[k] = acc[k];
-      }
-      cx<R> s[12];
-      if (FL & F_SELF) {
-        load_spinor<P, true, ST>(a.self + rhs * a.self_rs, vh, ih, s);
-        if (FL & F_SELF_CLOV) {
-          cx<R> ms[12];
-          clover_apply<P, ST>(a.clovM + p * cbb, vh, ih, s, ms);
-#pragma unroll
-          for (int k = 0; k < 12; ++k) v[k] = v[k] + s1 * ms[k];
-        } else {
-#pragma unroll
-          for (int k = 0; k < 12; ++k) v[k] = v[k] + s1 * s[k];
-        }
-      }
+      cx<R> v[12], s[12];
+      hop_site<P, FL, ST>(a, rhs, ih, c, xh, v, s);
       store_spinor<P>(a.out + rhs * a.out_rs, vh, ih, v);
-      if (RED == R_NORM) {
-        R n = 0;
-#pragma unroll
-        for (int k = 0; k < 12; ++k) n += v[k].r * v[k].r + v[k].i * v[k].i;
-        ps[0].add(n);
-      } else if (RED == R_DOT_A) {
-        cx<R> w[12];
-        load_spinor<P, true, ST>(a.avec + rhs * a.avec_rs, vh, ih, w);
-        cx<R> d = czero<R>();
-#pragma unroll
-        for (int k = 0; k < 12; ++k) d = d + cmul_conj(w[k], v[k]);
-        ps[0].add(d.r);
-        ps[1].add(d.i);
-      } else if (RED == R_TS) {
-        cx<R> d = czero<R>();
-        R n = 0;
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-          d = d + cmul_conj(v[k], s[k]);
-          n += v[k].r * v[k].r + v[k].i * v[k].i;
-        }
-        ps[0].add(d.r);
-        ps[1].add(d.i);
-        ps[2].add(n);
-      }
+      hop_reduce<P, RED, ST>(a, rhs, ih, v, s, ps);
     }
   }
   if (RED != R_NONE) {

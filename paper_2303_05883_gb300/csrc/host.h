@@ -109,7 +109,9 @@ struct Field {
     return buf->ptr + ((subset == BRIDGE_FULL && parity == 1) ? block : 0);
   }
 };
-Field make_field(int prec, int subset, int nrhs, long vh, cudaStream_t st = nullptr, bool stream_ordered = false);
+// at_least: bytes the buffer holds at the least.
+Field make_field(int prec, int subset, int nrhs, long vh, cudaStream_t st = nullptr, bool stream_ordered = false,
+                 size_t at_least = 0);
 
 // ----------------------------------------------------------- tuning
 // Launch shapes picked per (kernel class, precision, flags, lattice, nrhs).
@@ -132,6 +134,15 @@ struct Stats {
   std::vector<cudaEvent_t> pool;
 };
 
+// The fixed-point copy of FP64 operator data (dslash_fx.cuh): built on first
+// use, or found unsuitable (an entry out of its range, no memory for it).
+struct FxCopy {
+  enum State { UNKNOWN, READY, UNSUITABLE };
+  State state = UNKNOWN;
+  int e = 0;  // entries are below 2^e (links: at most 1), their unit 2^(e - 60)
+  std::unique_ptr<DevBuf> buf;
+};
+
 // Clover term T = 1 - kcsw sum sigma F and its inverse for one value of
 // kcsw = kappa c_sw: FP64 masters plus lazily converted copies.  Shared by
 // the solves that use it, so a solve keeps its set alive even after the
@@ -139,6 +150,7 @@ struct Stats {
 struct CloverSet {
   double kcsw = 0.0;
   std::unique_ptr<DevBuf> T[4], Tinv[4];
+  FxCopy Tfx, Tinvfx;
   std::mutex mu;
 };
 
@@ -178,6 +190,9 @@ struct bridge_lattice_s {
   cudaStream_t stream = nullptr;
   // links per precision; [0] (F64, 18 reals) is the master copy
   std::unique_ptr<bridge::DevBuf> gauge[4];
+  bridge::FxCopy gauge_fx;  // the FP64 links in fixed point
+  std::mutex fx_mu;
+  std::unique_ptr<bridge::DevBuf> fx_scratch;  // hop inputs in fixed point, for work on the lattice stream
   bool have_gauge = false;
   // clover sets for the most recently used values of kappa * c_sw
   std::vector<std::shared_ptr<bridge::CloverSet>> clovers;
@@ -223,6 +238,16 @@ const char* gauge_ptr(bridge_lattice_s* L, int prec);
 std::shared_ptr<CloverSet> clover_set(bridge_lattice_s* L, double kcsw);
 const char* clover_ptr(bridge_lattice_s* L, CloverSet& set, int prec, bool inverse);
 const char* clover_ptr(bridge_lattice_s* L, int prec, bool inverse, double kcsw);
+// The fixed-point copies of the FP64 links and clover blocks, or nullptr
+// where there is none and the FP64 kernels have to run: entries out of the
+// fixed-point range, no memory for the copy, or not built yet while st is
+// being captured into a graph.
+const char* gauge_fx_ptr(bridge_lattice_s* L, cudaStream_t st);
+const char* clover_fx_ptr(bridge_lattice_s* L, CloverSet& set, bool inverse, cudaStream_t st, int* e = nullptr);
+// Set the fixed-point pointers of an FP64 launch on stream st (set: the
+// clover set of the flags that need one; scratch as HopCall::fx_scratch) and
+// queue the conversion of its input; or leave them null.
+void set_fx_args(bridge_lattice_s* L, HopArgs& a, int flags, int red, CloverSet* set, char* scratch, cudaStream_t st);
 
 // ------------------------------------------------------- operators
 // Apply one hop-kernel variant (see dslash.cuh).  Field pointers are the
@@ -241,6 +266,8 @@ struct HopCall {
   RedArgs redargs{};
   const uint32_t* site_map = nullptr;  // HopArgs::site_map / n_map: a subset of the output sites
   uint32_t n_map = 0;
+  char* fx_scratch = nullptr;  // FP64: room for nrhs blocks of fx_block_bytes (default: the lattice's, for
+                               // work on the lattice stream; elsewhere the launch stays on the FP64 kernel)
   double work_fraction = 1.0;  // share of the sites the launch computes (for the byte and flop counts)
 };
 void run_hop(bridge_lattice_s* L, HopCall c, cudaStream_t st);

@@ -83,5 +83,11 @@ bool launch_gauge_convert(int prec, const Geom& g, const char* g64, char* gp, cu
 // Clover term T = 1 - kcsw * sum sigma F and its inverse, packed FP64 [parity].
 void launch_clover_build(const Geom& g, const char* g64, double kcsw, char* T64, char* Tinv64, cudaStream_t st);
 bool launch_clover_convert(int prec, const Geom& g, const char* c64, char* cp, cudaStream_t st);
+// FP64 half-lattice field src -> its fixed-point form dst (fx_block_bytes each).
+void launch_field_to_fx(const CopyArgs& a, int block, cudaStream_t st);
+// nb blocks, block_bytes apart, of n 16-byte entries (two doubles of magnitude
+// up to 2^e) -> the fixed-point form of dslash_fx.cuh, |entry| 2^(60 - e);
+// *top = the largest high word of an |entry|.
+void launch_to_fx(const char* src, char* dst, int nb, long n, long block_bytes, int e, uint32_t* top, cudaStream_t st);
 
 }  // namespace bridge

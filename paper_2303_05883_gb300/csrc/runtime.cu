@@ -4,6 +4,7 @@
 #include <cstring>
 #include <string>
 
+#include "dslash_fx.cuh"
 #include "host.h"
 
 namespace bridge {
@@ -75,7 +76,7 @@ DevBuf::~DevBuf() {
     cudaFree(ptr);
 }
 
-Field make_field(int prec, int subset, int nrhs, long vh, cudaStream_t st, bool stream_ordered) {
+Field make_field(int prec, int subset, int nrhs, long vh, cudaStream_t st, bool stream_ordered, size_t at_least) {
   Field f;
   f.prec = prec;
   f.subset = subset;
@@ -83,7 +84,7 @@ Field make_field(int prec, int subset, int nrhs, long vh, cudaStream_t st, bool 
   f.vh = vh;
   f.block = spinor_block_bytes(prec, vh);
   f.rs = (subset == BRIDGE_FULL ? 2 : 1) * f.block;
-  f.buf = std::make_shared<DevBuf>((size_t)(f.rs * (nrhs > 0 ? nrhs : 1)), st, stream_ordered);
+  f.buf = std::make_shared<DevBuf>(std::max((size_t)(f.rs * (nrhs > 0 ? nrhs : 1)), at_least), st, stream_ordered);
   return f;
 }
 
@@ -221,6 +222,111 @@ const char* clover_ptr(bridge_lattice_s* L, int prec, bool inverse, double kcsw)
   return clover_ptr(L, *s, prec, inverse);
 }
 
+static bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const bool known = cudaStreamIsCapturing(st, &cap) == cudaSuccess;
+  if (!known) cudaGetLastError();
+  return !known || cap != cudaStreamCaptureStatusNone;
+}
+
+// The copy is made on the lattice stream, which orders it after the FP64
+// data, and waited for: other streams may read it next.  top(e): the high
+// word an entry must stay below for exponent e; e from `elo` to `ehi`.
+static const char* fx_copy(bridge_lattice_s* L, FxCopy& fx, const DevBuf& src, int nb, long block_bytes, long n, int elo,
+                           int ehi, const std::function<uint32_t(int)>& top, cudaStream_t st) {
+  if (fx.state == FxCopy::READY) return fx.buf->ptr;
+  if (fx.state == FxCopy::UNSUITABLE || capturing(st) || capturing(L->stream)) return nullptr;
+  fx.state = FxCopy::UNSUITABLE;
+  // leave the memory to the fields of a solve (up to 4 KB a site, seven link
+  // copies) where it is scarce
+  size_t free_b = 0, total_b = 0;
+  BR_CUDA(cudaMemGetInfo(&free_b, &total_b));
+  if (src.bytes > free_b / 8) return nullptr;
+  std::unique_ptr<DevBuf> buf;
+  try {
+    buf.reset(new DevBuf(src.bytes + 256));  // (the last 256 bytes: the largest entry met)
+  } catch (const Error&) {
+    return nullptr;
+  }
+  uint32_t* word = reinterpret_cast<uint32_t*>(buf->ptr + src.bytes);
+  for (int e = elo; e <= ehi; ++e) {
+    uint32_t seen = 0;
+    BR_CUDA(cudaMemsetAsync(word, 0, 256, L->stream));
+    note_launch(L, K_SETUP, 2.0 * src.bytes, 0, L->stream, true);
+    launch_to_fx(src.ptr, buf->ptr, nb, n, block_bytes, e, word, L->stream);
+    note_launch(L, K_SETUP, 0, 0, L->stream, false);
+    BR_CUDA(cudaGetLastError());
+    BR_CUDA(cudaMemcpyAsync(&seen, word, sizeof(seen), cudaMemcpyDeviceToHost, L->stream));
+    BR_CUDA(cudaStreamSynchronize(L->stream));
+    if (seen < top(e)) {
+      fx.buf = std::move(buf);
+      fx.e = e;
+      fx.state = FxCopy::READY;
+      return fx.buf->ptr;
+    }
+    if (seen >= top(ehi)) break;
+  }
+  return nullptr;
+}
+
+const char* gauge_fx_ptr(bridge_lattice_s* L, cudaStream_t st) {
+  std::lock_guard<std::mutex> lk(L->fx_mu);
+  return fx_copy(L, L->gauge_fx, *L->gauge[P_F64], 8, link_block_bytes(P_F64, L->vh), 9 * L->vh, 0, 0,
+                 [](int) { return FX_LINK_TOP; }, st);
+}
+
+const char* clover_fx_ptr(bridge_lattice_s* L, CloverSet& set, bool inverse, cudaStream_t st, int* e) {
+  std::lock_guard<std::mutex> lk(set.mu);
+  FxCopy& fx = inverse ? set.Tinvfx : set.Tfx;
+  const char* p = fx_copy(L, fx, inverse ? *set.Tinv[P_F64] : *set.T[P_F64], 2, clover_block_bytes(P_F64, L->vh),
+                          36 * L->vh, 1, FX_CLOV_EMAX, fx_clov_top, st);
+  if (e) *e = fx.e;
+  return p;
+}
+
+void set_fx_args(bridge_lattice_s* L, HopArgs& a, int flags, int red, CloverSet* set, char* scratch, cudaStream_t st) {
+  a.gauge_fx = a.clovE_fx = a.clovM_fx = nullptr;
+  if (!fx_has(flags, red)) return;
+  const size_t need = (size_t)a.nrhs * fx_block_bytes(L->vh);
+  if (!scratch && st != L->stream) return;
+  const char* E = (flags & F_E_CLOV) ? clover_fx_ptr(L, *set, true, st, &a.eE_fx) : nullptr;
+  const char* M = (flags & F_SELF_CLOV) ? clover_fx_ptr(L, *set, false, st, &a.eM_fx) : nullptr;
+  if (((flags & F_E_CLOV) && !E) || ((flags & F_SELF_CLOV) && !M)) return;
+  const char* U = gauge_fx_ptr(L, st);
+  if (!U) return;
+  if (!scratch) {
+    if (!L->fx_scratch || L->fx_scratch->bytes < need) {
+      if (capturing(st)) return;
+      L->fx_scratch.reset();
+      try {
+        L->fx_scratch.reset(new DevBuf(need));
+      } catch (const Error&) {
+        return;  // no room: the FP64 kernel needs none
+      }
+    }
+    scratch = L->fx_scratch->ptr;
+  }
+  CopyArgs c;
+  std::memset(&c, 0, sizeof(c));
+  c.vh = (uint32_t)L->vh;
+  c.nrhs = a.nrhs;
+  c.nblk = (int)((L->vh + 255) / 256);
+  c.src = a.in;
+  c.src_rs = a.in_rs;
+  c.dst = scratch;
+  c.dst_rs = fx_block_bytes(L->vh);
+  c.red = a.red;  // right-hand sides whose solve has ended are skipped
+  const double bytes = (double)L->vh * a.nrhs * (192 + 196);
+  note_launch(L, K_CONVERT, bytes, 0, st, true);
+  launch_field_to_fx(c, 256, st);
+  note_launch(L, K_CONVERT, bytes, 0, st, false);
+  a.in_fx = scratch;
+  a.in_fx_rs = c.dst_rs;
+  a.gauge_fx = U;
+  a.clovE_fx = E;
+  a.clovM_fx = M;
+}
+
 // ------------------------------------------------------------ operators
 static long spinor_site_bytes(int prec) { return prec == P_F64 ? 192 : prec == P_F32 ? 96 : 52; }
 static long link_site_bytes(int prec) { return prec == P_F64 ? 144 : prec == P_F32 ? 48 : 24; }
@@ -270,9 +376,9 @@ void run_hop(bridge_lattice_s* L, HopCall c, cudaStream_t st) {
   a.avec = c.avec;
   a.avec_rs = c.avec_rs;
   a.gauge = gauge_ptr(L, c.prec);
+  std::shared_ptr<CloverSet> keep;
+  CloverSet* cs = c.clov;
   if (c.flags & (F_E_CLOV | F_SELF_CLOV)) {
-    std::shared_ptr<CloverSet> keep;
-    CloverSet* cs = c.clov;
     if (!cs) {
       keep = clover_set(L, c.kcsw);
       cs = keep.get();
@@ -280,6 +386,8 @@ void run_hop(bridge_lattice_s* L, HopCall c, cudaStream_t st) {
     a.clovE = (c.flags & F_E_CLOV) ? clover_ptr(L, *cs, c.prec, true) : nullptr;
     a.clovM = (c.flags & F_SELF_CLOV) ? clover_ptr(L, *cs, c.prec, false) : nullptr;
   }
+  a.red = c.redargs;
+  if (c.prec == P_F64 && !c.site_map) set_fx_args(L, a, c.flags, c.red, cs, c.fx_scratch, st);
   const std::string key = "hop/" + std::to_string(c.prec) + "/" + std::to_string(c.flags) + "/" +
                           std::to_string(c.red) + "/" + dims_key(L) + "/" + std::to_string(c.nrhs);
   LaunchShape sh = shape_for(L, key, L->vh, c.nrhs, [&](int block) {
@@ -288,9 +396,10 @@ void run_hop(bridge_lattice_s* L, HopCall c, cudaStream_t st) {
     return n;
   });
   a.nblk = sh.nblk;
-  a.red = c.redargs;
   if (c.red != R_NONE && a.red.partials == nullptr) {
-    ensure_red_scratch(L, (long)sh.nblk * c.nrhs, c.nrhs);
+    // a fixed-point launch takes up to one block for 64 sites
+    const long nb = a.gauge_fx ? std::max<long>(sh.nblk, (L->vh + 63) / 64) : sh.nblk;
+    ensure_red_scratch(L, nb * c.nrhs, c.nrhs);
     a.red.partials = reinterpret_cast<double*>(L->red_partials->ptr);
     a.red.counter = reinterpret_cast<unsigned*>(L->red_counter->ptr);
     a.red.result = reinterpret_cast<double*>(L->red_result->ptr);

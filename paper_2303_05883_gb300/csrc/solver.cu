@@ -24,6 +24,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "dslash_fx.cuh"
 #include "solver.h"
 
 namespace bridge {
@@ -83,6 +84,9 @@ size_t solve_footprint(const bridge_lattice_s* L, const bridge_solver& prm, int 
                      + 7 * sP       // bh, r, rhat, p, v, s, t (even)
                      + sX + sP      // xin, xinp
                      + 2 * sP);     // tmp, eo (odd)
+  // (of these, eo shares tmp's memory and xinp r's; the room left takes the fixed-point input of the FP64 hops)
+  const double fx = (double)fx_block_bytes(vh);
+  b += nrhs * std::max(0.0, P == P_F64 ? fx - 2 * sP : fx - sP - 2 * sP);
   b += nrhs * 2.0 * 2 * s64;        // canonical b and x held by the engine
   b += (double)nrhs * ((vh + 63) / 64) * 4 * 8 + 65536;
   return (size_t)b;
@@ -116,13 +120,17 @@ SolveState::SolveState(bridge_lattice_s* L, const bridge_op& op, const bridge_so
   r_ = make_field(P_, BRIDGE_EVEN, nrhs, vh, st_, true);
   rhat_ = make_field(P_, BRIDGE_EVEN, nrhs, vh, st_, true);
   p_ = make_field(P_, BRIDGE_EVEN, nrhs, vh, st_, true);
-  v_ = make_field(P_, BRIDGE_EVEN, nrhs, vh, st_, true);
   s_ = make_field(P_, BRIDGE_EVEN, nrhs, vh, st_, true);
   t_ = make_field(P_, BRIDGE_EVEN, nrhs, vh, st_, true);
   xin_ = make_field(PX_, BRIDGE_EVEN, nrhs, vh, st_, true);
-  if (PX_ != P_) xinp_ = make_field(P_, BRIDGE_EVEN, nrhs, vh, st_, true);
+  if (PX_ != P_) xinp_ = r_;  // the solution is read out when the iteration's vectors are done with
   tmp_ = make_field(P_, BRIDGE_ODD, nrhs, vh, st_, true);
-  eo_ = make_field(P_, BRIDGE_ODD, nrhs, vh, st_, true);
+  eo_ = tmp_;
+  // v: between the inner solves its memory holds the fixed-point input of the
+  // FP64 residual; a plain FP64 solve needs one beside it
+  const size_t fx_bytes = (size_t)nrhs * fx_block_bytes(vh);
+  v_ = make_field(P_, BRIDGE_EVEN, nrhs, vh, st_, true, P_ == P_F64 ? 0 : fx_bytes);
+  if (P_ == P_F64) fxs_.reset(new DevBuf(fx_bytes, st_, true));
   scal_.reset(new DevBuf(sizeof(BiCGScalars) * nrhs, st_, true));
   partials_.reset(new DevBuf((size_t)nrhs * ((vh + 63) / 64) * 4 * sizeof(double), st_, true));
   counter_.reset(new DevBuf(256, st_, true));
@@ -153,7 +161,10 @@ SolveState::SolveState(bridge_lattice_s* L, const bridge_op& op, const bridge_so
     clov_ = clover_set(L_, kcsw_);
     clover_ptr(L_, *clov_, P_, true);
     clover_ptr(L_, *clov_, P_F64, false);
+    clover_fx_ptr(L_, *clov_, false, st_);
+    if (P_ == P_F64) clover_fx_ptr(L_, *clov_, true, st_);
   }
+  gauge_fx_ptr(L_, st_);
   if (st_ != L_->stream) BR_CUDA(cudaStreamSynchronize(L_->stream));
 }
 
@@ -189,6 +200,7 @@ void SolveState::enqueue_residual() {
   for (int q = 0; q < 2; ++q) {
     HopCall c;
     c.prec = P_F64;
+    c.fx_scratch = fx_scratch();
     c.flags = F_AUX | F_SELF | (clover_ ? F_SELF_CLOV : 0);
     c.red = R_NORM;
     c.cls = K_RESID;
@@ -280,6 +292,7 @@ void SolveState::begin_inner() {
   // b^_e = T_ee^-1 (r_e + kappa H_eo T_oo^-1 r_o)
   HopCall c;
   c.prec = P_;
+  c.fx_scratch = fx_scratch();
   c.nrhs = nrhs_;
   c.kcsw = kcsw_;
   c.clov = clov_.get();
@@ -337,6 +350,7 @@ void SolveState::enqueue_iteration() {
   const double S = P_ == P_F64 ? 192 : P_ == P_F32 ? 96 : 52, SX = PX_ == P_F64 ? 192 : PX_ == P_F32 ? 96 : 52;
   HopCall c;
   c.prec = P_;
+  c.fx_scratch = fx_scratch();
   c.nrhs = nrhs_;
   c.kcsw = kcsw_;
   c.clov = clov_.get();
@@ -419,6 +433,7 @@ RedArgs SolveState::cg_red(int fin, bool check_done) {
 void SolveState::cg_dhat_norm(const Field& in, const Field& out) {
   HopCall c;
   c.prec = P_;
+  c.fx_scratch = fx_scratch();
   c.nrhs = nrhs_;
   c.kcsw = kcsw_;
   c.clov = clov_.get();
@@ -471,6 +486,7 @@ void SolveState::cg_dhat_dag(const Field& in, const Field& out, bool check_done)
   BR_CUDA(cudaGetLastError());
   HopCall c;
   c.prec = P_;
+  c.fx_scratch = fx_scratch();
   c.nrhs = nrhs_;
   c.kcsw = kcsw_;
   c.clov = clov_.get();
@@ -739,6 +755,7 @@ void SolveState::finish_inner() {
   }
   HopCall c;
   c.prec = P_;
+  c.fx_scratch = fx_scratch();
   c.nrhs = nrhs_;
   c.kcsw = kcsw_;
   c.clov = clov_.get();

@@ -125,10 +125,10 @@ static std::vector<Candidate> candidates(long vh, int nrhs, const std::vector<in
 
 static std::vector<int> hop_variants(int prec, int flags, int red, int nrhs) {
   std::vector<int> v = {0};
-  if (!hop_has_variants(flags, red)) return v;
+  if (!hop_has_variants(flags, red) || prec == P_F64) return v;
   for (int k = 1; k < 6; ++k) v.push_back(k);
   const bool residual = (flags & F_SELF_CLOV) != 0;
-  if (prec != P_F64 && !residual) {
+  if (!residual) {
     for (int k = 6; k < 9; ++k)
       if (hop_variant_rpt(k) <= nrhs) v.push_back(k);
     if (nrhs >= 2)
@@ -209,6 +209,7 @@ void tune_solver_kernels(bridge_lattice_s* L, const bridge_op& op, int prec, int
     if (v.flags & F_E_CLOV) a.clovE = clover_ptr(L, *cs, prec, true);
     if (v.flags & F_SELF_CLOV) a.clovM = clover_ptr(L, *cs, prec, false);
     if (v.flags & F_SELF_CLOV) a.s1 = -1.0;
+    if (prec == P_F64) set_fx_args(L, a, v.flags, v.red, cs.get(), nullptr, st);
     a.red = red;
     a.red.fin = v.red == R_NONE ? FIN_NONE : FIN_STORE;
     const std::string key = "hop/" + std::to_string(prec) + "/" + std::to_string(v.flags) + "/" + std::to_string(v.red) +
