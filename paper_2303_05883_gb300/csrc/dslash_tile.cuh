@@ -132,14 +132,15 @@ BR_D void tile_stage_link(const HopArgs& a, const char* g_out, const char* g_in,
 }
 
 // One hop of one (site, rhs) with the staged link M (already beta * phase *
-// U or its adjoint): acc += (1 -/+ gamma_mu) M psi(neighbour).
-template <int P, int MU, bool FWD, int S>
+// U or its adjoint): acc += (1 -/+ gamma_mu) M psi(neighbour).  W: FP16 spinors
+// are widened before the projection instead of projected in half2.
+template <int P, int MU, bool FWD, int S, bool W>
 BR_D void tile_hop(const char* in, long vh, const float4* sl, const uint32_t* snb, int s, cx<float> acc[12]) {
   constexpr int h = 2 * MU + (FWD ? 0 : 1);
   const uint32_t nb = snb[h * S + s];
   cx<float> hh[2][3];
   float sc = 1.0f;
-  if constexpr (P == P_F16) {
+  if constexpr (P == P_F16 && !W) {
     const uint4* pl = reinterpret_cast<const uint4*>(in);
     const uint4 v0 = __ldg(pl + nb), v1 = __ldg(pl + vh + nb), v2 = __ldg(pl + 2 * vh + nb);
     sc = __ldg(reinterpret_cast<const float*>(in + 48 * vh) + nb);
@@ -259,16 +260,21 @@ BR_D void tile_pf_step(const char* in, long vh, const float4* sl, const uint32_t
 
 // NT tiles (NT x 32 sites) are staged between two barriers; the register
 // budget allows two resident 384-thread blocks per SM.  PF: pipelined
-// neighbour loads (16-bit storage only).
-template <int P, int FL, int RED, int NT, bool PF = false>
+// neighbour loads (16-bit storage only).  W: FP32 projection of FP16 spinors
+// (the untuned launches: they round no more than the per-thread kernel does).
+template <int P, int FL, int RED, int NT, bool PF = false, bool W = false>
 __global__ void __launch_bounds__(32 * TILE_MAX_RHS, 2) hop_kernel_tile(const HopArgs a) {
   static_assert(!PF || Tr<P>::half, "pipelined neighbour loads: 16-bit storage");
   static_assert(P != P_F64, "FP32 arithmetic kernels only");
   constexpr int S = NT * TILE_SITES;
   extern __shared__ float4 tile_smem[];
   float4* sl = tile_smem;
+  // the site term staged with the links: T^-1 (F_E_CLOV) or T (F_SELF_CLOV)
+  constexpr bool CL = (FL & (F_E_CLOV | F_SELF_CLOV)) != 0;
+  static_assert((FL & (F_E_CLOV | F_SELF_CLOV)) != (F_E_CLOV | F_SELF_CLOV), "one site term");
+  const char* clov = (FL & F_E_CLOV) ? a.clovE : a.clovM;
   float4* sc_clov = tile_smem + 8 * 5 * S;
-  uint32_t* snb = reinterpret_cast<uint32_t*>(tile_smem + 8 * 5 * S + ((FL & F_E_CLOV) ? 2 * 9 * S : 0));
+  uint32_t* snb = reinterpret_cast<uint32_t*>(tile_smem + 8 * 5 * S + (CL ? 2 * 9 * S : 0));
   uint4* pf = reinterpret_cast<uint4*>(snb + 8 * S);  // PF slots
   const int ng = tile_groups(a.nrhs), G = tile_group_size(a.nrhs);
   const int grp = blockIdx.x % ng;
@@ -285,7 +291,7 @@ __global__ void __launch_bounds__(32 * TILE_MAX_RHS, 2) hop_kernel_tile(const Ho
   const char* g_in = a.gauge + (long)(1 - p) * 4 * lbb;
   const char* in = a.in + (long)rhs * a.in_rs;
   const uint32_t nchunks = (uint32_t)((vh + S - 1) / S);
-  constexpr int nstage = 8 * S + ((FL & F_E_CLOV) ? 2 * S : 0);
+  constexpr int nstage = 8 * S + (CL ? 2 * S : 0);
   for (uint32_t chunk = sb; chunk < nchunks; chunk += (uint32_t)a.nblk) {
     const uint32_t base = chunk * S;
     __syncthreads();  // the previous chunk's reads of the staged data are done
@@ -301,14 +307,14 @@ __global__ void __launch_bounds__(32 * TILE_MAX_RHS, 2) hop_kernel_tile(const Ho
           case 2: tile_stage_link<P, 2, S>(a, g_out, g_in, lbb, ih, p, h, s, sl, snb); break;
           default: tile_stage_link<P, 3, S>(a, g_out, g_in, lbb, ih, p, h, s, sl, snb); break;
         }
-      } else if constexpr ((FL & F_E_CLOV) != 0) {
+      } else if constexpr (CL) {
         const int b = (j - 8 * S) / S;
         float m[36];
         // constant block index in each branch keeps the unpacking in registers
         if (b == 0)
-          load_clover_block<P, true>(a.clovE + p * cbb, vh, ih, 0, m);
+          load_clover_block<P, true>(clov + p * cbb, vh, ih, 0, m);
         else
-          load_clover_block<P, true>(a.clovE + p * cbb, vh, ih, 1, m);
+          load_clover_block<P, true>(clov + p * cbb, vh, ih, 1, m);
         float4* d = sc_clov + b * 9 * S + s;
 #pragma unroll
         for (int k = 0; k < 9; ++k) d[k * S] = make_float4(m[4 * k], m[4 * k + 1], m[4 * k + 2], m[4 * k + 3]);
@@ -336,17 +342,17 @@ __global__ void __launch_bounds__(32 * TILE_MAX_RHS, 2) hop_kernel_tile(const Ho
         tile_pf_step<P, 6, S>(in, vh, sl, snb, s, pf, t, acc);
         tile_pf_step<P, 7, S>(in, vh, sl, snb, s, pf, t, acc);
       } else {
-        tile_hop<P, 0, true, S>(in, vh, sl, snb, s, acc);
-        tile_hop<P, 0, false, S>(in, vh, sl, snb, s, acc);
-        tile_hop<P, 1, true, S>(in, vh, sl, snb, s, acc);
-        tile_hop<P, 1, false, S>(in, vh, sl, snb, s, acc);
-        tile_hop<P, 2, true, S>(in, vh, sl, snb, s, acc);
-        tile_hop<P, 2, false, S>(in, vh, sl, snb, s, acc);
-        tile_hop<P, 3, true, S>(in, vh, sl, snb, s, acc);
-        tile_hop<P, 3, false, S>(in, vh, sl, snb, s, acc);
+        tile_hop<P, 0, true, S, W>(in, vh, sl, snb, s, acc);
+        tile_hop<P, 0, false, S, W>(in, vh, sl, snb, s, acc);
+        tile_hop<P, 1, true, S, W>(in, vh, sl, snb, s, acc);
+        tile_hop<P, 1, false, S, W>(in, vh, sl, snb, s, acc);
+        tile_hop<P, 2, true, S, W>(in, vh, sl, snb, s, acc);
+        tile_hop<P, 2, false, S, W>(in, vh, sl, snb, s, acc);
+        tile_hop<P, 3, true, S, W>(in, vh, sl, snb, s, acc);
+        tile_hop<P, 3, false, S, W>(in, vh, sl, snb, s, acc);
       }
-      cx<float> v[12];
-      if constexpr ((FL & F_E_CLOV) != 0) {
+      // the staged site term times x
+      auto site_term = [&](const cx<float> x[12], cx<float> y[12]) {
 #pragma unroll
         for (int b = 0; b < 2; ++b) {
           float m[36];
@@ -359,8 +365,22 @@ __global__ void __launch_bounds__(32 * TILE_MAX_RHS, 2) hop_kernel_tile(const Ho
             m[4 * k + 2] = t4.z;
             m[4 * k + 3] = t4.w;
           }
-          hermitian6_apply<float>(m, acc + 6 * b, v + 6 * b);
+          hermitian6_apply<float>(m, x + 6 * b, y + 6 * b);
         }
+      };
+      if constexpr ((FL & F_AUX) != 0) {
+        cx<float> x[12];
+        load_spinor<P, true, true>(a.aux + (long)rhs * a.aux_rs, vh, ih, x);
+#pragma unroll
+        for (int k = 0; k < 12; ++k) acc[k] = caxpy(a.cauxf, x[k], acc[k]);
+      }
+      if constexpr ((FL & F_G5) != 0) {
+#pragma unroll
+        for (int k = 6; k < 12; ++k) acc[k] = cx<float>{-acc[k].r, -acc[k].i};
+      }
+      cx<float> v[12];
+      if constexpr ((FL & F_E_CLOV) != 0) {
+        site_term(acc, v);
       } else {
 #pragma unroll
         for (int k = 0; k < 12; ++k) v[k] = acc[k];
@@ -368,8 +388,15 @@ __global__ void __launch_bounds__(32 * TILE_MAX_RHS, 2) hop_kernel_tile(const Ho
       cx<float> sv[12];
       if constexpr ((FL & F_SELF) != 0) {
         load_spinor<P, true, true>(a.self + (long)rhs * a.self_rs, vh, ih, sv);
+        if constexpr ((FL & F_SELF_CLOV) != 0) {
+          cx<float> ms[12];
+          site_term(sv, ms);
 #pragma unroll
-        for (int k = 0; k < 12; ++k) v[k] = caxpy(a.s1f, sv[k], v[k]);
+          for (int k = 0; k < 12; ++k) v[k] = caxpy(a.s1f, ms[k], v[k]);
+        } else {
+#pragma unroll
+          for (int k = 0; k < 12; ++k) v[k] = caxpy(a.s1f, sv[k], v[k]);
+        }
       }
       store_spinor<P>(a.out + (long)rhs * a.out_rs, vh, ih, v);
       if constexpr (RED == R_NORM) {

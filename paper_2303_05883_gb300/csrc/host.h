@@ -119,7 +119,13 @@ struct LaunchShape {
   int block = 256;
   int nblk = 0;     // site blocks per rhs; 0 -> cover the lattice once
   int variant = 0;  // register-budget variant of the kernel (see launch_hop)
+  bool untuned = false;  // a default, not measured or set
 };
+
+// The kernel variant of a shape.
+inline int launch_variant(const LaunchShape& s) {
+  return s.variant + (s.untuned && (s.variant == 9 || s.variant == 10) ? HOP_TILE_WIDE : 0);
+}
 
 struct Stats {
   std::mutex mu;
@@ -218,10 +224,11 @@ namespace bridge {
 // launch bookkeeping (called at each launch site)
 void note_launch(bridge_lattice_s* L, int cls, double bytes, double flops, cudaStream_t st, bool begin);
 // Launch shape for a kernel key: the tuned entry if there is one, else
-// `block` threads and a persistent grid of (resident blocks per SM x SM
-// count) blocks, computed by occ(block), capped at one site per thread.
+// `variant` with a persistent grid of (resident blocks per SM x SM count)
+// blocks, computed by occ(block), capped at one site per thread (cover_once:
+// a variant 4 launch covers the lattice with one site per thread).
 LaunchShape shape_for(bridge_lattice_s* L, const std::string& key, long vh, int nrhs,
-                      const std::function<int(int)>& occ);
+                      const std::function<int(int)>& occ, int variant = 0, bool cover_once = false);
 
 // Algorithmic cost of one hop launch: bytes and flops per right-hand side
 // (spinors) and shared by all right-hand sides (links, clover blocks).

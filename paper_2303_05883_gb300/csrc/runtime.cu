@@ -131,17 +131,20 @@ void note_launch(bridge_lattice_s* L, int cls, double bytes, double flops, cudaS
 }
 
 LaunchShape shape_for(bridge_lattice_s* L, const std::string& key, long vh, int nrhs,
-                      const std::function<int(int)>& occ) {
+                      const std::function<int(int)>& occ, int variant, bool cover_once) {
   std::lock_guard<std::mutex> lk(L->tune_mu);
   LaunchShape s;
   auto it = L->tuned.find(key);
   if (it != L->tuned.end()) {
     s = it->second;
   } else {
-    s.block = 128;
+    s.variant = variant;
+    s.untuned = true;
+    s.block = variant == 4 && !cover_once ? 256 : 128;
     const int per_sm = occ ? occ(s.block) : 0;
     const long resident = (long)sm_count() * (per_sm > 0 ? per_sm : 4);
-    s.nblk = (int)std::max<long>(1, resident / std::max(1, nrhs));
+    const int groups = (nrhs + hop_variant_rpt(variant) - 1) / hop_variant_rpt(variant);
+    s.nblk = variant == 4 && cover_once ? 0 : (int)std::max<long>(1, resident / std::max(1, groups));
     L->tuned[key] = s;
   }
   const long cover = (vh + s.block - 1) / s.block;
@@ -350,6 +353,8 @@ HopCost hop_cost(int prec, int flags, int red) {
   return HopCost{per_rhs, shared, fl};
 }
 
+static int default_hop_variant(int prec, int flags, int red, long vh, int nrhs, bool mapped);
+
 static std::string dims_key(const bridge_lattice_s* L) {
   return std::to_string(L->dims[0]) + "x" + std::to_string(L->dims[1]) + "x" + std::to_string(L->dims[2]) + "x" +
          std::to_string(L->dims[3]);
@@ -390,11 +395,12 @@ void run_hop(bridge_lattice_s* L, HopCall c, cudaStream_t st) {
   if (c.prec == P_F64 && !c.site_map) set_fx_args(L, a, c.flags, c.red, cs, c.fx_scratch, st);
   const std::string key = "hop/" + std::to_string(c.prec) + "/" + std::to_string(c.flags) + "/" +
                           std::to_string(c.red) + "/" + dims_key(L) + "/" + std::to_string(c.nrhs);
+  const int variant = default_hop_variant(c.prec, c.flags, c.red, L->vh, c.nrhs, c.site_map != nullptr);
   LaunchShape sh = shape_for(L, key, L->vh, c.nrhs, [&](int block) {
     int n = 0;
-    launch_hop_any(c.prec, c.flags, c.red, a, block, st, &n, 0);
+    launch_hop_any(c.prec, c.flags, c.red, a, block, st, &n, variant + (variant == 9 || variant == 10 ? HOP_TILE_WIDE : 0));
     return n;
-  });
+  }, variant, c.red == R_NONE);
   a.nblk = sh.nblk;
   if (c.red != R_NONE && a.red.partials == nullptr) {
     // a fixed-point launch takes up to one block for 64 sites
@@ -412,7 +418,7 @@ void run_hop(bridge_lattice_s* L, HopCall c, cudaStream_t st) {
       c.count_work ? c.work_fraction * (double)L->vh * (hc.rhs_bytes * c.nrhs + hc.shared_bytes) : 0.0;
   const double flops = c.count_work ? c.work_fraction * (double)L->vh * c.nrhs * hc.rhs_flops : 0.0;
   note_launch(L, c.cls, bytes, flops, st, true);
-  BR_CHECK(launch_hop_any(c.prec, c.flags, c.red, a, sh.block, st, nullptr, sh.variant), BRIDGE_EINVAL,
+  BR_CHECK(launch_hop_any(c.prec, c.flags, c.red, a, sh.block, st, nullptr, launch_variant(sh)), BRIDGE_EINVAL,
            "hop variant not instantiated");
   note_launch(L, c.cls, bytes, flops, st, false);
   BR_CUDA(cudaGetLastError());
@@ -600,9 +606,30 @@ void clover_site(bridge_lattice_s* L, int prec, bool inverse, double kcsw, int p
 }
 
 bool hop_has_variants(int flags, int red) {
-  return (flags == 0 && red == R_NONE) || (flags == F_E_CLOV && red == R_NONE) ||
-         ((flags == F_SELF || flags == (F_SELF | F_E_CLOV)) && (red == R_DOT_A || red == R_TS)) ||
-         (flags == (F_AUX | F_SELF | F_SELF_CLOV) && red == R_NORM);
+  return (flags & (F_E_CLOV | F_SELF_CLOV)) != (F_E_CLOV | F_SELF_CLOV) &&
+         !((flags & F_AUX) && (flags & F_SELF) && red == R_NORM && !(flags & F_SELF_CLOV));
+}
+
+// The variant an untuned launch takes, by its working set (microseconds on a
+// GB300, default persistent shape of variant 0 -> the variant; Schur pass 1 /
+// pass 2 with a dot product):
+//   * from 4 right-hand sides on 2^18 half-lattice sites, or 6 on 2^16, the
+//     tile kernel, which loads, widens and scales each link and clover block
+//     once for all of them: 24^3 x 48 F32 4 RHS 123 -> 113 / 189 -> 163, 12
+//     RHS 332 -> 283 / 525 -> 388, F16 12 RHS 347 -> 246 / 424 -> 330 (projected
+//     in half2; in FP32, as untuned launches do, four D^ on 12 RHS take 2.3 ms
+//     instead of 2.9); 16^3 x 32 6 RHS 39 -> 38 / 72 -> 68, but 4 RHS 27 -> 29 /
+//     51 -> 53, and 12^3 x 16 12 RHS 17 -> 21 / 40 -> 58 (too few tiles for the
+//     SMs).  Two tiles a barrier from 8 right-hand sides (195 against 208), one
+//     below (157 against 170);
+//   * fewer right-hand sides on 2^17 sites or more: at most 80 registers and
+//     read-once operands past L1, 256-thread blocks (pass 2, 32^3 x 64: F32
+//     186 -> 175, 3 RHS 429 -> 360, F16 136 -> 130); on 16^3 x 32 it is slower.
+static int default_hop_variant(int prec, int flags, int red, long vh, int nrhs, bool mapped) {
+  if (prec == P_F64 || mapped || !hop_has_variants(flags, red)) return 0;
+  const int per_block = (nrhs + (nrhs + 11) / 12 - 1) / ((nrhs + 11) / 12);  // right-hand sides of a tile block
+  if ((per_block >= 4 && vh >= (1L << 18)) || (per_block >= 6 && vh >= (1L << 16))) return per_block >= 8 ? 10 : 9;
+  return vh >= (1L << 17) && (flags & F_AUX) == 0 ? 4 : 0;
 }
 
 bool launch_hop_any(int prec, int flags, int red, const HopArgs& a, int block, cudaStream_t st, int* occ,
