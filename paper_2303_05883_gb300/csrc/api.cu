@@ -142,27 +142,20 @@ static void mult_dev(bridge_lattice_s* L, const bridge_op& op, int prec, int whi
     return;
   }
   BR_CHECK(which != APPLY_DHAT_DAG, BRIDGE_EINVAL, "bridge_mult_Dhat_dag is provided for MOBIUS operators only");
+  const int subset = which == BRIDGE_APPLY_D ? BRIDGE_FULL : which == BRIDGE_APPLY_DEO ? 1 - out_parity : BRIDGE_EVEN;
+  Field fi = workspace(L, "mult_in", prec, subset, nrhs);
+  // FP64: the input's fixed-point form is written with its layout conversion
+  if (prec == BRIDGE_F64) fi.fx = fx_input(L, op, which, nrhs * (subset == BRIDGE_FULL ? 2 : 1));
+  canon_to_field(L, in, fi, st);
+  Field& fo = workspace(L, "mult_out", prec, which == BRIDGE_APPLY_DEO ? out_parity : subset, nrhs);
   if (which == BRIDGE_APPLY_D) {
-    Field& fi = workspace(L, "mult_in", prec, BRIDGE_FULL, nrhs);
-    Field& fo = workspace(L, "mult_out", prec, BRIDGE_FULL, nrhs);
-    canon_to_field(L, in, fi, st);
     apply_d(L, op, fo, fi, st);
-    field_to_canon(L, fo, out, st);
   } else if (which == BRIDGE_APPLY_DEO) {
-    const int q = out_parity;
-    Field& fi = workspace(L, "mult_in", prec, 1 - q, nrhs);
-    Field& fo = workspace(L, "mult_out", prec, q, nrhs);
-    canon_to_field(L, in, fi, st);
-    apply_deo(L, op, q, fo, fi, st);
-    field_to_canon(L, fo, out, st);
+    apply_deo(L, op, out_parity, fo, fi, st);
   } else {
-    Field& fi = workspace(L, "mult_in", prec, BRIDGE_EVEN, nrhs);
-    Field& fo = workspace(L, "mult_out", prec, BRIDGE_EVEN, nrhs);
-    Field& ft = workspace(L, "mult_tmp", prec, BRIDGE_ODD, nrhs);
-    canon_to_field(L, in, fi, st);
-    apply_dhat(L, op, fo, fi, ft, st);
-    field_to_canon(L, fo, out, st);
+    apply_dhat(L, op, fo, fi, workspace(L, "mult_tmp", prec, BRIDGE_ODD, nrhs), st);
   }
+  field_to_canon(L, fo, out, st);
 }
 
 static int mult_common(bridge_lattice L, const bridge_op* op, int prec, int which, int out_parity, const double* in,

@@ -153,6 +153,11 @@ BR_HD long clover_block_bytes(int prec, long vh) {  // one parity
   return pad256(b);
 }
 
+// A half-lattice field in fixed point: the 12 complex planes of the FP64
+// field as 64-bit integers in units of 2^(E - 1081), then one int a site: the
+// exponent E, 0 where the spinor is zero, -1 where it has no such form.
+BR_HD long fx_block_bytes(long vh) { return pad256(196 * vh); }
+
 // ------------------------------------------------------- 16-bit helpers
 template <int P>
 struct H16;

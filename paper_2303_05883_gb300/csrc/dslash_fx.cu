@@ -46,23 +46,11 @@ bool launch_hop_fx(int flags, int red, const HopArgs& args, int block, cudaStrea
 __global__ void __launch_bounds__(256) k_field_to_fx(const CopyArgs a) {
   const int rhs = blockIdx.x % a.nrhs;
   if (rhs_finished(a.red, rhs)) return;
-  const long vh = a.vh;
-  const uint4* src = reinterpret_cast<const uint4*>(a.src + rhs * a.src_rs);
-  uint4* dst = reinterpret_cast<uint4*>(a.dst + rhs * a.dst_rs);
-  int* ex = reinterpret_cast<int*>(a.dst + rhs * a.dst_rs + 192 * vh);
   for (uint32_t ih = (uint32_t)(blockIdx.x / a.nrhs) * blockDim.x + threadIdx.x; ih < a.vh;
        ih += (uint32_t)a.nblk * blockDim.x) {
-    uint4 w[12];
-#pragma unroll
-    for (int k = 0; k < 12; ++k) w[k] = __ldg(src + k * vh + ih);
-    const uint32_t m = fx_max_word<12>(w);
-    const int E = (int)(m >> 20);
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      const long long r = fx_from_bits<6>(w[k].x, w[k].y, E, 0), i = fx_from_bits<6>(w[k].z, w[k].w, E, 0);
-      dst[k * vh + ih] = make_uint4((uint32_t)r, (uint32_t)(r >> 32), (uint32_t)i, (uint32_t)(i >> 32));
-    }
-    ex[ih] = m == 0 ? 0 : (E < FX_EMIN || E > FX_EMAX) ? -1 : E;
+    cx<double> s[12];
+    load_spinor<P_F64>(a.src + rhs * a.src_rs, a.vh, ih, s);
+    fx_store(a.dst + rhs * a.dst_rs, a.vh, ih, s);
   }
 }
 

@@ -45,10 +45,6 @@ namespace bridge {
 constexpr int FX_EMIN = 128, FX_EMAX = 1900;  // biased exponents a spinor may have
 constexpr int FX_THREADS = 128;               // block of the stencil: two lanes a site
 constexpr int FX_SITES = FX_THREADS / 2;
-// A half-lattice field in fixed point: the 12 complex planes of the FP64
-// field as 64-bit integers in units of 2^(E - 1081), then one int a site: the
-// exponent E, 0 where the spinor is zero, -1 where it has no such form.
-BR_HD long fx_block_bytes(long vh) { return pad256(196 * vh); }
 constexpr uint32_t FX_LINK_TOP = 0x3ff00001u;  // links: at most 1 (+ rounding), unit 2^-60
 constexpr int FX_CLOV_EMAX = 2;                // clover entries: below 2^e, unit 2^(e - 60), e = 1 or 2
 BR_HD uint32_t fx_clov_top(int e) { return (uint32_t)(1023 + e) << 20; }  // high word of 2^e
@@ -87,6 +83,25 @@ BR_D uint32_t fx_max_word(const uint4 w[N]) {
 #pragma unroll
   for (int k = 0; k < N; ++k) m = max(m, max(w[k].y & 0x7fffffffu, w[k].w & 0x7fffffffu));
   return m;
+}
+
+// The fixed-point form of one FP64 spinor, stored at site ih of a block
+// (layout: fx_block_bytes).
+BR_D void fx_store(char* block, long vh, uint32_t ih, const cx<double> s[12]) {
+  uint4 w[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k)
+    w[k] = make_uint4((uint32_t)__double2loint(s[k].r), (uint32_t)__double2hiint(s[k].r), (uint32_t)__double2loint(s[k].i),
+                      (uint32_t)__double2hiint(s[k].i));
+  const uint32_t m = fx_max_word<12>(w);
+  const int E = (int)(m >> 20);
+  uint4* dst = reinterpret_cast<uint4*>(block) + ih;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    const long long r = fx_from_bits<6>(w[k].x, w[k].y, E, 0), i = fx_from_bits<6>(w[k].z, w[k].w, E, 0);
+    dst[k * vh] = make_uint4((uint32_t)r, (uint32_t)(r >> 32), (uint32_t)i, (uint32_t)(i >> 32));
+  }
+  reinterpret_cast<int*>(block + 192 * vh)[ih] = m == 0 ? 0 : (E < FX_EMIN || E > FX_EMAX) ? -1 : E;
 }
 
 BR_D long long fx_shift_round(long long x, int d) {  // x / 2^d to nearest, d in 0 .. 62

@@ -108,6 +108,14 @@ struct Field {
   char* ptr(int parity) const {  // block of this parity for rhs 0
     return buf->ptr + ((subset == BRIDGE_FULL && parity == 1) ? block : 0);
   }
+  // FP64: where the field's fixed-point form stands or goes (not owned, one
+  // block for each block of buf; null: nowhere).  Set on a copy of the Field
+  // for the calls between which it is valid.
+  char* fx = nullptr;
+  char* fx_ptr(int parity) const {
+    return fx ? fx + ((subset == BRIDGE_FULL && parity == 1) ? fx_block_bytes(vh) : 0) : nullptr;
+  }
+  long fx_rs() const { return (subset == BRIDGE_FULL ? 2 : 1) * fx_block_bytes(vh); }
 };
 // at_least: bytes the buffer holds at the least.
 Field make_field(int prec, int subset, int nrhs, long vh, cudaStream_t st = nullptr, bool stream_ordered = false,
@@ -255,6 +263,9 @@ const char* clover_fx_ptr(bridge_lattice_s* L, CloverSet& set, bool inverse, cud
 // clover set of the flags that need one; scratch as HopCall::fx_scratch) and
 // queue the conversion of its input; or leave them null.
 void set_fx_args(bridge_lattice_s* L, HopArgs& a, int flags, int red, CloverSet* set, char* scratch, cudaStream_t st);
+// Where the FP64 application `which` (bridge_apply_op) of op on the lattice
+// stream runs in fixed point, room for nblocks half-lattice inputs; else null.
+char* fx_input(bridge_lattice_s* L, const bridge_op& op, int which, int nblocks);
 
 // ------------------------------------------------------- operators
 // Apply one hop-kernel variant (see dslash.cuh).  Field pointers are the
@@ -273,6 +284,8 @@ struct HopCall {
   RedArgs redargs{};
   const uint32_t* site_map = nullptr;  // HopArgs::site_map / n_map: a subset of the output sites
   uint32_t n_map = 0;
+  const char* in_fx = nullptr;  // FP64: `in` in fixed point, where the caller has it already
+  long in_fx_rs = 0;
   char* fx_scratch = nullptr;  // FP64: room for nrhs blocks of fx_block_bytes (default: the lattice's, for
                                // work on the lattice stream; elsewhere the launch stays on the FP64 kernel)
   double work_fraction = 1.0;  // share of the sites the launch computes (for the byte and flop counts)

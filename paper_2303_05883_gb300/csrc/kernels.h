@@ -51,7 +51,6 @@ bool launch_blas(int op, int prec, int px, const BlasArgs& a, int block, cudaStr
 struct CopyArgs {
   uint32_t vh;
   int nrhs, nblk;
-  int parity;   // parity of the half-lattice block (full-canonical conversions)
   Geom g;
   long V;       // full volume (canonical full-lattice strides)
   const double* canon;  // canonical FP64 (re, im) pairs
@@ -62,11 +61,15 @@ struct CopyArgs {
   long src_rs;
   char* dst;
   long dst_rs;
+  const char* src2;     // whole canonical lattices: the odd parity's block (src / dst the even one's)
+  char* dst2;
+  char *fx, *fx2;       // canonical -> FP64: the fixed-point form too (null: none), even and odd block
+  long fx_rs;
   const int* mask;      // per rhs; 0 -> write zeros (may be null)
   RedArgs red;          // norm of the source (FIN_STORE) when red.partials != null
 };
-bool launch_canon_to_field(int prec, const CopyArgs& a, int block, cudaStream_t st);
-bool launch_field_to_canon(int prec, const CopyArgs& a, int block, cudaStream_t st);
+bool launch_canon_to_field(int prec, const CopyArgs& a, cudaStream_t st);
+bool launch_field_to_canon(int prec, const CopyArgs& a, cudaStream_t st);
 bool launch_convert(int ps, int pd, const CopyArgs& a, int block, cudaStream_t st);   // dst = mask ? src : 0
 bool launch_accumulate64(int ps, const CopyArgs& a, int block, cudaStream_t st);      // dst(F64) += src
 bool launch_norm2(int prec, const CopyArgs& a, int block, cudaStream_t st);           // |src|^2 -> FIN_STORE

@@ -133,7 +133,7 @@ extern "C" int bridge_mult_Dhat_noalloc(bridge_lattice L, const bridge_op* op, i
     ca.canon_full = 0;
     ca.dst = f_in;
     ca.dst_rs = block;
-    BR_CHECK(launch_canon_to_field(prec, ca, 256, st), BRIDGE_EINVAL, "precision");
+    BR_CHECK(launch_canon_to_field(prec, ca, st), BRIDGE_EINVAL, "precision");
 
     HopArgs a;
     std::memset(&a, 0, sizeof(a));
@@ -183,7 +183,7 @@ extern "C" int bridge_mult_Dhat_noalloc(bridge_lattice L, const bridge_op* op, i
     ca.canon_out = out_dev;
     ca.src = f_out;
     ca.src_rs = block;
-    BR_CHECK(launch_field_to_canon(prec, ca, 256, st), BRIDGE_EINVAL, "precision");
+    BR_CHECK(launch_field_to_canon(prec, ca, st), BRIDGE_EINVAL, "precision");
     BR_CUDA(cudaGetLastError());
     g_launches.fetch_add(4);
   } catch (const Error& e) {

@@ -287,44 +287,49 @@ const char* clover_fx_ptr(bridge_lattice_s* L, CloverSet& set, bool inverse, cud
   return p;
 }
 
+char* fx_scratch(bridge_lattice_s* L, int nblocks) {
+  const size_t need = (size_t)nblocks * fx_block_bytes(L->vh);
+  if (!L->fx_scratch || L->fx_scratch->bytes < need) {
+    if (capturing(L->stream)) return nullptr;
+    L->fx_scratch.reset();
+    try {
+      L->fx_scratch.reset(new DevBuf(need));
+    } catch (const Error&) {
+      return nullptr;  // no room: the FP64 kernel needs none
+    }
+  }
+  return L->fx_scratch->ptr;
+}
+
 void set_fx_args(bridge_lattice_s* L, HopArgs& a, int flags, int red, CloverSet* set, char* scratch, cudaStream_t st) {
   a.gauge_fx = a.clovE_fx = a.clovM_fx = nullptr;
   if (!fx_has(flags, red)) return;
-  const size_t need = (size_t)a.nrhs * fx_block_bytes(L->vh);
-  if (!scratch && st != L->stream) return;
+  if (!a.in_fx && !scratch && st != L->stream) return;
   const char* E = (flags & F_E_CLOV) ? clover_fx_ptr(L, *set, true, st, &a.eE_fx) : nullptr;
   const char* M = (flags & F_SELF_CLOV) ? clover_fx_ptr(L, *set, false, st, &a.eM_fx) : nullptr;
   if (((flags & F_E_CLOV) && !E) || ((flags & F_SELF_CLOV) && !M)) return;
   const char* U = gauge_fx_ptr(L, st);
   if (!U) return;
-  if (!scratch) {
-    if (!L->fx_scratch || L->fx_scratch->bytes < need) {
-      if (capturing(st)) return;
-      L->fx_scratch.reset();
-      try {
-        L->fx_scratch.reset(new DevBuf(need));
-      } catch (const Error&) {
-        return;  // no room: the FP64 kernel needs none
-      }
-    }
-    scratch = L->fx_scratch->ptr;
+  if (!a.in_fx) {
+    if (!scratch) scratch = fx_scratch(L, a.nrhs);
+    if (!scratch) return;
+    CopyArgs c;
+    std::memset(&c, 0, sizeof(c));
+    c.vh = (uint32_t)L->vh;
+    c.nrhs = a.nrhs;
+    c.nblk = (int)((L->vh + 255) / 256);
+    c.src = a.in;
+    c.src_rs = a.in_rs;
+    c.dst = scratch;
+    c.dst_rs = fx_block_bytes(L->vh);
+    c.red = a.red;  // right-hand sides whose solve has ended are skipped
+    const double bytes = (double)L->vh * a.nrhs * (192 + 196);
+    note_launch(L, K_CONVERT, bytes, 0, st, true);
+    launch_field_to_fx(c, 256, st);
+    note_launch(L, K_CONVERT, bytes, 0, st, false);
+    a.in_fx = scratch;
+    a.in_fx_rs = c.dst_rs;
   }
-  CopyArgs c;
-  std::memset(&c, 0, sizeof(c));
-  c.vh = (uint32_t)L->vh;
-  c.nrhs = a.nrhs;
-  c.nblk = (int)((L->vh + 255) / 256);
-  c.src = a.in;
-  c.src_rs = a.in_rs;
-  c.dst = scratch;
-  c.dst_rs = fx_block_bytes(L->vh);
-  c.red = a.red;  // right-hand sides whose solve has ended are skipped
-  const double bytes = (double)L->vh * a.nrhs * (192 + 196);
-  note_launch(L, K_CONVERT, bytes, 0, st, true);
-  launch_field_to_fx(c, 256, st);
-  note_launch(L, K_CONVERT, bytes, 0, st, false);
-  a.in_fx = scratch;
-  a.in_fx_rs = c.dst_rs;
   a.gauge_fx = U;
   a.clovE_fx = E;
   a.clovM_fx = M;
@@ -392,6 +397,8 @@ void run_hop(bridge_lattice_s* L, HopCall c, cudaStream_t st) {
     a.clovM = (c.flags & F_SELF_CLOV) ? clover_ptr(L, *cs, c.prec, false) : nullptr;
   }
   a.red = c.redargs;
+  a.in_fx = c.in_fx;
+  a.in_fx_rs = c.in_fx_rs;
   if (c.prec == P_F64 && !c.site_map) set_fx_args(L, a, c.flags, c.red, cs, c.fx_scratch, st);
   const std::string key = "hop/" + std::to_string(c.prec) + "/" + std::to_string(c.flags) + "/" +
                           std::to_string(c.red) + "/" + dims_key(L) + "/" + std::to_string(c.nrhs);
@@ -424,6 +431,17 @@ void run_hop(bridge_lattice_s* L, HopCall c, cudaStream_t st) {
   BR_CUDA(cudaGetLastError());
 }
 
+// Whether the FP64 hops of op run in fixed point, and the scratch for the
+// fixed-point form of nblocks half-lattice inputs (null: they do not).
+char* fx_input(bridge_lattice_s* L, const bridge_op& op, int which, int nblocks) {
+  if (!gauge_fx_ptr(L, L->stream)) return nullptr;
+  if (op_is_clover(op) && which != BRIDGE_APPLY_DEO) {
+    auto set = clover_set(L, op_kcsw(op));
+    if (!clover_fx_ptr(L, *set, which == BRIDGE_APPLY_DHAT, L->stream)) return nullptr;
+  }
+  return fx_scratch(L, nblocks);
+}
+
 void apply_deo(bridge_lattice_s* L, const bridge_op& op, int q, const Field& out, const Field& in, cudaStream_t st) {
   HopCall c;
   c.prec = in.prec;
@@ -437,6 +455,8 @@ void apply_deo(bridge_lattice_s* L, const bridge_op& op, int q, const Field& out
   c.out_rs = out.rs;
   c.in = in.ptr(1 - q);
   c.in_rs = in.rs;
+  c.in_fx = in.fx_ptr(1 - q);
+  c.in_fx_rs = in.fx_rs();
   run_hop(L, c, st);
 }
 
@@ -457,6 +477,8 @@ void apply_d(bridge_lattice_s* L, const bridge_op& op, const Field& out, const F
     c.out_rs = out.rs;
     c.in = in.ptr(1 - q);
     c.in_rs = in.rs;
+    c.in_fx = in.fx_ptr(1 - q);
+    c.in_fx_rs = in.fx_rs();
     c.self = in.ptr(q);
     c.self_rs = in.rs;
     run_hop(L, c, st);
@@ -480,7 +502,10 @@ void apply_dhat(bridge_lattice_s* L, const bridge_op& op, const Field& out, cons
   c.out_rs = tmp.rs;
   c.in = in.ptr(0);
   c.in_rs = in.rs;
+  c.in_fx = in.fx_ptr(0);
+  c.in_fx_rs = in.fx_rs();
   run_hop(L, c, st);
+  c.in_fx = nullptr;
   // pass 2: out_e = in_e - T_ee^-1 (-kappa H_eo tmp_o)
   c.flags = F_SELF | (clov ? F_E_CLOV : 0);
   c.cls = K_DHAT2;
@@ -497,12 +522,11 @@ void apply_dhat(bridge_lattice_s* L, const bridge_op& op, const Field& out, cons
 }
 
 // ------------------------------------------------------------ layouts
-static CopyArgs copy_args(bridge_lattice_s* L, const Field& f, int parity) {
+static CopyArgs copy_args(bridge_lattice_s* L, const Field& f) {
   CopyArgs a;
   std::memset(&a, 0, sizeof(a));
   a.vh = (uint32_t)L->vh;
   a.nrhs = f.nrhs;
-  a.parity = parity;
   a.g = L->g;
   a.V = L->V;
   const int block = 256;
@@ -512,42 +536,42 @@ static CopyArgs copy_args(bridge_lattice_s* L, const Field& f, int parity) {
 
 void canon_to_field(bridge_lattice_s* L, const double* canon, const Field& f, cudaStream_t st, const int* mask,
                     long canon_rs) {
-  const int lo = f.subset == BRIDGE_FULL ? 0 : f.subset, hi = f.subset == BRIDGE_FULL ? 1 : f.subset;
-  for (int p = lo; p <= hi; ++p) {
-    CopyArgs a = copy_args(L, f, p);
-    a.canon = canon;
-    a.canon_rs = canon_rs / 2;
-    a.canon_full = f.subset == BRIDGE_FULL;
-    a.dst = f.ptr(p);
-    a.dst_rs = f.rs;
-    a.mask = mask;
-    const double bytes = (double)L->vh * f.nrhs * (192 + spinor_site_bytes(f.prec));
-    note_launch(L, K_CONVERT, bytes, 0, st, true);
-    launch_canon_to_field(f.prec, a, 256, st);
-    note_launch(L, K_CONVERT, bytes, 0, st, false);
-  }
+  CopyArgs a = copy_args(L, f);
+  a.canon = canon;
+  a.canon_rs = canon_rs / 2;
+  a.canon_full = f.subset == BRIDGE_FULL;
+  a.dst = f.ptr(a.canon_full ? 0 : f.subset);
+  if (a.canon_full) a.dst2 = f.ptr(1);
+  a.dst_rs = f.rs;
+  a.fx = f.fx;
+  a.fx2 = f.fx ? f.fx_ptr(1) : nullptr;
+  a.fx_rs = f.fx_rs();
+  a.mask = mask;
+  const double sites = (double)(a.canon_full ? L->V : L->vh) * f.nrhs;
+  const double bytes = sites * (192 + spinor_site_bytes(f.prec) + (f.fx ? 196 : 0));
+  note_launch(L, K_CONVERT, bytes, 0, st, true);
+  launch_canon_to_field(f.prec, a, st);
+  note_launch(L, K_CONVERT, bytes, 0, st, false);
   BR_CUDA(cudaGetLastError());
 }
 
 void field_to_canon(bridge_lattice_s* L, const Field& f, double* canon, cudaStream_t st, long canon_rs) {
-  const int lo = f.subset == BRIDGE_FULL ? 0 : f.subset, hi = f.subset == BRIDGE_FULL ? 1 : f.subset;
-  for (int p = lo; p <= hi; ++p) {
-    CopyArgs a = copy_args(L, f, p);
-    a.canon_out = canon;
-    a.canon_rs = canon_rs / 2;
-    a.canon_full = f.subset == BRIDGE_FULL;
-    a.src = f.ptr(p);
-    a.src_rs = f.rs;
-    const double bytes = (double)L->vh * f.nrhs * (192 + spinor_site_bytes(f.prec));
-    note_launch(L, K_CONVERT, bytes, 0, st, true);
-    launch_field_to_canon(f.prec, a, 256, st);
-    note_launch(L, K_CONVERT, bytes, 0, st, false);
-  }
+  CopyArgs a = copy_args(L, f);
+  a.canon_out = canon;
+  a.canon_rs = canon_rs / 2;
+  a.canon_full = f.subset == BRIDGE_FULL;
+  a.src = f.ptr(a.canon_full ? 0 : f.subset);
+  if (a.canon_full) a.src2 = f.ptr(1);
+  a.src_rs = f.rs;
+  const double bytes = (double)(a.canon_full ? L->V : L->vh) * f.nrhs * (192 + spinor_site_bytes(f.prec));
+  note_launch(L, K_CONVERT, bytes, 0, st, true);
+  launch_field_to_canon(f.prec, a, st);
+  note_launch(L, K_CONVERT, bytes, 0, st, false);
   BR_CUDA(cudaGetLastError());
 }
 
 void convert_field(bridge_lattice_s* L, const Field& src, const Field& dst, int parity, cudaStream_t st, const int* mask) {
-  CopyArgs a = copy_args(L, src, parity);
+  CopyArgs a = copy_args(L, src);
   a.src = src.ptr(parity);
   a.src_rs = src.rs;
   a.dst = dst.ptr(parity);
@@ -562,7 +586,7 @@ void convert_field(bridge_lattice_s* L, const Field& src, const Field& dst, int 
 
 void accumulate64(bridge_lattice_s* L, const Field& src, int sp, const Field& dst, int dp, cudaStream_t st,
                   const int* mask) {
-  CopyArgs a = copy_args(L, src, sp);
+  CopyArgs a = copy_args(L, src);
   a.src = src.ptr(sp);
   a.src_rs = src.rs;
   a.dst = dst.ptr(dp);
@@ -576,7 +600,7 @@ void accumulate64(bridge_lattice_s* L, const Field& src, int sp, const Field& ds
 }
 
 void norm2_field(bridge_lattice_s* L, const Field& f, int parity, RedArgs red, cudaStream_t st) {
-  CopyArgs a = copy_args(L, f, parity);
+  CopyArgs a = copy_args(L, f);
   a.src = f.ptr(parity);
   a.src_rs = f.rs;
   a.red = red;
@@ -592,7 +616,7 @@ void clover_site(bridge_lattice_s* L, int prec, bool inverse, double kcsw, int p
                  const Field& dst, int dp, int nrhs, cudaStream_t st, CloverSet* set) {
   const char* cl = (set ? clover_ptr(L, *set, prec, inverse) : clover_ptr(L, prec, inverse, kcsw)) +
                    (long)parity * clover_block_bytes(prec, L->vh);
-  CopyArgs a = copy_args(L, src, sp);
+  CopyArgs a = copy_args(L, src);
   a.nrhs = nrhs;
   a.src = src.ptr(sp);
   a.src_rs = src.rs;

@@ -109,9 +109,7 @@ void vec_dispatch(int op, const StagVecArgs& a, cudaStream_t st) {
     case SV_CGP: stag_vec_kernel<P, PB, SV_CGP><<<grid, kThreads, 0, st>>>(a); break;
     case SV_NORM: stag_vec_kernel<P, PB, SV_NORM><<<grid, kThreads, 0, st>>>(a); break;
     case SV_CONVERT: stag_vec_kernel<P, PB, SV_CONVERT><<<grid, kThreads, 0, st>>>(a); break;
-    case SV_ACCUM: stag_vec_kernel<P, PB, SV_ACCUM><<<grid, kThreads, 0, st>>>(a); break;
-    case SV_FROM_CANON: stag_vec_kernel<P, PB, SV_FROM_CANON><<<grid, kThreads, 0, st>>>(a); break;
-    default: stag_vec_kernel<P, PB, SV_TO_CANON><<<grid, kThreads, 0, st>>>(a); break;
+    default: stag_vec_kernel<P, PB, SV_ACCUM><<<grid, kThreads, 0, st>>>(a); break;
   }
 }
 
@@ -175,15 +173,12 @@ void run_stag_hop(bridge_lattice_s* L, const bridge_op& op, const StagHop& c, cu
   BR_CUDA(cudaGetLastError());
 }
 
-StagVecArgs vec_args(bridge_lattice_s* L, int nrhs, int parity) {
+StagVecArgs vec_args(bridge_lattice_s* L, int nrhs) {
   StagVecArgs a;
   std::memset(static_cast<void*>(&a), 0, sizeof(a));
-  a.g = L->g;
   a.vh = (uint32_t)L->vh;
   a.nrhs = nrhs;
   a.nblk = vec_nblk(L->vh, nrhs);
-  a.parity = parity;
-  a.V = L->V;
   return a;
 }
 
@@ -198,28 +193,40 @@ void run_vec(bridge_lattice_s* L, int op, int prec, int precb, StagVecArgs a, do
 }  // namespace
 
 // ------------------------------------------------------------ conversions
+namespace {
+template <int P, bool TO_CANON>
+void stag_canon(bridge_lattice_s* L, const Field& f, double* canon, bool full, cudaStream_t st) {
+  StagCanonArgs a;
+  a.g = L->g;
+  a.vh = (uint32_t)L->vh;
+  a.nrhs = f.nrhs;
+  a.V = L->V;
+  a.full = full ? 1 : 0;
+  a.canon = canon;
+  a.even = f.ptr(f.subset == BRIDGE_FULL ? 0 : f.subset);
+  a.odd = f.ptr(1);
+  a.rs = f.rs;
+  const long n = full ? L->V : L->vh;
+  const double bytes = (double)n * f.nrhs * (48 + stag_site_bytes(f.prec));
+  note_launch(L, K_STAG_VEC, bytes, 0, st, true);
+  stag_canon_kernel<P, TO_CANON><<<(unsigned)((n + SC_SITES - 1) / SC_SITES * f.nrhs), SC_SITES, 0, st>>>(a);
+  note_launch(L, K_STAG_VEC, bytes, 0, st, false);
+  BR_CUDA(cudaGetLastError());
+}
+}  // namespace
+
 void stag_canon_to_field(bridge_lattice_s* L, const double* canon, const Field& f, bool canon_full, cudaStream_t st) {
-  const int lo = f.subset == BRIDGE_FULL ? 0 : f.subset, hi = f.subset == BRIDGE_FULL ? 1 : f.subset;
-  for (int p = lo; p <= hi; ++p) {
-    StagVecArgs a = vec_args(L, f.nrhs, p);
-    a.canon = const_cast<double*>(canon);
-    a.canon_full = canon_full;
-    a.a = f.ptr(p);
-    a.a_rs = f.rs;
-    run_vec(L, SV_FROM_CANON, f.prec, P_F64, a, 48 + stag_site_bytes(f.prec), st);
-  }
+  if (f.prec == P_F64)
+    stag_canon<P_F64, false>(L, f, const_cast<double*>(canon), canon_full, st);
+  else
+    stag_canon<P_F32, false>(L, f, const_cast<double*>(canon), canon_full, st);
 }
 
 void stag_field_to_canon(bridge_lattice_s* L, const Field& f, double* canon, bool canon_full, cudaStream_t st) {
-  const int lo = f.subset == BRIDGE_FULL ? 0 : f.subset, hi = f.subset == BRIDGE_FULL ? 1 : f.subset;
-  for (int p = lo; p <= hi; ++p) {
-    StagVecArgs a = vec_args(L, f.nrhs, p);
-    a.canon = canon;
-    a.canon_full = canon_full;
-    a.a = f.ptr(p);
-    a.a_rs = f.rs;
-    run_vec(L, SV_TO_CANON, f.prec, P_F64, a, 48 + stag_site_bytes(f.prec), st);
-  }
+  if (f.prec == P_F64)
+    stag_canon<P_F64, true>(L, f, canon, canon_full, st);
+  else
+    stag_canon<P_F32, true>(L, f, canon, canon_full, st);
 }
 
 // ------------------------------------------------------------ operators
@@ -326,7 +333,7 @@ int stag_solve(bridge_lattice_s* L, const bridge_op& op, const bridge_solver& pr
   auto norms = [&](const Field& f) {
     std::vector<double> out(nrhs, 0.0);
     for (int p = 0; p < 2; ++p) {
-      StagVecArgs a = vec_args(L, nrhs, p);
+      StagVecArgs a = vec_args(L, nrhs);
       a.a = f.ptr(p);
       a.a_rs = f.rs;
       a.red = red_of(FIN_STORE, 0, reinterpret_cast<double*>(resbuf.ptr) + p * 4 * nrhs);
@@ -404,7 +411,7 @@ int stag_solve(bridge_lattice_s* L, const bridge_op& op, const bridge_solver& pr
     for (int r = 0; r < nrhs; ++r) hmask[r] = (!done[r] && !failed[r]) ? 1 : 0;
     BR_CUDA(cudaMemcpyAsync(mask.ptr, hmask.data(), sizeof(int) * nrhs, cudaMemcpyHostToDevice, st));
     for (int p = 0; p < 2; ++p) {
-      StagVecArgs a = vec_args(L, nrhs, p);
+      StagVecArgs a = vec_args(L, nrhs);
       a.a = defect->ptr(p);
       a.a_rs = defect->rs;
       a.b = rin.ptr(p);
@@ -447,7 +454,7 @@ int stag_solve(bridge_lattice_s* L, const bridge_op& op, const bridge_solver& pr
     BR_CUDA(cudaMemcpyAsync(pe.buf->ptr, bh.buf->ptr, pe.buf->bytes, cudaMemcpyDeviceToDevice, st));
     BR_CUDA(cudaMemsetAsync(xe.buf->ptr, 0, xe.buf->bytes, st));
     {
-      StagVecArgs a = vec_args(L, nrhs, 0);
+      StagVecArgs a = vec_args(L, nrhs);
       a.a = cr.ptr(0);
       a.a_rs = cr.rs;
       a.red = red_of(FIN_CG_INIT, 0);
@@ -481,7 +488,7 @@ int stag_solve(bridge_lattice_s* L, const bridge_op& op, const bridge_solver& pr
       h2.out_rs = qe.rs;
       h2.redargs = red_of(FIN_CG_ALPHA, 1);
       run_stag_hop(L, op, h2, st);
-      StagVecArgs u = vec_args(L, nrhs, 0);
+      StagVecArgs u = vec_args(L, nrhs);
       u.a = xe.ptr(0);
       u.b = cr.ptr(0);
       u.c = pe.ptr(0);
@@ -489,7 +496,7 @@ int stag_solve(bridge_lattice_s* L, const bridge_op& op, const bridge_solver& pr
       u.a_rs = u.b_rs = u.c_rs = u.d_rs = xe.rs;
       u.red = red_of(FIN_CG_BETA, 1);
       run_vec(L, SV_CGUPD, P, P_F64, u, 6 * stag_site_bytes(P), st);
-      StagVecArgs v = vec_args(L, nrhs, 0);
+      StagVecArgs v = vec_args(L, nrhs);
       v.a = pe.ptr(0);
       v.b = cr.ptr(0);
       v.a_rs = v.b_rs = pe.rs;
@@ -538,7 +545,7 @@ int stag_solve(bridge_lattice_s* L, const bridge_op& op, const bridge_solver& pr
     }
     for (int p = 0; p < 2; ++p) {
       const Field& src = p == 0 ? xe : eo;
-      StagVecArgs a = vec_args(L, nrhs, p);
+      StagVecArgs a = vec_args(L, nrhs);
       a.a = src.ptr(p);
       a.a_rs = src.rs;
       a.b = x64.ptr(p);
