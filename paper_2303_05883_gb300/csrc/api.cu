@@ -94,26 +94,19 @@ static void mult_dev(bridge_lattice_s* L, const bridge_op& op, int prec, int whi
   if (op_is_staggered(op)) {
     BR_CHECK(prec == BRIDGE_F64 || prec == BRIDGE_F32, BRIDGE_EINVAL, "STAGGERED operators run in F64 or F32");
     BR_CHECK(which != APPLY_DHAT_DAG, BRIDGE_EINVAL, "bridge_mult_Dhat_dag is provided for MOBIUS operators only");
-    if (which == BRIDGE_APPLY_D) {
-      Field& fi = stag_workspace(L, "mult_in", prec, BRIDGE_FULL, nrhs);
-      Field& fo = stag_workspace(L, "mult_out", prec, BRIDGE_FULL, nrhs);
-      stag_canon_to_field(L, in, fi, true, st);
+    const bool full = which == BRIDGE_APPLY_D;
+    const int subset = full ? BRIDGE_FULL : which == BRIDGE_APPLY_DEO ? 1 - out_parity : BRIDGE_EVEN;
+    Field fi = stag_workspace(L, "mult_in", prec, subset, nrhs);
+    if (prec == BRIDGE_F64) fi.fx = stag_fx_input(L, nrhs * (full ? 2 : 1));
+    Field& fo = stag_workspace(L, "mult_out", prec, which == BRIDGE_APPLY_DEO ? out_parity : subset, nrhs);
+    stag_canon_to_field(L, in, fi, full, st);
+    if (full)
       stag_apply_d(L, op, fo, fi, st);
-      stag_field_to_canon(L, fo, out, true, st);
-    } else if (which == BRIDGE_APPLY_DEO) {
-      const int q = out_parity;
-      Field& fi = stag_workspace(L, "mult_in", prec, 1 - q, nrhs);
-      Field& fo = stag_workspace(L, "mult_out", prec, q, nrhs);
-      stag_canon_to_field(L, in, fi, false, st);
-      stag_apply_deo(L, op, q, fo, fi, st);
-      stag_field_to_canon(L, fo, out, false, st);
-    } else {
-      Field& fi = stag_workspace(L, "mult_in", prec, BRIDGE_EVEN, nrhs);
-      Field& fo = stag_workspace(L, "mult_out", prec, BRIDGE_EVEN, nrhs);
-      stag_canon_to_field(L, in, fi, false, st);
+    else if (which == BRIDGE_APPLY_DEO)
+      stag_apply_deo(L, op, out_parity, fo, fi, st);
+    else
       stag_apply_dhat(L, op, fo, fi, st);
-      stag_field_to_canon(L, fo, out, false, st);
-    }
+    stag_field_to_canon(L, fo, out, full, st);
     return;
   }
   if (op_is_mobius(op)) {

@@ -263,6 +263,9 @@ const char* clover_fx_ptr(bridge_lattice_s* L, CloverSet& set, bool inverse, cud
 // clover set of the flags that need one; scratch as HopCall::fx_scratch) and
 // queue the conversion of its input; or leave them null.
 void set_fx_args(bridge_lattice_s* L, HopArgs& a, int flags, int red, CloverSet* set, char* scratch, cudaStream_t st);
+// The lattice's scratch for hop inputs in fixed point (work on the lattice
+// stream), grown to `bytes`; null where there is no room or no growing now.
+char* fx_scratch(bridge_lattice_s* L, size_t bytes);
 // Where the FP64 application `which` (bridge_apply_op) of op on the lattice
 // stream runs in fixed point, room for nblocks half-lattice inputs; else null.
 char* fx_input(bridge_lattice_s* L, const bridge_op& op, int which, int nblocks);

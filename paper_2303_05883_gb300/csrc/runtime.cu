@@ -287,8 +287,7 @@ const char* clover_fx_ptr(bridge_lattice_s* L, CloverSet& set, bool inverse, cud
   return p;
 }
 
-char* fx_scratch(bridge_lattice_s* L, int nblocks) {
-  const size_t need = (size_t)nblocks * fx_block_bytes(L->vh);
+char* fx_scratch(bridge_lattice_s* L, size_t need) {
   if (!L->fx_scratch || L->fx_scratch->bytes < need) {
     if (capturing(L->stream)) return nullptr;
     L->fx_scratch.reset();
@@ -311,7 +310,7 @@ void set_fx_args(bridge_lattice_s* L, HopArgs& a, int flags, int red, CloverSet*
   const char* U = gauge_fx_ptr(L, st);
   if (!U) return;
   if (!a.in_fx) {
-    if (!scratch) scratch = fx_scratch(L, a.nrhs);
+    if (!scratch) scratch = fx_scratch(L, (size_t)a.nrhs * fx_block_bytes(L->vh));
     if (!scratch) return;
     CopyArgs c;
     std::memset(&c, 0, sizeof(c));
@@ -439,7 +438,7 @@ char* fx_input(bridge_lattice_s* L, const bridge_op& op, int which, int nblocks)
     auto set = clover_set(L, op_kcsw(op));
     if (!clover_fx_ptr(L, *set, which == BRIDGE_APPLY_DHAT, L->stream)) return nullptr;
   }
-  return fx_scratch(L, nblocks);
+  return fx_scratch(L, (size_t)nblocks * fx_block_bytes(L->vh));
 }
 
 void apply_deo(bridge_lattice_s* L, const bridge_op& op, int q, const Field& out, const Field& in, cudaStream_t st) {

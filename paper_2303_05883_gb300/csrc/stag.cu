@@ -82,7 +82,31 @@ int stag_nblk(int prec, int red, long vh, int nrhs) {
                           : hop_nblk<P_F32, SR_DOT_SELF>(vh, nrhs);
 }
 
+// Site blocks of a fixed-point launch.
+template <int RED>
+int fx_nblk(long vh, int nrhs) {
+  static int n = 0;
+  if (n == 0) {
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, stag_hop_fx_kernel<RED>, SFX_THREADS, 0);
+    if (n <= 0) n = 1;
+  }
+  const long cover = (vh + SFX_THREADS - 1) / SFX_THREADS, persist = (long)sm_count() * n / std::max(1, nrhs);
+  return (int)std::max<long>(1, std::min(cover, persist));
+}
+
+template <int RED>
+void launch_fx(StagArgs a, cudaStream_t st) {
+  a.nblk = fx_nblk<RED>(a.g.vh, a.nrhs);
+  stag_hop_fx_kernel<RED><<<(unsigned)(a.nblk * a.nrhs), SFX_THREADS, 0, st>>>(a);
+}
+
 void launch_stag_hop(int prec, int red, StagArgs a, cudaStream_t st) {
+  if (a.gauge_fx) {
+    if (red == SR_NONE) launch_fx<SR_NONE>(a, st);
+    else if (red == SR_NORM) launch_fx<SR_NORM>(a, st);
+    else launch_fx<SR_DOT_SELF>(a, st);
+    return;
+  }
   a.nblk = stag_nblk(prec, red, a.g.vh, a.nrhs);
   const unsigned grid = (unsigned)(a.nblk * a.nrhs);
   if (prec == P_F64) {
@@ -126,8 +150,16 @@ struct StagHop {
   const char *in = nullptr, *self = nullptr, *aux = nullptr;
   char* out = nullptr;
   long in_rs = 0, out_rs = 0, self_rs = 0, aux_rs = 0;
+  const char* in_fx = nullptr;  // FP64: `in` in fixed point, where the caller has it already
+  long in_fx_rs = 0;
   RedArgs redargs{};
 };
+
+// The fixed-point form of a field's parity block (Field::fx), and the stride.
+const char* fx_of(const Field& f, int parity) {
+  return f.fx ? f.fx + ((f.subset == BRIDGE_FULL && parity == 1) ? stag_fx_block_bytes(f.vh) : 0) : nullptr;
+}
+long fx_stride(const Field& f) { return (f.subset == BRIDGE_FULL ? 2 : 1) * stag_fx_block_bytes(f.vh); }
 
 void run_stag_hop(bridge_lattice_s* L, const bridge_op& op, const StagHop& c, cudaStream_t st) {
   StagArgs a;
@@ -155,8 +187,29 @@ void run_stag_hop(bridge_lattice_s* L, const bridge_op& op, const StagHop& c, cu
   a.aux_rs = c.aux_rs;
   a.gauge = gauge_ptr(L, c.prec);
   a.red = c.redargs;
+  if (c.prec == P_F64) {
+    // in fixed point, unless the links have no such copy or there is no room for the input's
+    const char* U = gauge_fx_ptr(L, st);
+    a.in_fx = c.in_fx;
+    a.in_fx_rs = c.in_fx_rs;
+    if (U && !a.in_fx && st == L->stream) {
+      char* to = fx_scratch(L, (size_t)c.nrhs * stag_fx_block_bytes(L->vh));
+      if (to) {
+        const int nb = vec_nblk(L->vh, c.nrhs);
+        const double bytes = (double)L->vh * c.nrhs * (48 + 52);
+        a.in_fx = to;
+        a.in_fx_rs = stag_fx_block_bytes(L->vh);
+        note_launch(L, K_STAG_VEC, bytes, 0, st, true);
+        stag_to_fx_kernel<<<(unsigned)(nb * c.nrhs), 256, 0, st>>>(c.in, c.in_rs, to, a.in_fx_rs, (uint32_t)L->vh, c.nrhs, nb,
+                                                                  c.redargs);
+        note_launch(L, K_STAG_VEC, bytes, 0, st, false);
+      }
+    }
+    if (a.in_fx) a.gauge_fx = U;
+  }
   if (c.red != SR_NONE && a.red.partials == nullptr) {
-    ensure_red_scratch(L, (long)stag_nblk(c.prec, c.red, L->vh, c.nrhs) * c.nrhs, c.nrhs);
+    const long nb = std::max<long>(stag_nblk(c.prec, c.red, L->vh, c.nrhs), (L->vh + SFX_THREADS - 1) / SFX_THREADS);
+    ensure_red_scratch(L, nb * c.nrhs, c.nrhs);
     a.red.partials = reinterpret_cast<double*>(L->red_partials->ptr);
     a.red.counter = reinterpret_cast<unsigned*>(L->red_counter->ptr);
     a.red.result = reinterpret_cast<double*>(L->red_result->ptr);
@@ -206,14 +259,21 @@ void stag_canon(bridge_lattice_s* L, const Field& f, double* canon, bool full, c
   a.even = f.ptr(f.subset == BRIDGE_FULL ? 0 : f.subset);
   a.odd = f.ptr(1);
   a.rs = f.rs;
+  a.fx = f.fx;
+  a.fx2 = f.fx ? f.fx + stag_fx_block_bytes(L->vh) : nullptr;
+  a.fx_rs = fx_stride(f);
   const long n = full ? L->V : L->vh;
-  const double bytes = (double)n * f.nrhs * (48 + stag_site_bytes(f.prec));
+  const double bytes = (double)n * f.nrhs * (48 + stag_site_bytes(f.prec) + (f.fx ? 52 : 0));
   note_launch(L, K_STAG_VEC, bytes, 0, st, true);
   stag_canon_kernel<P, TO_CANON><<<(unsigned)((n + SC_SITES - 1) / SC_SITES * f.nrhs), SC_SITES, 0, st>>>(a);
   note_launch(L, K_STAG_VEC, bytes, 0, st, false);
   BR_CUDA(cudaGetLastError());
 }
 }  // namespace
+
+char* stag_fx_input(bridge_lattice_s* L, int nblocks) {
+  return gauge_fx_ptr(L, L->stream) ? fx_scratch(L, (size_t)nblocks * stag_fx_block_bytes(L->vh)) : nullptr;
+}
 
 void stag_canon_to_field(bridge_lattice_s* L, const double* canon, const Field& f, bool canon_full, cudaStream_t st) {
   if (f.prec == P_F64)
@@ -238,6 +298,8 @@ void stag_apply_deo(bridge_lattice_s* L, const bridge_op& op, int q, const Field
   h.nrhs = in.nrhs;
   h.in = in.ptr(1 - q);
   h.in_rs = in.rs;
+  h.in_fx = fx_of(in, 1 - q);
+  h.in_fx_rs = fx_stride(in);
   h.out = out.ptr(q);
   h.out_rs = out.rs;
   run_stag_hop(L, op, h, st);
@@ -251,6 +313,8 @@ void stag_apply_d(bridge_lattice_s* L, const bridge_op& op, const Field& out, co
     h.nrhs = in.nrhs;
     h.in = in.ptr(1 - q);
     h.in_rs = in.rs;
+    h.in_fx = fx_of(in, 1 - q);
+    h.in_fx_rs = fx_stride(in);
     h.self = in.ptr(q);
     h.self_rs = in.rs;
     h.s1 = op.mass;
@@ -269,6 +333,8 @@ void stag_apply_dhat(bridge_lattice_s* L, const bridge_op& op, const Field& out,
   h1.nrhs = in.nrhs;
   h1.in = in.ptr(0);
   h1.in_rs = in.rs;
+  h1.in_fx = fx_of(in, 0);
+  h1.in_fx_rs = fx_stride(in);
   h1.out = t.ptr(1);
   h1.out_rs = t.rs;
   run_stag_hop(L, op, h1, st);
@@ -314,7 +380,7 @@ int stag_solve(bridge_lattice_s* L, const bridge_op& op, const bridge_solver& pr
   Field qe = make_stag_field(P, BRIDGE_EVEN, nrhs, L->vh), to = make_stag_field(P, BRIDGE_ODD, nrhs, L->vh);
   Field eo = make_stag_field(P, BRIDGE_ODD, nrhs, L->vh);
 
-  const long nblk_max = (L->vh + kThreads - 1) / kThreads;
+  const long nblk_max = (L->vh + SFX_THREADS - 1) / SFX_THREADS;  // the most site blocks of any launch
   DevBuf sc(sizeof(CGScalars) * nrhs), partials(sizeof(double) * 4 * nblk_max * nrhs), counter(256);
   DevBuf mask(sizeof(int) * nrhs), resbuf(sizeof(double) * 4 * nrhs * 2);
   PinnedBuf h_sc(sizeof(CGScalars) * nrhs), h_res(sizeof(double) * 4 * nrhs * 2);

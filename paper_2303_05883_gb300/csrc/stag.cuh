@@ -18,7 +18,7 @@
 // with an optional fused reduction of |out|^2 or Re <self, out>.
 #pragma once
 
-#include "common.cuh"
+#include "dslash_fx.cuh"
 #include "reduce.cuh"
 
 namespace bridge {
@@ -96,6 +96,9 @@ struct StagArgs {
   const char* aux;   // may be null
   long aux_rs;
   const char* gauge;  // [parity][mu] link blocks
+  const char* gauge_fx;  // FP64 in fixed point: the links and the input
+  const char* in_fx;
+  long in_fx_rs;
   RedArgs red;
 };
 
@@ -131,6 +134,49 @@ BR_D void stag_dir(const StagArgs& a, const char* in, const char* g_out, const c
   stag_hop_one<P, MU, false>(in, g_in + MU * lbb, a.g.vh, b, b, wb, bc, eta, acc);
 }
 
+// One output site: v, and s = the self vector (where there is one).
+template <int P>
+BR_D void stag_site(const StagArgs& a, int rhs, uint32_t ih, cx<typename Tr<P>::R> v[3], cx<typename Tr<P>::R> s[3]) {
+  using R = typename Tr<P>::R;
+  const int p = a.out_parity;
+  const long vh = a.g.vh, lbb = link_block_bytes(P, vh);
+  const char* g_out = a.gauge + (long)p * 4 * lbb;
+  const char* g_in = a.gauge + (long)(1 - p) * 4 * lbb;
+  const char* in = a.in + rhs * a.in_rs;
+  const R sc = pick<R>(a.scale, a.scalef), s1 = pick<R>(a.s1, a.s1f), ca = pick<R>(a.caux, a.cauxf);
+  int c[4];
+  uint32_t xh;
+  site_coords(a.g, ih, p, c, xh);
+  cx<R> acc[3] = {czero<R>(), czero<R>(), czero<R>()};
+  stag_dir<P, 0>(a, in, g_out, g_in, lbb, ih, c, xh, R(1), acc);
+  stag_dir<P, 1>(a, in, g_out, g_in, lbb, ih, c, xh, (c[0] & 1) ? R(-1) : R(1), acc);
+  stag_dir<P, 2>(a, in, g_out, g_in, lbb, ih, c, xh, ((c[0] + c[1]) & 1) ? R(-1) : R(1), acc);
+  stag_dir<P, 3>(a, in, g_out, g_in, lbb, ih, c, xh, ((c[0] + c[1] + c[2]) & 1) ? R(-1) : R(1), acc);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) v[k] = sc * acc[k];
+  if (a.self != nullptr) {
+    load_cvec<P>(a.self + rhs * a.self_rs, vh, ih, s);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) v[k] = v[k] + s1 * s[k];
+  }
+  if (a.aux != nullptr) {
+    cx<R> w[3];
+    load_cvec<P>(a.aux + rhs * a.aux_rs, vh, ih, w);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) v[k] = v[k] + ca * w[k];
+  }
+}
+
+// One site's contribution to the fused reduction.
+template <int RED, class R>
+BR_D R stag_red(const cx<R> v[3], const cx<R> s[3]) {
+  R n = 0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    n += RED == SR_NORM ? v[k].r * v[k].r + v[k].i * v[k].i : s[k].r * v[k].r + s[k].i * v[k].i;
+  return n;
+}
+
 template <int P, int RED>
 __global__ void __launch_bounds__(256) stag_hop_kernel(const StagArgs a) {
   using R = typename Tr<P>::R;
@@ -141,53 +187,191 @@ __global__ void __launch_bounds__(256) stag_hop_kernel(const StagArgs a) {
   PartialSum<R> ps;
   const bool skip = a.red.check_done && a.red.cg != nullptr && a.red.cg[rhs].done != RUNNING;
   if (!skip) {
-    const int p = a.out_parity;
-    const long lbb = link_block_bytes(P, vh);
-    const char* g_out = a.gauge + (long)p * 4 * lbb;
-    const char* g_in = a.gauge + (long)(1 - p) * 4 * lbb;
-    const char* in = a.in + rhs * a.in_rs;
-    const R sc = pick<R>(a.scale, a.scalef), s1 = pick<R>(a.s1, a.s1f), ca = pick<R>(a.caux, a.cauxf);
     const uint32_t stride = (uint32_t)a.nblk * blockDim.x;
     for (uint32_t ih = sb * blockDim.x + threadIdx.x; ih < (uint32_t)vh; ih += stride) {
-      int c[4];
-      uint32_t xh;
-      site_coords(a.g, ih, p, c, xh);
-      cx<R> acc[3] = {czero<R>(), czero<R>(), czero<R>()};
-      stag_dir<P, 0>(a, in, g_out, g_in, lbb, ih, c, xh, R(1), acc);
-      stag_dir<P, 1>(a, in, g_out, g_in, lbb, ih, c, xh, (c[0] & 1) ? R(-1) : R(1), acc);
-      stag_dir<P, 2>(a, in, g_out, g_in, lbb, ih, c, xh, ((c[0] + c[1]) & 1) ? R(-1) : R(1), acc);
-      stag_dir<P, 3>(a, in, g_out, g_in, lbb, ih, c, xh, ((c[0] + c[1] + c[2]) & 1) ? R(-1) : R(1), acc);
       cx<R> v[3], s[3];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) v[k] = sc * acc[k];
-      if (a.self != nullptr) {
-        load_cvec<P>(a.self + rhs * a.self_rs, vh, ih, s);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) v[k] = v[k] + s1 * s[k];
-      }
-      if (a.aux != nullptr) {
-        cx<R> w[3];
-        load_cvec<P>(a.aux + rhs * a.aux_rs, vh, ih, w);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) v[k] = v[k] + ca * w[k];
-      }
+      stag_site<P>(a, rhs, ih, v, s);
       store_cvec<P>(a.out + rhs * a.out_rs, vh, ih, v);
-      if (RED == SR_NORM) {
-        R n = 0;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) n += v[k].r * v[k].r + v[k].i * v[k].i;
-        ps.add(n);
-      } else if (RED == SR_DOT_SELF) {
-        R d = 0;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) d += s[k].r * v[k].r + s[k].i * v[k].i;
-        ps.add(d);
-      }
+      if (RED != SR_NONE) ps.add(stag_red<RED, R>(v, s));
     }
   }
   if (RED != SR_NONE) {
     double rv[1] = {ps.value()};
     reduce_finalize<1>(a.red, rhs, sb, a.nblk, nrhs, rv);
+  }
+}
+
+// ------------------------------------------------------------ fixed point
+// The FP64 hop in 64-bit fixed point, as dslash_fx.cuh: the same integer links,
+// the colour vectors in units of 2^(E - 1081) with one exponent a site (three
+// 16-byte planes, then one int a site), one rounding a hop.  36 products of
+// three IMAD.WIDE a hop; a site has nothing to project or reconstruct, so one
+// thread a site keeps its sum, a hop's rows and both hops' loads of a direction
+// in 128 registers.  Measured (one parity of 32^4): FP64 kernel 340 us, at the
+// FP64 pipe's limit (0.90 TFLOP/s); here 127 us = 5.3 TB/s, 0.79 of HBM.
+BR_HD long stag_fx_block_bytes(long vh) { return pad256(52 * vh); }
+constexpr int SFX_THREADS = 128;
+
+BR_D void stag_fx_store(char* block, long vh, uint32_t ih, const cx<double> v[3]) {
+  uint4 w[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    w[k] = make_uint4((uint32_t)__double2loint(v[k].r), (uint32_t)__double2hiint(v[k].r), (uint32_t)__double2loint(v[k].i),
+                      (uint32_t)__double2hiint(v[k].i));
+  const uint32_t m = fx_max_word<3>(w);
+  const int E = (int)(m >> 20);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const long long r = fx_from_bits<6>(w[k].x, w[k].y, E, 0), i = fx_from_bits<6>(w[k].z, w[k].w, E, 0);
+    reinterpret_cast<uint4*>(block)[k * vh + ih] =
+        make_uint4((uint32_t)r, (uint32_t)(r >> 32), (uint32_t)i, (uint32_t)(i >> 32));
+  }
+  reinterpret_cast<int*>(block + 48 * vh)[ih] = m == 0 ? 0 : (E < FX_EMIN || E > FX_EMAX) ? -1 : E;
+}
+
+// Slots of one site (direction 2 mu + backward): neighbour index, bit 31 the
+// sign of the hop (staggered and boundary phase, - for backward), exponent.
+template <int MU>
+BR_D void stag_fx_slots(const StagArgs& a, const int* ex, uint32_t ih, const int c[4], uint32_t xh, uint32_t eta_neg,
+                        uint2 (*w)[SFX_THREADS], int& Ea, bool& bad) {
+  uint32_t f, b;
+  bool wf, wb;
+  neighbours<MU>(a.g, ih, c, xh, f, b, wf, wb);
+  const uint32_t neg = a.bcf[MU] < 0.f;
+  const int ef = __ldg(ex + f), eb = __ldg(ex + b);
+  bad = bad || ef < 0 || eb < 0;
+  Ea = max(Ea, max(ef, eb));
+  w[2 * MU][threadIdx.x] = make_uint2(f | ((eta_neg ^ (wf & neg)) << 31), (uint32_t)ef);
+  w[2 * MU + 1][threadIdx.x] = make_uint2(b | ((eta_neg ^ (wb & neg) ^ 1u) << 31), (uint32_t)eb);
+}
+
+struct StagFxLoads {
+  uint4 v[3], l[9];
+};
+BR_D void stag_fx_load(StagFxLoads& f, const char* in, const char* g, long vs, uint32_t nb, uint32_t li) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) f.v[k] = __ldg(reinterpret_cast<const uint4*>(in + k * vs) + nb);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) f.l[k] = ldg4<true>(reinterpret_cast<const uint4*>(g + k * vs) + li);
+}
+
+template <bool FWD>
+BR_D void stag_fx_mac(const StagFxLoads& f, uint2 w, int Ea, cx<long long> acc[3]) {
+  long long rh[3] = {0, 0, 0}, rm[3] = {0, 0, 0}, jh[3] = {0, 0, 0}, jm[3] = {0, 0, 0};
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const cx<long long> v = fx_value(f.v[c]);
+    const Fx2 hr = fx_split(v.r), hi = fx_split(v.i);
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const uint4 l = f.l[FWD ? 3 * r + c : 3 * c + r];
+      const Fx2 ur = {(int)l.y, (int)l.x}, ui = {(int)l.w, (int)l.z}, nui = fx_neg(ui);
+      fx_mac(ur, hr, rh[r], rm[r]);
+      fx_mac(FWD ? nui : ui, hi, rh[r], rm[r]);
+      fx_mac(ur, hi, jh[r], jm[r]);
+      fx_mac(FWD ? ui : nui, hr, jh[r], jm[r]);
+    }
+  }
+  const int d = min(Ea - (int)w.y, 62);  // a zero neighbour (exponent 0): rounds to zero
+  const long long half = (1ll << d) >> 1;
+  const int m = -(int)(w.x >> 31);
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    acc[r].r += fx_sign((rh[r] + fx_split(rm[r]).h + half) >> d, m);
+    acc[r].i += fx_sign((jh[r] + fx_split(jm[r]).h + half) >> d, m);
+  }
+}
+
+// The site in FP64, where a neighbour has no fixed-point form.
+__device__ __noinline__ inline void stag_fx_site_fp64(const StagArgs& a, int rhs, uint32_t ih, double2* out) {
+  cx<double> v[3], s[3];
+  stag_site<P_F64>(a, rhs, ih, v, s);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) out[k] = make_double2(v[k].r, v[k].i);
+}
+
+template <int RED>
+__global__ void __launch_bounds__(SFX_THREADS, 4) stag_hop_fx_kernel(const StagArgs a) {
+  const int nrhs = a.nrhs;
+  const int rhs = blockIdx.x % nrhs;
+  const int sb = blockIdx.x / nrhs;
+  const long vh = a.g.vh, vs = 16 * vh;
+  __shared__ uint2 slot[8][SFX_THREADS];
+  PartialSum<double> ps;
+  const bool skip = a.red.check_done && a.red.cg != nullptr && a.red.cg[rhs].done != RUNNING;
+  if (!skip) {
+    const int p = a.out_parity;
+    const long lbb = link_block_bytes(P_F64, vh);
+    const char* g_out = a.gauge_fx + (long)p * 4 * lbb;
+    const char* g_in = a.gauge_fx + (long)(1 - p) * 4 * lbb;
+    const char* in = a.in_fx + rhs * a.in_fx_rs;
+    const int* ex = reinterpret_cast<const int*>(in + 48 * vh);
+    const uint32_t stride = (uint32_t)a.nblk * SFX_THREADS;
+    for (uint32_t ih = sb * SFX_THREADS + threadIdx.x; ih < (uint32_t)vh; ih += stride) {
+      int Ea = 0;
+      bool bad = false;
+      {
+        int c[4];
+        uint32_t xh;
+        site_coords(a.g, ih, p, c, xh);
+        stag_fx_slots<0>(a, ex, ih, c, xh, 0u, slot, Ea, bad);
+        stag_fx_slots<1>(a, ex, ih, c, xh, c[0] & 1, slot, Ea, bad);
+        stag_fx_slots<2>(a, ex, ih, c, xh, (c[0] + c[1]) & 1, slot, Ea, bad);
+        stag_fx_slots<3>(a, ex, ih, c, xh, (c[0] + c[1] + c[2]) & 1, slot, Ea, bad);
+      }
+      cx<double> v[3], s[3];
+      if (a.self != nullptr) load_cvec<P_F64>(a.self + rhs * a.self_rs, vh, ih, s);
+      if (bad) {
+        double2 w[3];
+        stag_fx_site_fp64(a, rhs, ih, w);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) v[k] = {w[k].x, w[k].y};
+      } else {
+        cx<long long> acc[3] = {{0, 0}, {0, 0}, {0, 0}};
+#pragma unroll 1
+        for (int mu = 0; mu < 4; ++mu) {
+          StagFxLoads f, b;
+          const uint2 wf = slot[2 * mu][threadIdx.x], wb = slot[2 * mu + 1][threadIdx.x];
+          const uint32_t nf = wf.x & 0x7fffffffu, nb = wb.x & 0x7fffffffu;
+          stag_fx_load(f, in, g_out + mu * lbb, vs, nf, ih);
+          stag_fx_load(b, in, g_in + mu * lbb, vs, nb, nb);
+          stag_fx_mac<true>(f, wf, Ea, acc);
+          stag_fx_mac<false>(b, wb, Ea, acc);
+        }
+        const double sc = Ea == 0 ? 0.0 : a.scale * fx_pow2(Ea - 54);
+        cx<double> t[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) t[k] = czero<double>();
+        if (a.aux != nullptr) {
+          load_cvec<P_F64>(a.aux + rhs * a.aux_rs, vh, ih, t);
+#pragma unroll
+          for (int k = 0; k < 3; ++k) t[k] = a.caux * t[k];
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          if (a.self != nullptr) t[k] = caxpy(a.s1, s[k], t[k]);
+          v[k] = caxpy(sc, cx<double>{(double)acc[k].r, (double)acc[k].i}, t[k]);
+        }
+      }
+      store_cvec<P_F64>(a.out + rhs * a.out_rs, vh, ih, v);
+      if (RED != SR_NONE) ps.add(stag_red<RED, double>(v, s));
+    }
+  }
+  if (RED != SR_NONE) {
+    double rv[1] = {ps.value()};
+    reduce_finalize<1>(a.red, rhs, sb, a.nblk, nrhs, rv);
+  }
+}
+
+// FP64 colour vectors -> their fixed-point form.
+__global__ void __launch_bounds__(256) stag_to_fx_kernel(const char* src, long src_rs, char* dst, long dst_rs, uint32_t vh,
+                                                         int nrhs, int nblk, RedArgs red) {
+  const int rhs = blockIdx.x % nrhs;
+  if (rhs_finished(red, rhs)) return;
+  for (uint32_t ih = (blockIdx.x / nrhs) * blockDim.x + threadIdx.x; ih < vh; ih += (uint32_t)nblk * blockDim.x) {
+    cx<double> v[3];
+    load_cvec<P_F64>(src + rhs * src_rs, vh, ih, v);
+    stag_fx_store(dst + rhs * dst_rs, vh, ih, v);
   }
 }
 
@@ -295,19 +479,21 @@ struct StagCanonArgs {
   double* canon;
   char *even, *odd;   // the parity blocks (half-lattice: `even`)
   long rs;
+  char *fx, *fx2;     // from canonical FP64: the fixed-point form too (null: none), as even and odd
+  long fx_rs;
 };
 
 // Parity block and half-lattice index of canonical site k.
-BR_D char* stag_where(const StagCanonArgs& a, long k, uint32_t& ih) {
+BR_D int stag_where(const StagCanonArgs& a, long k, uint32_t& ih) {
   if (!a.full) {
     ih = (uint32_t)k;
-    return a.even;
+    return 0;
   }
   int c[4];
   uint32_t xh;
   ih = (uint32_t)(k >> 1);
   site_coords(a.g, ih, 0, c, xh);
-  return ((int)(k & 1) ^ (c[0] & 1)) ? a.odd : a.even;
+  return (int)(k & 1) ^ (c[0] & 1);
 }
 
 template <int P, bool TO_CANON>
@@ -328,7 +514,8 @@ __global__ void __launch_bounds__(SC_SITES) stag_canon_kernel(const StagCanonArg
   }
   if (t < n) {
     uint32_t ih;
-    char* block = stag_where(a, base + t, ih) + rhs * a.rs;
+    const int p = stag_where(a, base + t, ih);
+    char* block = (p ? a.odd : a.even) + rhs * a.rs;
     cx<R> v[3];
     if (TO_CANON) {
       load_cvec<P>(block, a.vh, ih, v);
@@ -341,6 +528,8 @@ __global__ void __launch_bounds__(SC_SITES) stag_canon_kernel(const StagCanonArg
         v[k] = {(R)w.x, (R)w.y};
       }
       store_cvec<P>(block, a.vh, ih, v);
+      if constexpr (P == P_F64)
+        if (a.fx) stag_fx_store((p ? a.fx2 : a.fx) + rhs * a.fx_rs, a.vh, ih, v);
     }
   }
   if (TO_CANON) {

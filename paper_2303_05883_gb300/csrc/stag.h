@@ -18,6 +18,10 @@ Field& stag_workspace(bridge_lattice_s* L, const std::string& name, int prec, in
 void stag_canon_to_field(bridge_lattice_s* L, const double* canon, const Field& f, bool canon_full, cudaStream_t st);
 void stag_field_to_canon(bridge_lattice_s* L, const Field& f, double* canon, bool canon_full, cudaStream_t st);
 
+// Room for the fixed-point form of nblocks half-lattice FP64 inputs (to set as
+// Field::fx of a hop input), or null where FP64 hops do not run in fixed point.
+char* stag_fx_input(bridge_lattice_s* L, int nblocks);
+
 // D, D_eo / D_oe and the Schur operator of Eq. 1, asynchronous on st.
 void stag_apply_d(bridge_lattice_s* L, const bridge_op& op, const Field& out, const Field& in, cudaStream_t st);
 void stag_apply_deo(bridge_lattice_s* L, const bridge_op& op, int out_parity, const Field& out, const Field& in,

@@ -122,3 +122,46 @@ def test_values_without_a_fixed_point_form(api, value):
         inner = [i for i in range(130, 270) if np.abs(b[i]).max() < 1e-300]
         for i in inner:
             assert np.abs(a[i] - b[i]).max() <= 8e-15 * np.abs(b[i]).max() + 1e-320
+
+
+@pytest.mark.parametrize("dims,nrhs", [((2, 2, 2, 2), 1), ((4, 4, 4, 4), 2), ((6, 4, 10, 6), 3)])
+@pytest.mark.parametrize("bc", [(1, 1, 1, -1), (-1, 1, -1, 1)])
+def test_staggered_fixed_point_equals_the_fp64_kernel(api, dims, nrhs, bc):
+    """Links 2 U with mass 2 m give 2 D on the FP64 kernel (links above 1)."""
+    U = synth.gauge_field(dims, 0.4, 3)
+    V = int(np.prod(dims))
+    chi = synth.gaussian_spinor(dims, 5, nrhs=nrhs)[:, :, 0].copy()
+    chi *= 10.0 ** np.random.default_rng(1).uniform(-12, 12, (nrhs, V, 1))
+    chi[:, V // 3] = 0
+    chi[0, V // 2, 1] = 1e-303  # a site without a fixed-point form, finite
+    chi[0, V // 2, [0, 2]] = 0
+    got = []
+    for s in (1.0, 2.0):
+        L = api.Lattice(dims)
+        op = api.make_staggered(0.1 * s, bc)
+        L.upload(s * U, op)
+        half = chi[:, : V // 2].copy()
+        got.append([L.D(op, chi) / s, L.Deo(op, half, 0) / s, L.Deo(op, half, 1) / s, L.Dhat(op, half)])
+    for a, b in zip(*got):
+        assert rel(a, b) < TOL
+        scale = np.abs(b).max(axis=2)
+        assert np.all(np.abs(a - b).max(axis=2) <= 8e-15 * scale + 1e-318)
+
+
+def test_staggered_nan_and_infinity(api):
+    dims = (6, 4, 10, 6)
+    U = synth.gauge_field(dims, 0.4, 3)
+    chi = synth.gaussian_spinor(dims, 5)[:, 0].copy()
+    chi[7, 1] = np.nan
+    chi[500, 2] = np.inf
+    got = []
+    with np.errstate(all="ignore"):
+        for s in (1.0, 2.0):
+            L = api.Lattice(dims)
+            op = api.make_staggered(0.1 * s)
+            L.upload(s * U, op)
+            got.append(L.D(op, chi) / s)
+    a, b = (g.view(np.float64) for g in got)
+    assert np.array_equal(np.isnan(a), np.isnan(b)) and np.array_equal(np.isinf(a), np.isinf(b))
+    ok = np.isfinite(b)
+    assert rel(a[ok], b[ok]) < TOL
