@@ -231,12 +231,34 @@ std::string mix_key(const bridge_lattice_s* L, int prec, int mode, int Ls, int n
   return "dwfmix/" + std::to_string(prec) + "/" + std::to_string(mode) + "/Ls" + std::to_string(Ls) + "/" +
          dims_tag(L) + "/" + std::to_string(nrhs);
 }
-// Tuned (threads, variant) for a key; FP32 default 256 threads, variant 0.
-LaunchShape dwf_shape(bridge_lattice_s* L, int prec, const std::string& key) {
+// What an untuned FP32 launch takes.  Below 2^17 five-dimensional sites of
+// one parity every shape takes the same time (the launch and the latency of
+// one block); above, fewer registers for more resident warps win, and for the
+// longest epilogue two slices a thread.  Microseconds on a GB300, 256 threads
+// of variant 0 -> the choice, at 16^3 x 32 with Ls 4 / 8 / 16 and 24^4 with Ls 10:
+//   mix                  21 -> 17, 29 -> 23, 53 -> 43,             111 -> 84
+//   pass 1               45 -> 35, 62 -> 51, 103 -> 92,            227 -> 189
+//   pass 2               44 -> 36, 64 -> 54, 107 -> 95,            224 -> 181
+//   pass 2 with |q|^2    54 -> 48, 83 -> 69, 141 -> 113,           282 -> 222
+//   pass 2 with CG update 66 -> 65, 97 -> 93, 167 -> 155,          332 -> 293
+//   D_eo                 27 -> 25, 46 -> 41, 78 -> 69,             144 -> 115
+//   two operands (prepare, D) 55 -> 48, 72 -> 69, 125 -> 113,      276 -> 243
+LaunchShape dwf_default(long sites5, int Ls, bool hop, bool m1, int m2, int epi) {
+  if (sites5 < (1L << 17)) return LaunchShape{256, 0, 0};
+  if (!hop || !m1) return LaunchShape{128, 0, 1};
+  const int wide = Ls >= 16 ? 256 : 128;
+  if (m2 == DM2_DENSE) return LaunchShape{wide, 0, 1};
+  if (epi == DE_NORM) return LaunchShape{256, 0, 2};
+  if (epi == DE_CGUPD) return LaunchShape{256, 0, Ls >= 10 ? 4 : 1};
+  return LaunchShape{wide, 0, 2};
+}
+
+// Tuned (threads, variant) for a key, else the default.
+LaunchShape dwf_shape(bridge_lattice_s* L, int prec, const std::string& key, const LaunchShape& dflt) {
   if (prec == P_F64) return LaunchShape{kMinThreads, 0, 0};
   std::lock_guard<std::mutex> lk(L->tune_mu);
   auto it = L->tuned.find(key);
-  if (it == L->tuned.end()) return LaunchShape{256, 0, 0};
+  if (it == L->tuned.end()) return dflt;
   LaunchShape s = it->second;  // (a hand-set entry may ask for fewer threads than the scratch is sized for)
   s.block = std::max(s.block, kMinThreads);
   if (s.variant < 0 || s.variant >= DWF_NVARIANT) s.variant = 0;
@@ -260,7 +282,9 @@ struct DwfHop {
 void run_dwf_hop(bridge_lattice_s* L, const DwfSet& set, const bridge_op& op, const DwfHop& c, cudaStream_t st) {
   const int m2mode = c.self_plain ? DM2_PLAIN : c.m2 >= 0 ? DM2_DENSE : DM2_NONE;
   const LaunchShape sh =
-      c.shape ? *c.shape : dwf_shape(L, c.prec, hop_key(L, c.prec, c.m1 >= 0, m2mode, c.epi, c.Ls, c.nrhs));
+      c.shape ? *c.shape
+              : dwf_shape(L, c.prec, hop_key(L, c.prec, c.m1 >= 0, m2mode, c.epi, c.Ls, c.nrhs),
+                          dwf_default(L->vh * c.Ls * c.nrhs, c.Ls, true, c.m1 >= 0, m2mode, c.epi));
   DwfArgs a;
   std::memset(static_cast<void*>(&a), 0, sizeof(a));
   a.g = L->g;
@@ -340,7 +364,10 @@ struct DwfMix {
 };
 
 void run_dwf_mix(bridge_lattice_s* L, const DwfSet& set, const DwfMix& c, cudaStream_t st) {
-  const LaunchShape sh = c.shape ? *c.shape : dwf_shape(L, c.prec, mix_key(L, c.prec, c.mode, c.Ls, c.nrhs));
+  const LaunchShape sh =
+      c.shape ? *c.shape
+              : dwf_shape(L, c.prec, mix_key(L, c.prec, c.mode, c.Ls, c.nrhs),
+                          dwf_default(L->vh * c.Ls * c.nrhs, c.Ls, false, false, DM2_NONE, DE_NONE));
   DwfMixArgs a;
   std::memset(static_cast<void*>(&a), 0, sizeof(a));
   a.vh = (uint32_t)L->vh;
