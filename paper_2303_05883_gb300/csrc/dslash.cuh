@@ -282,6 +282,7 @@ __global__ void __launch_bounds__(256, MINB) hop_kernel(const HopArgs a) {
   constexpr int NV = RED == R_NORM ? 1 : RED == R_DOT_A ? 2 : 3;
   PartialSum<R> ps[NV];
   const bool skip = rhs_finished(a.red, rhs);
+  if (skip && all_finished(a.red, nrhs)) return;
   if (!skip) {
     const int p = a.out_parity;
     const uint32_t stride = (uint32_t)a.nblk * blockDim.x;
@@ -386,6 +387,7 @@ __global__ void __launch_bounds__(256) hop_kernel_mr(const HopArgs a) {
     live[r] = (r0 + r < a.nrhs) && !rhs_finished(a.red, r0 + r);
     any = any || live[r];
   }
+  if (!any && all_finished(a.red, a.nrhs)) return;
   PartialSum<T> ps[NR][NV];
   const T beta = pick<T>(a.beta, a.betaf), s1 = pick<T>(a.s1, a.s1f), ca = pick<T>(a.caux, a.cauxf);
   if (any) {

@@ -301,7 +301,9 @@ __global__ void __launch_bounds__(FX_THREADS, 4) hop_kernel_fx(const HopArgs a) 
   constexpr int NV = RED == R_NORM ? 1 : RED == R_DOT_A ? 2 : 3;
   __shared__ FxSlots sh;
   PartialSum<double> ps[NV];
-  if (!rhs_finished(a.red, rhs)) {
+  const bool skip = rhs_finished(a.red, rhs);
+  if (skip && all_finished(a.red, nrhs)) return;
+  if (!skip) {
     const int p = a.out_parity, site = threadIdx.x >> 1, k = threadIdx.x & 1;
     const long lbb = link_block_bytes(P_F64, vh), cbb = clover_block_bytes(P_F64, vh);
     const char* g_out = a.gauge_fx + (long)p * 4 * lbb;

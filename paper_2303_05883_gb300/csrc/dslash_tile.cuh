@@ -284,6 +284,7 @@ __global__ void __launch_bounds__(32 * TILE_MAX_RHS, 2) hop_kernel_tile(const Ho
   const long vh = a.g.vh;
   constexpr int NV = RED == R_NORM ? 1 : RED == R_DOT_A ? 2 : 3;
   const bool live = rhs < a.nrhs && w < G && !rhs_finished(a.red, rhs);
+  if (rhs_finished(a.red, grp * G) && all_finished(a.red, a.nrhs)) return;
   PartialSum<float> ps[NV];
   const int p = a.out_parity;
   const long lbb = link_block_bytes(P, vh), cbb = clover_block_bytes(P, vh);
@@ -430,14 +431,14 @@ __global__ void __launch_bounds__(32 * TILE_MAX_RHS, 2) hop_kernel_tile(const Ho
     // one warp per right-hand side: the warp's sum is the block's partial
     double rv[NV];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      rv[k] = ps[k].value();
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) rv[k] += __shfl_xor_sync(0xffffffffu, rv[k], off);
+    for (int k = 0; k < NV; ++k) rv[k] = ps[k].value();
+    const double t = warp_sum<NV>(rv);
+    constexpr int W = warp_sum_lanes<NV>();
+    if (lane % W == 0 && lane / W < NV && rhs < a.nrhs && w < G) {
+      a.red.partials[((long)rhs * a.nblk + sb) * 4 + lane / W] = t;
+      __threadfence();
     }
-    if (lane == 0 && rhs < a.nrhs && w < G)
-#pragma unroll
-      for (int k = 0; k < NV; ++k) a.red.partials[((long)rhs * a.nblk + sb) * 4 + k] = rv[k];
+    __syncthreads();
     grid_finish<NV>(a.red, a.nblk, a.nrhs);
   }
 }

@@ -447,6 +447,7 @@ __global__ void __launch_bounds__(256, MINB) dwf_hop_kernel(const DwfArgs a) {
   const long vh = a.g.vh;
   const bool live = s0 < lss;
   const bool skip = a.red.check_done && a.red.cg != nullptr && a.red.cg[rhs].done != RUNNING;
+  if (skip && all_finished(a.red, a.nrhs)) return;
   const bool valid = live && ih < (uint32_t)vh && !skip;
   const long q0 = (long)rhs * Ls + s0;  // slice j of this thread: q0 + j * lss
 

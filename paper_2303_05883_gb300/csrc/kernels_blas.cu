@@ -63,6 +63,7 @@ __global__ void __launch_bounds__(256) k_blas_xr(const BlasArgs a) {
   const int rhs = blockIdx.x % a.nrhs, sb = blockIdx.x / a.nrhs;
   const BiCGScalars* q = a.red.sc + rhs;
   PartialSum<R> ps[3];
+  if (q->done != RUNNING && all_finished(a.red, a.nrhs)) return;
   if (q->done == RUNNING) {
     const cx<R> al = {(R)q->alpha_r, (R)q->alpha_i}, om = {(R)q->omega_r, (R)q->omega_i};
     BR_SITE_LOOP(a.vh, a.nblk) {
@@ -147,6 +148,7 @@ __global__ void __launch_bounds__(256) k_cg_xr(const BlasArgs a) {
   const int rhs = blockIdx.x % a.nrhs, sb = blockIdx.x / a.nrhs;
   const CGScalars* q = a.red.cg + rhs;
   PartialSum<R> ps;
+  if (q->done != RUNNING && all_finished(a.red, a.nrhs)) return;
   if (q->done == RUNNING) {
     const R al = (R)q->alpha;
     BR_SITE_LOOP(a.vh, a.nblk) {

@@ -410,8 +410,9 @@ __global__ void __launch_bounds__(256) mg_coarse_kernel(const MgCoarseArgs a) {
   const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
   const int n2 = N2 > 0 ? N2 : a.n2;
   const bool skip = RED != MG_CR_NONE && a.red.sc != nullptr && a.red.sc[0].done != RUNNING;
+  if (skip) return;
   double rv[3] = {0.0, 0.0, 0.0};
-  if (!skip && t < (long)a.m.nblocks * n2) {
+  if (t < (long)a.m.nblocks * n2) {
     const int X = (int)(t / n2), row = (int)(t % n2);
     // the tiled FP16 copy of the unrolled row lengths goes to mg_coarse_tma_kernel
     cx<float> s;
@@ -469,9 +470,9 @@ __global__ void __launch_bounds__(256) mg_coarse_tma_kernel(const MgCoarseArgs a
   constexpr long CT = TILE / 9;  // bytes of one coupling
   const int tid = threadIdx.x, nt = blockDim.x;
   const int stages = a.stages;
-  const bool skip = RED != MG_CR_NONE && a.red.sc != nullptr && a.red.sc[0].done != RUNNING;
+  if (RED != MG_CR_NONE && a.red.sc != nullptr && a.red.sc[0].done != RUNNING) return;
   const int nsites = a.parity < 0 ? a.m.nblocks : a.m.nblocks / 2, first = blockIdx.x, step = gridDim.x;
-  const int mine = (skip || first >= nsites) ? 0 : (nsites - first + step - 1) / step;
+  const int mine = first >= nsites ? 0 : (nsites - first + step - 1) / step;
   const int d0 = a.d0, nd = a.d1 - a.d0;
   const uint32_t cbytes = (uint32_t)(nd * CT);
   auto site = [&](int k) { return a.parity < 0 ? k : mg_colour_block(a.m, a.parity, k); };
@@ -707,13 +708,13 @@ struct MgCBicgArgs {
 template <int OP>
 __global__ void __launch_bounds__(256) mg_cbicg_kernel(const MgCBicgArgs a) {
   const BiCGScalars* q = a.red.sc;
-  const bool skip = OP != MG_CB_INIT && q->done != RUNNING;
+  if (OP != MG_CB_INIT && q->done != RUNNING) return;
   PartialSum<float> p0, p1, p2;
   auto c = [](float2 f) { return cx<float>{f.x, f.y}; };
   auto f2 = [](cx<float> v) { return make_float2(v.r, v.i); };
   const cx<float> al{(float)q->alpha_r, (float)q->alpha_i}, om{(float)q->omega_r, (float)q->omega_i};
   const cx<float> be{(float)q->beta_r, (float)q->beta_i};
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; !skip && i < a.n; i += (long)gridDim.x * blockDim.x) {
+  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += (long)gridDim.x * blockDim.x) {
     if (OP == MG_CB_INIT) {
       const float2 bb = a.b[i];
       a.x[i] = make_float2(0.f, 0.f);

@@ -186,6 +186,7 @@ __global__ void __launch_bounds__(256) stag_hop_kernel(const StagArgs a) {
   const long vh = a.g.vh;
   PartialSum<R> ps;
   const bool skip = a.red.check_done && a.red.cg != nullptr && a.red.cg[rhs].done != RUNNING;
+  if (skip && all_finished(a.red, a.nrhs)) return;
   if (!skip) {
     const uint32_t stride = (uint32_t)a.nblk * blockDim.x;
     for (uint32_t ih = sb * blockDim.x + threadIdx.x; ih < (uint32_t)vh; ih += stride) {
@@ -299,6 +300,7 @@ __global__ void __launch_bounds__(SFX_THREADS, 4) stag_hop_fx_kernel(const StagA
   __shared__ uint2 slot[8][SFX_THREADS];
   PartialSum<double> ps;
   const bool skip = a.red.check_done && a.red.cg != nullptr && a.red.cg[rhs].done != RUNNING;
+  if (skip && all_finished(a.red, a.nrhs)) return;
   if (!skip) {
     const int p = a.out_parity;
     const long lbb = link_block_bytes(P_F64, vh);
@@ -402,6 +404,7 @@ __global__ void __launch_bounds__(256) stag_vec_kernel(const StagVecArgs a) {
   PartialSum<R> ps;
   const bool skip = (OP == SV_CGUPD || OP == SV_CGP) && a.red.cg != nullptr && a.red.cg[rhs].done != RUNNING;
   const bool on = a.mask == nullptr || a.mask[rhs] != 0;
+  if (skip && all_finished(a.red, a.nrhs)) return;
   if (!skip) {
     const uint32_t stride = (uint32_t)a.nblk * blockDim.x;
     for (uint32_t ih = sb * blockDim.x + threadIdx.x; ih < a.vh; ih += stride) {
