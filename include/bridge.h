@@ -67,9 +67,11 @@ enum bridge_status {
 };
 
 /* Storage precision of a field or of an operator application.  F64 computes
- * in FP64; F32 stores and computes in FP32; F16/BF16 store spinors as 16-bit
- * values times a per-site FP32 scale (max |component|), links and clover
- * blocks as plain 16-bit values, and compute in FP32. */
+ * to FP64 accuracy (Wilson, clover and staggered hopping terms in 64-bit fixed
+ * point where links and clover blocks are in its range, else in FP64); F32
+ * stores and computes in FP32; F16/BF16 store spinors as 16-bit values times a
+ * per-site FP32 scale (max |component|), links and clover blocks as plain
+ * 16-bit values, and compute in FP32. */
 enum bridge_prec { BRIDGE_F64 = 0, BRIDGE_F32 = 1, BRIDGE_F16 = 2, BRIDGE_BF16 = 3 };
 
 enum bridge_kind { BRIDGE_WILSON = 0, BRIDGE_CLOVER = 1, BRIDGE_MOBIUS = 2, BRIDGE_STAGGERED = 3 };
@@ -133,7 +135,7 @@ typedef struct {
   int inner_prec;    /* bridge_prec of the inner solver (mixed = 1) */
   double inner_tol;  /* inner relative tolerance; <= 0 picks 1e-5 (F32), 2e-3 (F16/BF16) */
   int mixed;         /* 1: FP64 defect correction around an inner_prec solver; 0: plain FP64 */
-  int check_every;   /* iterations between host convergence polls (<= 0: 16) */
+  int check_every;   /* at most this many iterations between host convergence polls (<= 0: 16) */
   int use_graph;     /* 1: replay iteration batches as CUDA graphs */
   int max_outer;     /* limit on defect-correction passes (<= 0: 50) */
   int method;        /* WILSON/CLOVER inner solver: BRIDGE_METHOD_AUTO (0) BiCGStab, switching to CG on the
