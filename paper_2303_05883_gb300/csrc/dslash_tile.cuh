@@ -433,9 +433,9 @@ __global__ void __launch_bounds__(32 * TILE_MAX_RHS, 2) hop_kernel_tile(const Ho
 #pragma unroll
     for (int k = 0; k < NV; ++k) rv[k] = ps[k].value();
     const double t = warp_sum<NV>(rv);
-    constexpr int W = warp_sum_lanes<NV>();
-    if (lane % W == 0 && lane / W < NV && rhs < a.nrhs && w < G) {
-      a.red.partials[((long)rhs * a.nblk + sb) * 4 + lane / W] = t;
+    constexpr int LW = warp_sum_lanes<NV>();
+    if (lane % LW == 0 && lane / LW < NV && rhs < a.nrhs && w < G) {
+      a.red.partials[((long)rhs * a.nblk + sb) * 4 + lane / LW] = t;
       __threadfence();
     }
     __syncthreads();
