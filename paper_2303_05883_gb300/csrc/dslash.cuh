@@ -517,7 +517,7 @@ bool hop_has_variants(int flags, int red);
 // storage only, v = 11, 12; dslash_tile.cuh).
 inline int hop_variant_rpt(int variant) { return variant >= 9 ? 12 : variant >= 6 ? variant - 4 : 1; }
 constexpr int HOP_NVARIANT = 13;
-// Added to 9 or 10 by the untuned launches: FP16 spinors projected in FP32.
+// Added to 9 or 10 by the untuned launches: the tile kernel rounding as variant 0.
 constexpr int HOP_TILE_WIDE = 4;
 inline bool hop_variant_for_prec(int variant, int prec) { return variant < 11 || prec == P_F16 || prec == P_BF16; }
 inline bool hop_variant_is_tile(int variant) { return variant >= 9; }

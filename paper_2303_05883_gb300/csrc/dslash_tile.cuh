@@ -7,9 +7,9 @@
 // right-hand side (group start + w) for the 32 sites of the tile, so every
 // spinor access of a warp is one coalesced 512-byte row per plane.  Per tile
 // the block first stages, once for all G right-hand sides,
-//   * the eight links of each site (row 2 rebuilt, the backward links stored
-//     as their adjoint, every link pre-multiplied by beta and by the boundary
-//     phase of its hop) as FP32 in shared memory,
+//   * the eight links of each site (row 2 rebuilt, pre-multiplied by the
+//     boundary phase of its hop; except in PT launches also by beta and, for
+//     the backward links, as their adjoint) as FP32 in shared memory,
 //   * the T^-1 blocks of the site (F_E_CLOV), unpacked to FP32,
 //   * the half-lattice indices of the eight neighbours,
 // and then each thread runs the eight projected hops of its (site, rhs) with
@@ -103,8 +103,10 @@ BR_D void project_f16(const uint32_t w[12], cx<float> hh[2][3]) {
   }
 }
 
-// Stage the link of hop h (= 2 mu + backward) of chunk site s (S sites per chunk).
-template <int P, int MU, int S>
+// Stage the link of hop h (= 2 mu + backward) of chunk site s (S sites per
+// chunk): beta * phase * U, or its adjoint for a backward hop; PT: phase * U
+// (exact, the phase is 1, -1 or 0) for both, row 2 conjugated.
+template <int P, int MU, int S, bool PT>
 BR_D void tile_stage_link(const HopArgs& a, const char* g_out, const char* g_in, long lbb, uint32_t ih, int p, int h,
                           int s, float4* sl, uint32_t* snb) {
   int c[4];
@@ -116,12 +118,14 @@ BR_D void tile_stage_link(const HopArgs& a, const char* g_out, const char* g_in,
   const bool fwd = (h & 1) == 0;
   Link<float> U;
   load_link<P, true>((fwd ? g_out : g_in) + MU * lbb, a.g.vh, fwd ? ih : b, U);
-  const float coef = a.betaf * ((fwd ? wf : wb) ? a.bcf[MU] : 1.0f);
+  const float phase = (fwd ? wf : wb) ? a.bcf[MU] : 1.0f;
+  const float coef = PT ? phase : a.betaf * phase;
   cx<float> m[9];
 #pragma unroll
   for (int r = 0; r < 3; ++r)
 #pragma unroll
-    for (int q = 0; q < 3; ++q) m[3 * r + q] = fwd ? coef * U.m[r][q] : coef * conj(U.m[q][r]);
+    for (int q = 0; q < 3; ++q)
+      m[3 * r + q] = PT ? coef * (r == 2 ? conj(U.m[2][q]) : U.m[r][q]) : fwd ? coef * U.m[r][q] : coef * conj(U.m[q][r]);
   float4* d = sl + h * 5 * S + s;
   d[0 * S] = make_float4(m[0].r, m[0].i, m[1].r, m[1].i);
   d[1 * S] = make_float4(m[2].r, m[2].i, m[3].r, m[3].i);
@@ -132,15 +136,15 @@ BR_D void tile_stage_link(const HopArgs& a, const char* g_out, const char* g_in,
 }
 
 // One hop of one (site, rhs) with the staged link M (already beta * phase *
-// U or its adjoint): acc += (1 -/+ gamma_mu) M psi(neighbour).  W: FP16 spinors
-// are widened before the projection instead of projected in half2.
-template <int P, int MU, bool FWD, int S, bool W>
+// U or its adjoint): acc += (1 -/+ gamma_mu) M psi(neighbour).  PT: the same
+// operations in the same order as hop_one, on M = phase * U.
+template <int P, int MU, bool FWD, int S, bool PT>
 BR_D void tile_hop(const char* in, long vh, const float4* sl, const uint32_t* snb, int s, cx<float> acc[12]) {
   constexpr int h = 2 * MU + (FWD ? 0 : 1);
   const uint32_t nb = snb[h * S + s];
   cx<float> hh[2][3];
   float sc = 1.0f;
-  if constexpr (P == P_F16 && !W) {
+  if constexpr (P == P_F16 && !PT) {
     const uint4* pl = reinterpret_cast<const uint4*>(in);
     const uint4 v0 = __ldg(pl + nb), v1 = __ldg(pl + vh + nb), v2 = __ldg(pl + 2 * vh + nb);
     sc = __ldg(reinterpret_cast<const float*>(in + 48 * vh) + nb);
@@ -159,15 +163,32 @@ BR_D void tile_hop(const char* in, long vh, const float4* sl, const uint32_t* sn
   const float4 q0 = q[0], q1 = q[S], q2 = q[2 * S], q3 = q[3 * S], q4 = q[4 * S];
   const cx<float> m00 = {q0.x, q0.y}, m01 = {q0.z, q0.w}, m02 = {q1.x, q1.y};
   const cx<float> m10 = {q1.z, q1.w}, m11 = {q2.x, q2.y}, m12 = {q2.z, q2.w};
-  const cx<float> m20 = {q3.x, q3.y}, m21 = {q3.z, q3.w}, m22 = {q4.x, q4.y};
+  cx<float> m20 = {q3.x, q3.y}, m21 = {q3.z, q3.w}, m22 = {q4.x, q4.y};
+  if constexpr (PT) {  // a conjugate, as in recon_row2: products with it contract the other way round
+    m20 = conj(m20);
+    m21 = conj(m21);
+    m22 = conj(m22);
+  }
   cx<float> u[2][3];
+  if constexpr (PT && Tr<P>::half) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) hh[k][c] = sc * hh[k][c];
+  }
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
-    u[k][0] = crow3(m00, m01, m02, hh[k]);
-    u[k][1] = crow3(m10, m11, m12, hh[k]);
-    u[k][2] = crow3(m20, m21, m22, hh[k]);
+    if constexpr (PT && !FWD) {
+      u[k][0] = crow3_conj(m00, m10, m20, hh[k]);
+      u[k][1] = crow3_conj(m01, m11, m21, hh[k]);
+      u[k][2] = crow3_conj(m02, m12, m22, hh[k]);
+    } else {
+      u[k][0] = crow3(m00, m01, m02, hh[k]);
+      u[k][1] = crow3(m10, m11, m12, hh[k]);
+      u[k][2] = crow3(m20, m21, m22, hh[k]);
+    }
   }
-  if constexpr (Tr<P>::half)
+  if constexpr (Tr<P>::half && !PT)
     reconstruct_scaled<MU, FWD>(u, sc, acc);
   else
     reconstruct<float, MU, FWD>(u, acc);
@@ -260,9 +281,14 @@ BR_D void tile_pf_step(const char* in, long vh, const float4* sl, const uint32_t
 
 // NT tiles (NT x 32 sites) are staged between two barriers; the register
 // budget allows two resident 384-thread blocks per SM.  PF: pipelined
-// neighbour loads (16-bit storage only).  W: FP32 projection of FP16 spinors
-// (the untuned launches: they round no more than the per-thread kernel does).
-template <int P, int FL, int RED, int NT, bool PF = false, bool W = false>
+// neighbour loads (16-bit storage only).  PT: every site's result is that of
+// the per-thread kernel (hop_site) bit for bit, so that which of the two an
+// untuned launch takes, a matter of its working set, does not show in its
+// result: the projection of FP16 spinors in FP32, the per-site scale and beta
+// stay where that kernel has them.  Four D^ on 12 right-hand sides of 24^3 x
+// 48 in FP16: per-thread kernel 3752 us, PT 2908, with scale and beta folded
+// into links and sums 2805.
+template <int P, int FL, int RED, int NT, bool PF = false, bool PT = false>
 __global__ void __launch_bounds__(32 * TILE_MAX_RHS, 2) hop_kernel_tile(const HopArgs a) {
   static_assert(!PF || Tr<P>::half, "pipelined neighbour loads: 16-bit storage");
   static_assert(P != P_F64, "FP32 arithmetic kernels only");
@@ -303,10 +329,10 @@ __global__ void __launch_bounds__(32 * TILE_MAX_RHS, 2) hop_kernel_tile(const Ho
       if (j < 8 * S) {
         const int h = j / S;
         switch (h >> 1) {
-          case 0: tile_stage_link<P, 0, S>(a, g_out, g_in, lbb, ih, p, h, s, sl, snb); break;
-          case 1: tile_stage_link<P, 1, S>(a, g_out, g_in, lbb, ih, p, h, s, sl, snb); break;
-          case 2: tile_stage_link<P, 2, S>(a, g_out, g_in, lbb, ih, p, h, s, sl, snb); break;
-          default: tile_stage_link<P, 3, S>(a, g_out, g_in, lbb, ih, p, h, s, sl, snb); break;
+          case 0: tile_stage_link<P, 0, S, PT>(a, g_out, g_in, lbb, ih, p, h, s, sl, snb); break;
+          case 1: tile_stage_link<P, 1, S, PT>(a, g_out, g_in, lbb, ih, p, h, s, sl, snb); break;
+          case 2: tile_stage_link<P, 2, S, PT>(a, g_out, g_in, lbb, ih, p, h, s, sl, snb); break;
+          default: tile_stage_link<P, 3, S, PT>(a, g_out, g_in, lbb, ih, p, h, s, sl, snb); break;
         }
       } else if constexpr (CL) {
         const int b = (j - 8 * S) / S;
@@ -343,14 +369,14 @@ __global__ void __launch_bounds__(32 * TILE_MAX_RHS, 2) hop_kernel_tile(const Ho
         tile_pf_step<P, 6, S>(in, vh, sl, snb, s, pf, t, acc);
         tile_pf_step<P, 7, S>(in, vh, sl, snb, s, pf, t, acc);
       } else {
-        tile_hop<P, 0, true, S, W>(in, vh, sl, snb, s, acc);
-        tile_hop<P, 0, false, S, W>(in, vh, sl, snb, s, acc);
-        tile_hop<P, 1, true, S, W>(in, vh, sl, snb, s, acc);
-        tile_hop<P, 1, false, S, W>(in, vh, sl, snb, s, acc);
-        tile_hop<P, 2, true, S, W>(in, vh, sl, snb, s, acc);
-        tile_hop<P, 2, false, S, W>(in, vh, sl, snb, s, acc);
-        tile_hop<P, 3, true, S, W>(in, vh, sl, snb, s, acc);
-        tile_hop<P, 3, false, S, W>(in, vh, sl, snb, s, acc);
+        tile_hop<P, 0, true, S, PT>(in, vh, sl, snb, s, acc);
+        tile_hop<P, 0, false, S, PT>(in, vh, sl, snb, s, acc);
+        tile_hop<P, 1, true, S, PT>(in, vh, sl, snb, s, acc);
+        tile_hop<P, 1, false, S, PT>(in, vh, sl, snb, s, acc);
+        tile_hop<P, 2, true, S, PT>(in, vh, sl, snb, s, acc);
+        tile_hop<P, 2, false, S, PT>(in, vh, sl, snb, s, acc);
+        tile_hop<P, 3, true, S, PT>(in, vh, sl, snb, s, acc);
+        tile_hop<P, 3, false, S, PT>(in, vh, sl, snb, s, acc);
       }
       // the staged site term times x
       auto site_term = [&](const cx<float> x[12], cx<float> y[12]) {
@@ -369,11 +395,23 @@ __global__ void __launch_bounds__(32 * TILE_MAX_RHS, 2) hop_kernel_tile(const Ho
           hermitian6_apply<float>(m, x + 6 * b, y + 6 * b);
         }
       };
+      // r + s x; PT, with r = beta * acc (first): the product that is not
+      // rounded by itself is that with beta, as the per-thread kernel contracts
+      // its beta * acc + s * x
+      auto plus = [&](float s, cx<float> x, cx<float> r, bool first) {
+        if (PT && first) return cx<float>{fmaf(a.betaf, r.r, __fmul_rn(s, x.r)), fmaf(a.betaf, r.i, __fmul_rn(s, x.i))};
+        return caxpy(s, x, r);
+      };
+      constexpr bool fresh = !(FL & F_AUX) && !(FL & F_E_CLOV);
+      if constexpr (PT && !(FL & F_AUX) && ((FL & F_E_CLOV) || !(FL & F_SELF))) {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) acc[k] = a.betaf * acc[k];
+      }
       if constexpr ((FL & F_AUX) != 0) {
         cx<float> x[12];
         load_spinor<P, true, true>(a.aux + (long)rhs * a.aux_rs, vh, ih, x);
 #pragma unroll
-        for (int k = 0; k < 12; ++k) acc[k] = caxpy(a.cauxf, x[k], acc[k]);
+        for (int k = 0; k < 12; ++k) acc[k] = plus(a.cauxf, x[k], acc[k], true);
       }
       if constexpr ((FL & F_G5) != 0) {
 #pragma unroll
@@ -393,10 +431,10 @@ __global__ void __launch_bounds__(32 * TILE_MAX_RHS, 2) hop_kernel_tile(const Ho
           cx<float> ms[12];
           site_term(sv, ms);
 #pragma unroll
-          for (int k = 0; k < 12; ++k) v[k] = caxpy(a.s1f, ms[k], v[k]);
+          for (int k = 0; k < 12; ++k) v[k] = plus(a.s1f, ms[k], v[k], fresh);
         } else {
 #pragma unroll
-          for (int k = 0; k < 12; ++k) v[k] = caxpy(a.s1f, sv[k], v[k]);
+          for (int k = 0; k < 12; ++k) v[k] = plus(a.s1f, sv[k], v[k], fresh);
         }
       }
       store_spinor<P>(a.out + (long)rhs * a.out_rs, vh, ih, v);

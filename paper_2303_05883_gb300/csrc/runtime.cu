@@ -639,9 +639,9 @@ bool hop_has_variants(int flags, int red) {
 //   * from 4 right-hand sides on 2^18 half-lattice sites, or 6 on 2^16, the
 //     tile kernel, which loads, widens and scales each link and clover block
 //     once for all of them: 24^3 x 48 F32 4 RHS 123 -> 113 / 189 -> 163, 12
-//     RHS 332 -> 283 / 525 -> 388, F16 12 RHS 347 -> 246 / 424 -> 330 (projected
-//     in half2; in FP32, as untuned launches do, four D^ on 12 RHS take 2.3 ms
-//     instead of 2.9); 16^3 x 32 6 RHS 39 -> 38 / 72 -> 68, but 4 RHS 27 -> 29 /
+//     RHS 332 -> 283 / 525 -> 388, F16 12 RHS 347 -> 246 / 424 -> 330 (variants 9
+//     and 10; rounding as variant 0, as untuned launches do, four D^ on 12 RHS in
+//     F16 take 2.9 ms with their conversions instead of 3.8); 16^3 x 32 6 RHS 39 -> 38 / 72 -> 68, but 4 RHS 27 -> 29 /
 //     51 -> 53, and 12^3 x 16 12 RHS 17 -> 21 / 40 -> 58 (too few tiles for the
 //     SMs).  Two tiles a barrier from 8 right-hand sides (195 against 208), one
 //     below (157 against 170);
