@@ -336,7 +336,10 @@ int bridge_tune_table(bridge_lattice lat, char* out, int n);
  * loads for 0-5, 2-4 right-hand sides per thread for 6-8, the shared-link
  * tile kernel for 9-10, the same with pipelined neighbour loads for 11-12,
  * FP16/BF16 storage only; a variant a kernel does not have falls back to
- * 0).  Lets tests and users pin a launch shape; EINVAL for values out of
+ * 0).  The tile kernels choose their own block size: for 9 and 10, block 64
+ * is the kernel that folds scales into links and sums (FP16: projects in
+ * half precision), any other the one that rounds as variant 0, which untuned
+ * launches take.  Lets tests and users pin a launch shape; EINVAL for values out of
  * range. */
 int bridge_tune_set(bridge_lattice lat, const char* key, int block, int nblk, int variant);
 

@@ -127,12 +127,15 @@ struct LaunchShape {
   int block = 256;
   int nblk = 0;     // site blocks per rhs; 0 -> cover the lattice once
   int variant = 0;  // register-budget variant of the kernel (see launch_hop)
-  bool untuned = false;  // a default, not measured or set
 };
 
-// The kernel variant of a shape.
+// The kernel variant of a shape.  The tile kernels choose their own block
+// size; in a shape of variant 9 or 10 the block says which of them: 64 (what
+// the tuner writes) the one with folded scaling, another (the defaults) the
+// one that rounds as variant 0.  A line of the table names one kernel, set or
+// read back.
 inline int launch_variant(const LaunchShape& s) {
-  return s.variant + (s.untuned && (s.variant == 9 || s.variant == 10) ? HOP_TILE_WIDE : 0);
+  return s.variant + (s.block != 64 && (s.variant == 9 || s.variant == 10) ? HOP_TILE_WIDE : 0);
 }
 
 struct Stats {

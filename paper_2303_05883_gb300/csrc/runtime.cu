@@ -139,7 +139,6 @@ LaunchShape shape_for(bridge_lattice_s* L, const std::string& key, long vh, int 
     s = it->second;
   } else {
     s.variant = variant;
-    s.untuned = true;
     s.block = variant == 4 && !cover_once ? 256 : 128;
     const int per_sm = occ ? occ(s.block) : 0;
     const long resident = (long)sm_count() * (per_sm > 0 ? per_sm : 4);

@@ -52,3 +52,20 @@ def test_default_kernels_round_alike(api, links, kind, csw, prec, nrhs):
         got.append((L.D(op, psi, prec), L.Deo(op, half, 0, prec), L.Deo(op, half, 1, prec), L.Dhat(op, half, prec)))
     for a, b in zip(*got):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("prec,nrhs", [("f16", 6), ("f16", 9), ("f32", 6)])
+def test_the_printed_table_selects_the_same_kernels(api, links, prec, nrhs):
+    """Every line of bridge_tune_table, set on another lattice, runs the kernel it was printed for."""
+    half = synth.gaussian_spinor(DIMS, 4, nrhs=nrhs)[:, Lattice(DIMS).even]
+    op = api.make_op("clover", 0.12, 1.0)
+    got, table = [], {}
+    for _ in range(2):
+        L = api.Lattice(DIMS)
+        L.upload(links, op)
+        for key, shape in table.items():
+            api.bridge_tune_set(L.handle, key, *shape)
+        got.append(L.Dhat(op, half, prec))
+        table = api.bridge_tune_table(L.handle)
+        assert any(shape[2] in (9, 10) for shape in table.values())
+    assert np.array_equal(*got)
