@@ -510,7 +510,24 @@ template <>
 bool launch_hop<P_F16>(int flags, int red, const HopArgs& a, int block, cudaStream_t st, int* occ, int variant);
 template <>
 bool launch_hop<P_BF16>(int flags, int red, const HopArgs& a, int block, cudaStream_t st, int* occ, int variant);
-bool hop_has_variants(int flags, int red);
+// The (flags, reduction) pairs each family of variants is instantiated for
+// (dslash_inst.inc); hop_has_variant reads the same lists.
+// 1-5, register budget and read-once loads:
+#define BRIDGE_HOP_BUDGET_CASES(X)                                                      \
+  X(0, R_NONE) X(F_E_CLOV, R_NONE) X(F_SELF, R_DOT_A) X(F_SELF, R_TS)                   \
+  X(F_SELF | F_E_CLOV, R_DOT_A) X(F_SELF | F_E_CLOV, R_TS) X(F_AUX | F_SELF | F_SELF_CLOV, R_NORM)
+// of these 4 alone, the default of the operator applications:
+#define BRIDGE_HOP_APPLY_CASES(X) X(F_SELF, R_NONE) X(F_SELF | F_E_CLOV, R_NONE) X(F_SELF | F_SELF_CLOV, R_NONE)
+// 6-8, several right-hand sides per thread, and 9-12, tile kernels with folded scaling:
+#define BRIDGE_HOP_SHARED_CASES(X)                                                      \
+  X(0, R_NONE) X(F_E_CLOV, R_NONE) X(F_SELF, R_DOT_A) X(F_SELF, R_TS)                   \
+  X(F_SELF | F_E_CLOV, R_DOT_A) X(F_SELF | F_E_CLOV, R_TS)
+// the tile kernel that rounds as variant 0 besides (9, 10 too): operator
+// applications, even-odd preparation, CG on the normal equations
+#define BRIDGE_HOP_TILE_CASES(X)                                                        \
+  X(F_SELF, R_NONE) X(F_SELF | F_E_CLOV, R_NONE) X(F_SELF | F_SELF_CLOV, R_NONE)        \
+  X(F_AUX, R_NONE) X(F_AUX | F_E_CLOV, R_NONE) X(F_SELF, R_NORM) X(F_SELF | F_E_CLOV, R_NORM) X(F_SELF | F_G5, R_NONE)
+bool hop_has_variant(int prec, int flags, int red, int variant);
 // Right-hand sides covered by one block group of a variant: 1 for v < 6, NR
 // for the NR-per-thread kernels (v = 6, 7, 8) and up to 12 for the
 // shared-link tile kernels (v = 9, 10; with pipelined neighbour loads, 16-bit
@@ -519,7 +536,6 @@ inline int hop_variant_rpt(int variant) { return variant >= 9 ? 12 : variant >= 
 constexpr int HOP_NVARIANT = 13;
 // Added to 9 or 10 by the untuned launches: the tile kernel rounding as variant 0.
 constexpr int HOP_TILE_WIDE = 4;
-inline bool hop_variant_for_prec(int variant, int prec) { return variant < 11 || prec == P_F16 || prec == P_BF16; }
 inline bool hop_variant_is_tile(int variant) { return variant >= 9; }
 
 }  // namespace bridge

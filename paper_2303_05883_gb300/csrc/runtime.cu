@@ -627,9 +627,17 @@ void clover_site(bridge_lattice_s* L, int prec, bool inverse, double kcsw, int p
   BR_CUDA(cudaGetLastError());
 }
 
-bool hop_has_variants(int flags, int red) {
-  return (flags & (F_E_CLOV | F_SELF_CLOV)) != (F_E_CLOV | F_SELF_CLOV) &&
-         !((flags & F_AUX) && (flags & F_SELF) && red == R_NORM && !(flags & F_SELF_CLOV));
+bool hop_has_variant(int prec, int flags, int red, int variant) {
+#define BRIDGE_HOP_IS(FL, RD) || (flags == (FL) && red == (RD))
+  const bool budget = false BRIDGE_HOP_BUDGET_CASES(BRIDGE_HOP_IS), apply = false BRIDGE_HOP_APPLY_CASES(BRIDGE_HOP_IS);
+  const bool shared = false BRIDGE_HOP_SHARED_CASES(BRIDGE_HOP_IS), tile = false BRIDGE_HOP_TILE_CASES(BRIDGE_HOP_IS);
+#undef BRIDGE_HOP_IS
+  if (variant == 0) return true;
+  if (prec == P_F64) return false;
+  if (variant < 6) return budget || (variant == 4 && apply);
+  if (variant < 9) return shared;
+  if (variant < 11) return shared || tile;
+  return shared && (prec == P_F16 || prec == P_BF16);
 }
 
 // The variant an untuned launch takes, by its working set (microseconds on a
@@ -648,15 +656,16 @@ bool hop_has_variants(int flags, int red) {
 //     read-once operands past L1, 256-thread blocks (pass 2, 32^3 x 64: F32
 //     186 -> 175, 3 RHS 429 -> 360, F16 136 -> 130); on 16^3 x 32 it is slower.
 static int default_hop_variant(int prec, int flags, int red, long vh, int nrhs, bool mapped) {
-  if (prec == P_F64 || mapped || !hop_has_variants(flags, red)) return 0;
+  if (mapped) return 0;
   const int per_block = (nrhs + (nrhs + 11) / 12 - 1) / ((nrhs + 11) / 12);  // right-hand sides of a tile block
-  if ((per_block >= 4 && vh >= (1L << 18)) || (per_block >= 6 && vh >= (1L << 16))) return per_block >= 8 ? 10 : 9;
-  return vh >= (1L << 17) && (flags & F_AUX) == 0 ? 4 : 0;
+  if (((per_block >= 4 && vh >= (1L << 18)) || (per_block >= 6 && vh >= (1L << 16))) &&
+      hop_has_variant(prec, flags, red, 9))
+    return per_block >= 8 ? 10 : 9;
+  return vh >= (1L << 17) && (flags & F_AUX) == 0 && hop_has_variant(prec, flags, red, 4) ? 4 : 0;
 }
 
 bool launch_hop_any(int prec, int flags, int red, const HopArgs& a, int block, cudaStream_t st, int* occ,
                     int variant) {
-  if (!hop_has_variants(flags, red)) variant = 0;
   for (;;) {
     bool ok = false;
     switch (prec) {

@@ -125,16 +125,8 @@ static std::vector<Candidate> candidates(long vh, int nrhs, const std::vector<in
 
 static std::vector<int> hop_variants(int prec, int flags, int red, int nrhs) {
   std::vector<int> v = {0};
-  if (!hop_has_variants(flags, red) || prec == P_F64) return v;
-  for (int k = 1; k < 6; ++k) v.push_back(k);
-  const bool residual = (flags & F_SELF_CLOV) != 0;
-  if (!residual) {
-    for (int k = 6; k < 9; ++k)
-      if (hop_variant_rpt(k) <= nrhs) v.push_back(k);
-    if (nrhs >= 2)
-      for (int k = 9; k < HOP_NVARIANT; ++k)
-        if (hop_variant_for_prec(k, prec)) v.push_back(k);
-  }
+  for (int k = 1; k < HOP_NVARIANT; ++k)
+    if (hop_has_variant(prec, flags, red, k) && (k < 6 || (k < 9 ? hop_variant_rpt(k) <= nrhs : nrhs >= 2))) v.push_back(k);
   return v;
 }
 
