@@ -10,7 +10,7 @@
 // What bounds it is latency on the FP64 pipe (2 lanes a clock): a launch with
 // three dot products took 7.6 us where the same launch without took 2.4, 27 us
 // with twelve right-hand sides.  Hence the merged warp sums, one value a lane
-// over the partials, a warp for each right-hand side, one division a quotient,
+// over the partials, a warp for each right-hand side,
 // and nothing at all once every solve has ended.  Solves against the previous
 // tree: 8^4 4.94 -> 3.51 ms, 32^3 x 64 173 -> 167 ms, Moebius 16^3 x 32 x 16
 // 202 -> 198 ms, multigrid on 16^3 x 32 30.1 -> 26.6 ms.
@@ -47,11 +47,11 @@ struct zc {
   double r, i;
 };
 __device__ __forceinline__ zc zmul(zc a, zc b) { return {a.r * b.r - a.i * b.i, a.r * b.i + a.i * b.r}; }
-// One division: FP64 divides are the longest links of the finalizers' serial
-// chain (a few hundred clocks each on this GPU's FP64 pipe).
+// Two divisions, not one reciprocal: |b|^2 goes down to where 1 / |b|^2 is
+// infinite and the quotients are not (|b|^2 < 5.6e-309).
 __device__ __forceinline__ zc zdiv(zc a, zc b) {
-  const double d = 1.0 / (b.r * b.r + b.i * b.i);
-  return {(a.r * b.r + a.i * b.i) * d, (a.i * b.r - a.r * b.i) * d};
+  const double d = b.r * b.r + b.i * b.i;
+  return {(a.r * b.r + a.i * b.i) / d, (a.i * b.r - a.r * b.i) / d};
 }
 __device__ __forceinline__ double zabs2(zc a) { return a.r * a.r + a.i * a.i; }
 
@@ -92,9 +92,8 @@ __device__ inline void finalize(const RedArgs& ra, int rhs, const double s[4]) {
     case FIN_OMEGA: {  // s = <t, s>, |t|^2
       if (q->done) break;
       if (s[2] > 0.0) {
-        const double d = 1.0 / s[2];
-        q->omega_r = s[0] * d;
-        q->omega_i = s[1] * d;
+        q->omega_r = s[0] / s[2];
+        q->omega_i = s[1] / s[2];
       } else {
         q->omega_r = q->omega_i = 0.0;
       }
