@@ -472,10 +472,8 @@ __global__ void __launch_bounds__(32 * TILE_MAX_RHS, 2) hop_kernel_tile(const Ho
     for (int k = 0; k < NV; ++k) rv[k] = ps[k].value();
     const double t = warp_sum<NV>(rv);
     constexpr int LW = warp_sum_lanes<NV>();
-    if (lane % LW == 0 && lane / LW < NV && rhs < a.nrhs && w < G) {
+    if (lane % LW == 0 && lane / LW < NV && rhs < a.nrhs && w < G)
       a.red.partials[((long)rhs * a.nblk + sb) * 4 + lane / LW] = t;
-      __threadfence();
-    }
     __syncthreads();
     grid_finish<NV>(a.red, a.nblk, a.nrhs);
   }

@@ -223,18 +223,14 @@ __device__ __forceinline__ void block_sum(double v[NV], double (*sh)[4]) {
     for (int k = 0; k < NV; ++k) v[k] = __shfl_sync(0xffffffffu, t, k);
 }
 
-// Block partial of one right-hand side -> its slot in ra.partials, visible to
-// the device before thread 0 goes on.  Must be reached by every thread of the
-// block.
+// Block partial of one right-hand side -> its slot in ra.partials, written
+// before thread 0 goes on.  Must be reached by every thread of the block.
 template <int NV>
 __device__ __forceinline__ void block_partial(const RedArgs& ra, int rhs, int sb, int nblk, const double v[NV]) {
   __shared__ double sh[32][4];
   const double t = block_sum_spread<NV>(v, sh);
   if (threadIdx.x < 32) {
-    if (threadIdx.x < NV) {
-      ra.partials[((long)rhs * nblk + sb) * 4 + threadIdx.x] = t;
-      __threadfence();
-    }
+    if (threadIdx.x < NV) ra.partials[((long)rhs * nblk + sb) * 4 + threadIdx.x] = t;
     __syncwarp();
   }
 }
@@ -261,16 +257,20 @@ __device__ __forceinline__ double partials_sum(const double* p, int nblk, int l,
   return a;
 }
 
-// After this block's partials are visible (block_partial, or a fence by their
-// writers and a barrier): take a ticket; the last block of the grid sums every right-hand side's partials in
-// a fixed order and runs the finalizer -- the whole block for one right-hand
-// side with many partials, else a warp for each right-hand side.  Must be
-// reached by every thread of every block.
+// After this block's partials are written (block_partial, or its writers and a
+// barrier): thread 0 takes a ticket behind a fence, which covers what the
+// barrier ordered before it; the last block of the grid sums every right-hand
+// side's partials in a fixed order and runs the finalizer -- the whole block
+// for one right-hand side with many partials, else a warp for each right-hand
+// side.  Must be reached by every thread of every block.
 template <int NV>
 __device__ void grid_finish(const RedArgs& ra, int nblk, int nrhs) {
   __shared__ double sh[32][4];
   __shared__ int is_last;
-  if (threadIdx.x == 0) is_last = (atomicAdd(ra.counter, 1u) == gridDim.x - 1);
+  if (threadIdx.x == 0) {
+    __threadfence();
+    is_last = (atomicAdd(ra.counter, 1u) == gridDim.x - 1);
+  }
   __syncthreads();
   if (!is_last) return;
   __threadfence();
