@@ -67,8 +67,11 @@ enum bridge_status {
 };
 
 /* Storage precision of a field or of an operator application.  F64 computes
- * to FP64 accuracy (Wilson, clover and staggered hopping terms in 64-bit fixed
- * point where links and clover blocks are in its range, else in FP64); F32
+ * to FP64 accuracy: Wilson, clover and staggered hopping terms in 64-bit fixed
+ * point at the sites where every component is of the size of the neighbours it
+ * is summed from (to 2^-5; its error is then below 2^-49 of its terms
+ * typically, 2^-44 at most), in FP64 at the others and where links or clover
+ * blocks are out of the fixed-point range; F32
  * stores and computes in FP32; F16/BF16 store spinors as 16-bit values times a
  * per-site FP32 scale (max |component|), links and clover blocks as plain
  * 16-bit values, and compute in FP32. */

@@ -71,6 +71,7 @@ struct HopArgs {
   const char* clovE_fx;
   const char* clovM_fx;
   int eE_fx, eM_fx;  // their exponents: entries below 2^e
+  int eb_fx;         // 2^eb_fx <= |beta| (binary exponent; far below any field's for beta = 0)
   const char* in_fx;  // `in` in fixed point
   long in_fx_rs;
 };

@@ -19,10 +19,22 @@
 //   * the sum (63 bits) is converted to FP64 once, and the vector part of the
 //     epilogue (beta, self, aux, reductions) is FP64.
 //
-// Against FP64 arithmetic: each hop is rounded once at 2^-56 of the largest
-// neighbour component, where FP64 rounds every FMA at 2^-54 of its running
-// sum: relative error against the exact operator on Gaussian fields 0.97e-16
-// (FP64 kernel 1.1e-16) for Wilson, 1.8e-16 (1.9e-16) for clover.
+// Accuracy.  With w = 2^-54 times 2^E (E the largest exponent among the site's
+// neighbours), a hop's result is off by 0.35 w typically and 2.5 w at most:
+// the rounding 0.5, the products al bl left out 6/4, the inputs' truncation
+// 0.3, the links' 0.2; a component of the sum of eight by w and 20 w.  That is
+// relative to the largest neighbour component, where FP64 arithmetic is
+// relative to what the component itself is summed from.  Where the two differ
+// (components that do not mix: unit or block-diagonal links, spins and colours
+// of very different size), the site is computed in FP64: every real component
+// of the sum has to be reached, by at least one of its eight hops, with 2^-5 of
+// 2^E (fx_reaches), and the site term's operand must not exceed the neighbours
+// by more than 2^6 |beta|.  A component that stays in fixed point is thus off
+// by 2^-49 of its own terms typically, the bound of FP64 arithmetic with its
+// seventeen roundings in a row.  On Gaussian fields practically no site goes to
+// FP64, on the solution of a point source about two in a thousand.  Relative error
+// against the exact operator on Gaussian fields 0.97e-16 (FP64 kernel 1.1e-16)
+// for Wilson, 1.8e-16 (1.9e-16) for clover.
 //
 // Measured (full clover D, one parity of 24^3 x 48, one right-hand side): FP64
 // kernel 780 us = 0.81 TFLOP/s, its pipe's limit; here 242 us = 3.2 TB/s plus
@@ -31,9 +43,9 @@
 // 0.5 of the issue slots, sixteen warps an SM waiting on loads and on the
 // fixed latency of the integer chains; DRAM at 0.4 of its rate.
 //
-// Sites where this does not apply -- a neighbour component that is not
-// finite, or within 2^128 of the ends of the FP64 range -- are computed by
-// the FP64 code (fx_site_fp64), so infinities and NaN propagate as there.
+// Other sites where fixed point does not apply -- a neighbour component that
+// is not finite, or within 2^128 of the ends of the FP64 range -- are computed
+// by the FP64 code (fx_site_fp64) too, so infinities and NaN propagate as there.
 // Links with an entry above 1 and clover blocks with one of 4 or more have no
 // fixed-point copy, and their lattice keeps the FP64 kernel.
 #pragma once
@@ -46,6 +58,8 @@ constexpr int FX_EMIN = 128, FX_EMAX = 1900;  // biased exponents a spinor may h
 constexpr int FX_THREADS = 128;               // block of the stencil: two lanes a site
 constexpr int FX_SITES = FX_THREADS / 2;
 constexpr uint32_t FX_LINK_TOP = 0x3ff00001u;  // links: at most 1 (+ rounding), unit 2^-60
+constexpr int FX_NO_HOP = -2;                  // "exponent" of a hop with phase 0
+constexpr int FX_SELF = 6;                     // T x: |x| below 2^FX_SELF |beta| times the largest neighbour
 constexpr int FX_CLOV_EMAX = 2;                // clover entries: below 2^e, unit 2^(e - 60), e = 1 or 2
 BR_HD uint32_t fx_clov_top(int e) { return (uint32_t)(1023 + e) << 20; }  // high word of 2^e
 
@@ -109,10 +123,21 @@ BR_D long long fx_shift_round(long long x, int d) {  // x / 2^d to nearest, d in
 }
 
 // The slots of one site: neighbour index (bit 31: its hop wraps with phase -1)
-// and exponent, in the order of the directions 2 mu + backward.
+// and exponent (or FX_NO_HOP), in the order of the directions 2 mu + backward.
 struct FxSlots {
   uint2 w[8][FX_SITES];
 };
+
+// Bit 0 and bit 3: whether the real and the imaginary part of a hop's result u
+// (unit 2^(Ea - 1077)) reach 2^-FX_KEEP times 2^(Ea - 1023).  FX_KEEP: at 4 the
+// solution of a point source (24^3 x 48, kappa 0.125) has a site in twenty with
+// a component below, in every second warp; at 5 one in 600, at 6 one in 3000.
+constexpr int FX_KEEP = 5;
+BR_D uint32_t fx_reaches(cx<long long> u) {
+  const int r = (int)(u.r >> 32), i = (int)(u.i >> 32);
+  constexpr int least = 1 << (54 - FX_KEEP - 32);
+  return ((r ^ (r >> 31)) >= least ? 1u : 0u) | ((i ^ (i >> 31)) >= least ? 8u : 0u);
+}
 
 template <int MU>
 BR_D void fx_neighbours(const HopArgs& a, const int* ex, uint32_t ih, const int c[4], uint32_t xh, FxSlots& sh, int site,
@@ -123,8 +148,8 @@ BR_D void fx_neighbours(const HopArgs& a, const int* ex, uint32_t ih, const int 
   const float bc = a.bcf[MU];
   int ef = __ldg(ex + f), eb = __ldg(ex + b);
   bad |= (ef < 0) | (eb < 0);
-  if (wf && bc == 0.f) ef = 0;  // no hop here
-  if (wb && bc == 0.f) eb = 0;
+  if (wf && bc == 0.f) ef = FX_NO_HOP;
+  if (wb && bc == 0.f) eb = FX_NO_HOP;
   Ea = max(Ea, max(ef, eb));
   sh.w[2 * MU][site] = make_uint2(f | ((wf && bc < 0.f) ? 0x80000000u : 0u), (uint32_t)ef);
   sh.w[2 * MU + 1][site] = make_uint2(b | ((wb && bc < 0.f) ? 0x80000000u : 0u), (uint32_t)eb);
@@ -149,13 +174,15 @@ BR_D cx<long long> fx_shfl(cx<long long> v) {
 //   h = p_k + s Q p_partner,  u = U h,  spin k += u,  partner += s conj(Q) u
 // (s = +1 for a forward hop, flipped for a backward one, for k = 1 with mu =
 // 1, 2 and for mu = 3).  up: spin k; low[0], low[1]: what goes to the partner
-// of mu = 0, 1 and of mu = 2, 3.  Units 2^(Ea - 1077).
+// of mu = 0, 1 and of mu = 2, 3.  Units 2^(Ea - 1077).  Returned: bits 0-5,
+// 12-17, 6-11: the components of up, low[0], low[1] that some hop reaches
+// (real parts, then imaginary parts; fx_reaches).
 //
 // A loop over the directions around one body, the loads of the next colour
 // issued while one is multiplied: unrolled over the directions the code
 // (115 KB) ran out of the instruction cache, and without the early loads the
 // kernel took 1.25 times as long.
-BR_D void fx_hops(const HopArgs& a, const char* in, const char* g_out, const char* g_in, long lbb, uint32_t ih, int Ea,
+BR_D uint32_t fx_hops(const HopArgs& a, const char* in, const char* g_out, const char* g_in, long lbb, uint32_t ih, int Ea,
                   const FxSlots& sh, int site, int k, cx<long long> up[3], cx<long long> low[2][3]) {
   const long vs = 16 * a.g.vh;  // bytes of a plane
   const char* pk = in + 3 * k * vs;
@@ -175,15 +202,18 @@ BR_D void fx_hops(const HopArgs& a, const char* in, const char* g_out, const cha
   };
 #pragma unroll
   for (int c = 0; c < 3; ++c) up[c] = low[0][c] = low[1][c] = {0, 0};
+  uint32_t reach = 0;
   load(b[0], 0, 0);
 #pragma unroll 1
   for (int dir = 0; dir < 8; ++dir) {
-    if (dir == 4)
+    if (dir == 4) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         low[0][c] = low[1][c];
         low[1][c] = {0, 0};
       }
+      reach = (reach & 0x3fu) | ((reach & 0xfc0u) << 6);
+    }
     const uint2 w = sh.w[dir][site];
     const int mu = dir >> 1;
     const bool fwd = (dir & 1) == 0, rot = (mu & 1) == 0;
@@ -213,14 +243,18 @@ BR_D void fx_hops(const HopArgs& a, const char* in, const char* g_out, const cha
     const int d = min(Ea - (int)w.y, 62);  // 62 where there is no contribution: rounds to zero
     const long long half = (1ll << d) >> 1;
     const bool flip = __any_sync(0xffffffffu, w.x >> 31);
+    uint32_t hit = 0;
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
       cx<long long> u = {(rh[r] + fx_split(rm[r]).h + half) >> d, (jh[r] + fx_split(jm[r]).h + half) >> d};
+      hit |= fx_reaches(u) << r;
       if (flip && (w.x >> 31)) u = {-u.r, -u.i};
       up[r] = up[r] + u;
       low[1][r] = low[1][r] + cx<long long>{fx_sign(rot ? u.i : u.r, m), fx_sign(rot ? u.r : u.i, mr)};
     }
+    reach |= hit | ((rot ? (hit >> 3) | ((hit & 7u) << 3) : hit) << 6);
   }
+  return reach;
 }
 
 // y = A x for one packed Hermitian 6x6 block in fixed point (entries below
@@ -272,18 +306,131 @@ BR_D void fx_hermitian6(const char* base, long vh, uint32_t i, int b, const cx<l
 // 2^(e - 1023) for a biased exponent e in 1 .. 2046.
 BR_D double fx_pow2(int e) { return __hiloint2double(e << 20, 0); }
 
-// The site in FP64 (not inlined: it runs only where a spinor has no
-// fixed-point form, and must not cost the other sites registers): spins 2 k,
-// 2 k + 1 of the output.
-template <int FL>
-__device__ __noinline__ void fx_site_fp64(const HopArgs& a, int rhs, uint32_t ih, int k, double2* out) {
-  int c[4];
-  uint32_t xh;
-  site_coords(a.g, ih, a.out_parity, c, xh);
-  cx<double> v[12], s[12];
-  hop_site<P_F64, FL, true>(a, rhs, ih, c, xh, v, s);
+// One hop in FP64 for the projected spin component k of this lane (signs and
+// partner spins as in fx_hops): up gets U h, low what goes to the partner.
+template <int MU, bool FWD>
+BR_D void fx_hop_fp64(const char* in, const char* lb, long vh, uint2 slot, uint32_t ih, int k, cx<double> up[3],
+                      cx<double> low[3]) {
+  constexpr bool rot = MU == 0 || MU == 2;
+  const bool neg = !FWD ^ (k && (MU == 1 || MU == 2)) ^ (MU == 3);
+  const uint32_t nb = slot.x & 0x7fffffffu;
+  const double phase = (int)slot.y == FX_NO_HOP ? 0.0 : (slot.x >> 31) ? -1.0 : 1.0;
+  const double2* pk = reinterpret_cast<const double2*>(in) + 3 * k * vh + nb;
+  const double2* px = reinterpret_cast<const double2*>(in) + (MU < 2 ? 3 * (3 - k) : 3 * (2 + k)) * vh + nb;
+  cx<double> h[3];
 #pragma unroll
-  for (int j = 0; j < 6; ++j) out[j] = k ? make_double2(v[6 + j].r, v[6 + j].i) : make_double2(v[j].r, v[j].i);
+  for (int c = 0; c < 3; ++c) {
+    const double2 p = __ldg(pk + c * vh), q = __ldg(px + c * vh);
+    const cx<double> x = rot ? cx<double>{-q.y, q.x} : cx<double>{q.x, q.y};
+    h[c] = neg ? cx<double>{p.x, p.y} - x : cx<double>{p.x, p.y} + x;
+    if (phase != 1.0) h[c] = phase * h[c];
+  }
+  Link<double> U;
+  load_link<P_F64, true>(lb, vh, FWD ? ih : nb, U);
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    const cx<double> u = FWD ? crow3(U.m[r][0], U.m[r][1], U.m[r][2], h) : crow3_conj(U.m[0][r], U.m[1][r], U.m[2][r], h);
+    const cx<double> w = rot ? times_mi(u) : u;
+    up[r] = up[r] + u;
+    low[r] = neg ? low[r] - w : low[r] + w;
+  }
+}
+template <int MU>
+BR_D void fx_dir_fp64(const HopArgs& a, const char* in, const char* g_out, const char* g_in, long lbb, uint32_t ih,
+                      const FxSlots& sh, int site, int k, cx<double> up[3], cx<double> low[3]) {
+  fx_hop_fp64<MU, true>(in, g_out + MU * lbb, a.g.vh, sh.w[2 * MU][site], ih, k, up, low);
+  fx_hop_fp64<MU, false>(in, g_in + MU * lbb, a.g.vh, sh.w[2 * MU + 1][site], ih, k, up, low);
+}
+
+// y = A x for one packed Hermitian 6x6 block in FP64, entry by entry.
+BR_D void fx_hermitian6_fp64(const char* base, long vh, uint32_t i, int b, const cx<double> x[6], cx<double> y[6]) {
+  const double2* p = reinterpret_cast<const double2*>(base) + 18 * b * vh + i;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const double2 d = ldg4<true>(p + k * vh);
+    y[2 * k] = d.x * x[2 * k];
+    y[2 * k + 1] = d.y * x[2 * k + 1];
+  }
+  int k = 3;
+#pragma unroll
+  for (int r = 1; r < 6; ++r)
+#pragma unroll
+    for (int c = 0; c < r; ++c) {
+      const double2 w = ldg4<true>(p + k * vh);
+      ++k;
+      y[r] = cfma(cx<double>{w.x, w.y}, x[c], y[r]);
+      y[c] = cfma_conj(cx<double>{w.x, w.y}, x[r], y[c]);
+    }
+}
+
+// The site in FP64 by its two lanes (spins 2 k, 2 k + 1 of the output to lane
+// k), the sums in the order of the FP64 kernel; called by whole warps (called
+// in a divergent branch it cost the other sites a tenth in spills).  Not
+// inlined: it runs only where fixed point does not do.  Split over the two
+// lanes it costs the FP64 pipe what the FP64 kernel does: full Wilson D on 24^3 x
+// 48 with every site here 1650 us, on the FP64 kernel 1421, in fixed point 532.
+template <int FL>
+__device__ __noinline__ void fx_site_fp64(const HopArgs& a, int rhs, uint32_t ih, int k, const FxSlots& sh,
+                                          int site, double2* out) {
+  const int p = a.out_parity;
+  const long vh = a.g.vh, lbb = link_block_bytes(P_F64, vh), cbb = clover_block_bytes(P_F64, vh);
+  auto other = [&](cx<double> z) {
+    return cx<double>{__shfl_xor_sync(0xffffffffu, z.r, 1), __shfl_xor_sync(0xffffffffu, z.i, 1)};
+  };
+  cx<double> v[6];
+  {
+    const char* g_out = a.gauge + (long)p * 4 * lbb;
+    const char* g_in = a.gauge + (long)(1 - p) * 4 * lbb;
+    const char* in = a.in + rhs * a.in_rs;
+    cx<double> up[3], low[3];  // spin k; the partner's sum: spin 3 - k for mu = 0, 1, then spin 2 + k
+#pragma unroll
+    for (int r = 0; r < 3; ++r) up[r] = low[r] = czero<double>();
+    fx_dir_fp64<0>(a, in, g_out, g_in, lbb, ih, sh, site, k, up, low);
+    fx_dir_fp64<1>(a, in, g_out, g_in, lbb, ih, sh, site, k, up, low);
+    // each sum goes on where the next directions add to it
+#pragma unroll
+    for (int r = 0; r < 3; ++r) low[r] = other(low[r]);
+    fx_dir_fp64<2>(a, in, g_out, g_in, lbb, ih, sh, site, k, up, low);
+    fx_dir_fp64<3>(a, in, g_out, g_in, lbb, ih, sh, site, k, up, low);
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const cx<double> x = other(k ? up[r] : low[r]);  // spin 1 to lane 0, spin 2 to lane 1
+      v[r] = a.beta * (k ? x : up[r]);
+      v[3 + r] = a.beta * (k ? low[r] : x);
+    }
+  }
+  auto plane = [&](const char* f, int j) {
+    const double2 w = ldg4<true>(reinterpret_cast<const double2*>(f) + (6 * k + j) * vh + ih);
+    return cx<double>{w.x, w.y};
+  };
+  if (FL & F_AUX)
+#pragma unroll
+    for (int j = 0; j < 6; ++j) v[j] = v[j] + a.caux * plane(a.aux + rhs * a.aux_rs, j);
+  if ((FL & F_G5) && k)
+#pragma unroll
+    for (int j = 0; j < 6; ++j) v[j] = {-v[j].r, -v[j].i};
+  if (FL & F_E_CLOV) {
+    cx<double> y[6];
+    fx_hermitian6_fp64(a.clovE + p * cbb, vh, ih, k, v, y);
+#pragma unroll
+    for (int j = 0; j < 6; ++j) v[j] = y[j];
+  }
+  if (FL & F_SELF) {
+    const char* self = a.self + rhs * a.self_rs;
+    if (FL & F_SELF_CLOV) {
+      cx<double> x[6], y[6];
+#pragma unroll
+      for (int j = 0; j < 6; ++j) x[j] = plane(self, j);
+      fx_hermitian6_fp64(a.clovM + p * cbb, vh, ih, k, x, y);
+#pragma unroll
+      for (int j = 0; j < 6; ++j) v[j] = v[j] + a.s1 * y[j];
+    } else {
+#pragma unroll
+      for (int j = 0; j < 6; ++j) v[j] = v[j] + a.s1 * plane(self, j);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 6; ++j) out[j] = make_double2(v[j].r, v[j].i);
 }
 
 // Two adjacent lanes share an output site: lane k forms the projected spin
@@ -333,7 +480,10 @@ __global__ void __launch_bounds__(FX_THREADS, 4) hop_kernel_fx(const HopArgs a) 
       cx<long long> q[6];
       {
         cx<long long> up[3], low[2][3];
-        fx_hops(a, in, g_out, g_in, lbb, ih, Ea, sh, site, k, up, low);
+        const uint32_t mine = fx_hops(a, in, g_out, g_in, lbb, ih, Ea, sh, site, k, up, low);
+        // spin 0 or 1 from this lane's hops; spin 2 (lane 0) or 3 (lane 1) from both lanes'
+        const uint32_t theirs = __shfl_xor_sync(0xffffffffu, mine, 1);
+        if (Ea != 0 && ((mine & 0x3fu) != 0x3fu || (((mine >> 6) | (theirs >> 12)) & 0x3fu) != 0x3fu)) bad = 1;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           const cx<long long> x = fx_shfl(k ? up[c] : low[1][c]);  // spin 1 to lane 0, spin 2's share to lane 1
@@ -342,7 +492,6 @@ __global__ void __launch_bounds__(FX_THREADS, 4) hop_kernel_fx(const HopArgs a) 
           q[3 + c] = k ? y + low[1][c] : x;
         }
       }
-      __syncwarp();
       // scale of the sum: beta times its unit (0 for an empty sum)
       int e = Ea - 54;
       if (FL & F_E_CLOV) {
@@ -394,7 +543,8 @@ __global__ void __launch_bounds__(FX_THREADS, 4) hop_kernel_fx(const HopArgs a) 
         for (int j = 0; j < 6; ++j) w[j] = ldg4<true>(reinterpret_cast<const uint4*>(self) + j * vh);
         const uint32_t m = fx_max_word<6>(w);
         const int Es = (int)(m >> 20);
-        if (m != 0 && (Es < FX_EMIN || Es > FX_EMAX)) bad = 1;
+        // the hops must reach the size of what T x is rounded against
+        if (m != 0 && (Es < FX_EMIN || Es > FX_EMAX || Ea == 0 || Es > Ea + a.eb_fx + FX_SELF)) bad = 1;
         if (m != 0 && !bad) {
           cx<long long> y[6];
 #pragma unroll
@@ -408,12 +558,14 @@ __global__ void __launch_bounds__(FX_THREADS, 4) hop_kernel_fx(const HopArgs a) 
         }
       }
       bad |= __shfl_xor_sync(0xffffffffu, bad, 1);
-      if (bad) {
+      if (__any_sync(0xffffffffu, bad)) {
         double2 w[6];
-        fx_site_fp64<FL>(a, rhs, ih, k, w);
+        fx_site_fp64<FL>(a, rhs, ih, k, sh, site, w);
+        if (bad)
 #pragma unroll
-        for (int j = 0; j < 6; ++j) v[j] = {w[j].x, w[j].y};
+          for (int j = 0; j < 6; ++j) v[j] = {w[j].x, w[j].y};
       }
+      __syncwarp();  // the slots have been read
       if (live) {
         double2* out = reinterpret_cast<double2*>(a.out + rhs * a.out_rs) + o;
 #pragma unroll

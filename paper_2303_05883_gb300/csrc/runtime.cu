@@ -1,6 +1,7 @@
 // Host runtime: device buffers, fields, gauge and clover storage, operator
 // application, launch statistics and launch shapes.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <string>
 
@@ -328,6 +329,7 @@ void set_fx_args(bridge_lattice_s* L, HopArgs& a, int flags, int red, CloverSet*
     a.in_fx = scratch;
     a.in_fx_rs = c.dst_rs;
   }
+  a.eb_fx = a.beta != 0.0 && std::isfinite(a.beta) ? std::ilogb(a.beta) : -5000;
   a.gauge_fx = U;
   a.clovE_fx = E;
   a.clovM_fx = M;

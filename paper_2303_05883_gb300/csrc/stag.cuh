@@ -205,7 +205,8 @@ __global__ void __launch_bounds__(256) stag_hop_kernel(const StagArgs a) {
 // ------------------------------------------------------------ fixed point
 // The FP64 hop in 64-bit fixed point, as dslash_fx.cuh: the same integer links,
 // the colour vectors in units of 2^(E - 1081) with one exponent a site (three
-// 16-byte planes, then one int a site), one rounding a hop.  36 products of
+// 16-byte planes, then one int a site), one rounding a hop, and the same test
+// that every component is reached by a hop.  36 products of
 // three IMAD.WIDE a hop; a site has nothing to project or reconstruct, so one
 // thread a site keeps its sum, a hop's rows and both hops' loads of a direction
 // in 128 registers.  Measured (one parity of 32^4): FP64 kernel 340 us, at the
@@ -256,8 +257,9 @@ BR_D void stag_fx_load(StagFxLoads& f, const char* in, const char* g, long vs, u
   for (int k = 0; k < 9; ++k) f.l[k] = ldg4<true>(reinterpret_cast<const uint4*>(g + k * vs) + li);
 }
 
+// The hop's result is added to acc; returned: the components it reaches (fx_reaches).
 template <bool FWD>
-BR_D void stag_fx_mac(const StagFxLoads& f, uint2 w, int Ea, cx<long long> acc[3]) {
+BR_D uint32_t stag_fx_mac(const StagFxLoads& f, uint2 w, int Ea, cx<long long> acc[3]) {
   long long rh[3] = {0, 0, 0}, rm[3] = {0, 0, 0}, jh[3] = {0, 0, 0}, jm[3] = {0, 0, 0};
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
@@ -276,11 +278,15 @@ BR_D void stag_fx_mac(const StagFxLoads& f, uint2 w, int Ea, cx<long long> acc[3
   const int d = min(Ea - (int)w.y, 62);  // a zero neighbour (exponent 0): rounds to zero
   const long long half = (1ll << d) >> 1;
   const int m = -(int)(w.x >> 31);
+  uint32_t hit = 0;
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
-    acc[r].r += fx_sign((rh[r] + fx_split(rm[r]).h + half) >> d, m);
-    acc[r].i += fx_sign((jh[r] + fx_split(jm[r]).h + half) >> d, m);
+    const cx<long long> u = {(rh[r] + fx_split(rm[r]).h + half) >> d, (jh[r] + fx_split(jm[r]).h + half) >> d};
+    hit |= fx_reaches(u) << r;
+    acc[r].r += fx_sign(u.r, m);
+    acc[r].i += fx_sign(u.i, m);
   }
+  return hit;
 }
 
 // The site in FP64, where a neighbour has no fixed-point form.
@@ -323,13 +329,9 @@ __global__ void __launch_bounds__(SFX_THREADS, 4) stag_hop_fx_kernel(const StagA
       }
       cx<double> v[3], s[3];
       if (a.self != nullptr) load_cvec<P_F64>(a.self + rhs * a.self_rs, vh, ih, s);
-      if (bad) {
-        double2 w[3];
-        stag_fx_site_fp64(a, rhs, ih, w);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) v[k] = {w[k].x, w[k].y};
-      } else {
-        cx<long long> acc[3] = {{0, 0}, {0, 0}, {0, 0}};
+      cx<long long> acc[3] = {{0, 0}, {0, 0}, {0, 0}};
+      if (!bad) {
+        uint32_t reach = 0;
 #pragma unroll 1
         for (int mu = 0; mu < 4; ++mu) {
           StagFxLoads f, b;
@@ -337,9 +339,17 @@ __global__ void __launch_bounds__(SFX_THREADS, 4) stag_hop_fx_kernel(const StagA
           const uint32_t nf = wf.x & 0x7fffffffu, nb = wb.x & 0x7fffffffu;
           stag_fx_load(f, in, g_out + mu * lbb, vs, nf, ih);
           stag_fx_load(b, in, g_in + mu * lbb, vs, nb, nb);
-          stag_fx_mac<true>(f, wf, Ea, acc);
-          stag_fx_mac<false>(b, wb, Ea, acc);
+          reach |= stag_fx_mac<true>(f, wf, Ea, acc);
+          reach |= stag_fx_mac<false>(b, wb, Ea, acc);
         }
+        bad = Ea != 0 && reach != 0x3fu;
+      }
+      if (bad) {
+        double2 w[3];
+        stag_fx_site_fp64(a, rhs, ih, w);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) v[k] = {w[k].x, w[k].y};
+      } else {
         const double sc = Ea == 0 ? 0.0 : a.scale * fx_pow2(Ea - 54);
         cx<double> t[3];
 #pragma unroll
