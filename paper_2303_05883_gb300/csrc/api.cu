@@ -97,8 +97,8 @@ static void mult_dev(bridge_lattice_s* L, const bridge_op& op, int prec, int whi
     const bool full = which == BRIDGE_APPLY_D;
     const int subset = full ? BRIDGE_FULL : which == BRIDGE_APPLY_DEO ? 1 - out_parity : BRIDGE_EVEN;
     Field fi = stag_workspace(L, "mult_in", prec, subset, nrhs);
-    if (prec == BRIDGE_F64) fi.fx = stag_fx_input(L, nrhs * (full ? 2 : 1));
     Field& fo = stag_workspace(L, "mult_out", prec, which == BRIDGE_APPLY_DEO ? out_parity : subset, nrhs);
+    if (prec == BRIDGE_F64) fi.fx = stag_fx_input(L, nrhs * (full ? 2 : 1));  // (last: it only makes things faster)
     stag_canon_to_field(L, in, fi, full, st);
     if (full)
       stag_apply_d(L, op, fo, fi, st);
@@ -137,16 +137,18 @@ static void mult_dev(bridge_lattice_s* L, const bridge_op& op, int prec, int whi
   BR_CHECK(which != APPLY_DHAT_DAG, BRIDGE_EINVAL, "bridge_mult_Dhat_dag is provided for MOBIUS operators only");
   const int subset = which == BRIDGE_APPLY_D ? BRIDGE_FULL : which == BRIDGE_APPLY_DEO ? 1 - out_parity : BRIDGE_EVEN;
   Field fi = workspace(L, "mult_in", prec, subset, nrhs);
+  Field& fo = workspace(L, "mult_out", prec, which == BRIDGE_APPLY_DEO ? out_parity : subset, nrhs);
+  Field* tmp = which == BRIDGE_APPLY_DHAT ? &workspace(L, "mult_tmp", prec, BRIDGE_ODD, nrhs) : nullptr;
   // FP64: the input's fixed-point form is written with its layout conversion
+  // (last of the buffers: it only makes things faster)
   if (prec == BRIDGE_F64) fi.fx = fx_input(L, op, which, nrhs * (subset == BRIDGE_FULL ? 2 : 1));
   canon_to_field(L, in, fi, st);
-  Field& fo = workspace(L, "mult_out", prec, which == BRIDGE_APPLY_DEO ? out_parity : subset, nrhs);
   if (which == BRIDGE_APPLY_D) {
     apply_d(L, op, fo, fi, st);
   } else if (which == BRIDGE_APPLY_DEO) {
     apply_deo(L, op, out_parity, fo, fi, st);
   } else {
-    apply_dhat(L, op, fo, fi, workspace(L, "mult_tmp", prec, BRIDGE_ODD, nrhs), st);
+    apply_dhat(L, op, fo, fi, *tmp, st);
   }
   field_to_canon(L, fo, out, st);
 }
@@ -305,19 +307,20 @@ static int gauge_upload(bridge_lattice L, const double* U, const bridge_op* op, 
   BR_CHECK(L->in_flight.load() == 0, BRIDGE_ESTATE, "requests on this lattice are still running");
   BR_CUDA(cudaStreamSynchronize(L->stream));
   for (int p = 0; p < 4; ++p) L->gauge[p].reset();
-  {
-    std::lock_guard<std::mutex> lk(L->fx_mu);
-    L->gauge_fx = FxCopy{};
-  }
+  L->gauge_fx_made = false;
   {
     std::lock_guard<std::mutex> lk(L->clover_mu);
     L->clovers.clear();
   }
-  L->gauge[P_F64].reset(new DevBuf((size_t)(8 * link_block_bytes(P_F64, L->vh))));
+  const size_t links = (size_t)(8 * link_block_bytes(P_F64, L->vh));
+  L->gauge[P_F64].reset(new DevBuf(links + 256));  // (behind the links: the largest entry met)
+  uint32_t* top = reinterpret_cast<uint32_t*>(L->gauge[P_F64]->ptr + links);
+  BR_CUDA(cudaMemsetAsync(top, 0, sizeof(uint32_t), L->stream));
   note_launch(L, K_SETUP, (double)n * 2, 0, L->stream, true);
-  launch_gauge_from_canon(src, L->g, L->gauge[P_F64]->ptr, L->stream);
+  launch_gauge_from_canon(src, L->g, L->gauge[P_F64]->ptr, top, L->stream);
   note_launch(L, K_SETUP, 0, 0, L->stream, false);
   BR_CUDA(cudaGetLastError());
+  BR_CUDA(cudaMemcpyAsync(&L->gauge_top, top, sizeof(uint32_t), cudaMemcpyDeviceToHost, L->stream));
   L->have_gauge = true;
   if (op && op_is_clover(*op)) {
     clover_ptr(L, P_F64, true, op_kcsw(*op));

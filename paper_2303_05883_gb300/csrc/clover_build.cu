@@ -175,7 +175,8 @@ __device__ void invert6(Z a[6][6], Z inv[6][6]) {
   }
 }
 
-__device__ void pack6(const Z m[6][6], double2* dst, long vh, uint32_t ih, int b) {
+// Returns the largest high word of an |entry|.
+__device__ uint32_t pack6(const Z m[6][6], double2* dst, long vh, uint32_t ih, int b) {
   double v[36];
   for (int r = 0; r < 6; ++r) v[r] = m[r][r].r;
   int k = 0;
@@ -185,10 +186,18 @@ __device__ void pack6(const Z m[6][6], double2* dst, long vh, uint32_t ih, int b
       v[6 + 2 * k + 1] = m[r][c].i;
       ++k;
     }
-  for (int q = 0; q < 18; ++q) dst[(18 * b + q) * vh + ih] = make_double2(v[2 * q], v[2 * q + 1]);
+  uint32_t top = 0;
+  for (int q = 0; q < 18; ++q) {
+    const double2 w = make_double2(v[2 * q], v[2 * q + 1]);
+    dst[(18 * b + q) * vh + ih] = w;
+    top = max(top, high_word(w));
+  }
+  return top;
 }
 
-__global__ void __launch_bounds__(128) k_clover_build(const Geom g, const char* g64, double kcsw, char* T64, char* Tinv64) {
+__global__ void __launch_bounds__(128) k_clover_build(const Geom g, const char* g64, double kcsw, char* T64, char* Tinv64,
+                                                      uint32_t* top) {
+  uint32_t mt = 0, mi = 0;
   const long vh = g.vh;
   const long lbb = link_block_bytes(P_F64, vh), cbb = clover_block_bytes(P_F64, vh);
   for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < 2 * vh; k += (long)gridDim.x * blockDim.x) {
@@ -222,19 +231,22 @@ __global__ void __launch_bounds__(128) k_clover_build(const Geom g, const char* 
           blk[3 + i][j] = czero<double>() - kcsw * (A + iB);
           blk[3 + i][3 + j] = Z{id, 0.0} + kcsw * C;
         }
-      pack6(blk, reinterpret_cast<double2*>(T64 + p * cbb), vh, ih, b);
+      mt = max(mt, pack6(blk, reinterpret_cast<double2*>(T64 + p * cbb), vh, ih, b));
       invert6(blk, inv);
-      pack6(inv, reinterpret_cast<double2*>(Tinv64 + p * cbb), vh, ih, b);
+      mi = max(mi, pack6(inv, reinterpret_cast<double2*>(Tinv64 + p * cbb), vh, ih, b));
     }
   }
+  warp_top(mt, top);
+  warp_top(mi, top + 1);
 }
 
-void launch_clover_build(const Geom& g, const char* g64, double kcsw, char* T64, char* Tinv64, cudaStream_t st) {
+void launch_clover_build(const Geom& g, const char* g64, double kcsw, char* T64, char* Tinv64, uint32_t* top,
+                         cudaStream_t st) {
   const long n = 2L * g.vh;
   const int block = 128;
   long grid = (n + block - 1) / block;
   if (grid > 152 * 32) grid = 152 * 32;
-  k_clover_build<<<(unsigned)grid, block, 0, st>>>(g, g64, kcsw, T64, Tinv64);
+  k_clover_build<<<(unsigned)grid, block, 0, st>>>(g, g64, kcsw, T64, Tinv64, top);
 }
 
 }  // namespace bridge

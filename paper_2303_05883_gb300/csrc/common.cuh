@@ -450,6 +450,16 @@ BR_D void clover_apply(const char* base, long vh, uint32_t i, const cx<typename 
   }
 }
 
+// *top = max(*top, m over the block's threads); every thread of each warp calls.
+BR_D void warp_top(uint32_t m, uint32_t* top) {
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(top, m);
+}
+// High word of the larger magnitude of a pair.
+BR_D uint32_t high_word(double2 v) {
+  return max((uint32_t)__double2hiint(v.x) & 0x7fffffffu, (uint32_t)__double2hiint(v.y) & 0x7fffffffu);
+}
+
 // -------------------------------------------------------------- geometry
 // Division by an invariant 32-bit divisor (Granlund and Montgomery, PLDI
 // 1994, unsigned case): q = (umulhi(n, m) + n) >> l with l = ceil(log2 d)

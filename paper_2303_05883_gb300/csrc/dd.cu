@@ -641,11 +641,13 @@ extern "C" int bridge_dd_create(bridge_lattice L, const bridge_op* op, int npart
     for (int b = 0; b < 8; ++b)
       copy_planes(s.L->gauge[P_F64]->ptr + b * link_block_bytes(P_F64, vhl), vhl,
                   L->gauge[P_F64]->ptr + b * link_block_bytes(P_F64, vh), vh, first, 9, s.L->stream);
+    s.L->gauge_top = L->gauge_top;
     s.L->have_gauge = true;
     if (clov) {
       // the slab's part of T and T^-1 of the whole field: [parity] blocks of 36 double2 planes
       auto cs = std::make_shared<CloverSet>();
       cs->kcsw = op_kcsw(*op);
+      for (int inv = 0; inv < 2; ++inv) cs->top[inv] = gset->top[inv];
       for (int inv = 0; inv < 2; ++inv) {
         std::unique_ptr<DevBuf>& dst = inv ? cs->Tinv[P_F64] : cs->T[P_F64];
         const DevBuf& src = inv ? *gset->Tinv[P_F64] : *gset->T[P_F64];

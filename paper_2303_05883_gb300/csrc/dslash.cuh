@@ -65,8 +65,9 @@ struct HopArgs {
   // blocking); the other sites are neither read nor written.
   const uint32_t* site_map;
   uint32_t n_map;
-  // FP64 only, non-null when the fixed-point kernel may run (dslash_fx.cuh):
-  // the same links and clover blocks as 64-bit fixed-point numbers.
+  // FP64 only (dslash_fx.cuh): an FxMode, and for FX_COPIES the links, clover
+  // blocks and `in` as 64-bit fixed-point numbers.
+  int fx;
   const char* gauge_fx;
   const char* clovE_fx;
   const char* clovM_fx;
@@ -75,6 +76,11 @@ struct HopArgs {
   const char* in_fx;  // `in` in fixed point
   long in_fx_rs;
 };
+
+// How an FP64 hop runs: on the FP64 pipe, in fixed point from copies of its
+// operands, or in fixed point converting the FP64 operands as it reads them
+// (the same integers, so the same result).
+enum FxMode { FX_OFF = 0, FX_COPIES = 1, FX_RAW = 2 };
 
 template <class R, int MU, bool FWD>
 BR_D void project(const cx<R> p[12], cx<R> h[2][3]) {

@@ -29,13 +29,17 @@ bool launch_hop_fx(int flags, int red, const HopArgs& args, int block, cudaStrea
   const long cover = ((long)a.g.vh + FX_SITES - 1) / FX_SITES;
   a.nblk = (int)((long)a.nblk * block >= (long)a.g.vh ? cover : std::min<long>(a.nblk, cover));
   const dim3 grid((unsigned)(a.nblk * a.nrhs));
-#define BRIDGE_FX_LAUNCH(FL, RD)                                                                                  \
-  if (flags == (FL) && red == (RD)) {                                                                             \
-    if (occ)                                                                                                       \
-      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, hop_kernel_fx<(FL), (RD)>, FX_THREADS, 0) ==  \
-             cudaSuccess;                                                                                          \
-    hop_kernel_fx<(FL), (RD)><<<grid, FX_THREADS, 0, st>>>(a);                                           \
-    return true;                                                                                                   \
+#define BRIDGE_FX_LAUNCH(FL, RD)                                                                                   \
+  if (flags == (FL) && red == (RD)) {                                                                               \
+    /* one grid for both kernels: the order of a reduction does not depend on which of them runs */                 \
+    if (occ)                                                                                                        \
+      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, hop_kernel_fx<(FL), (RD), false>, FX_THREADS, 0) == \
+             cudaSuccess;                                                                                           \
+    if (a.fx == FX_RAW)                                                                                             \
+      hop_kernel_fx<(FL), (RD), true><<<grid, FX_THREADS, 0, st>>>(a);                                              \
+    else                                                                                                            \
+      hop_kernel_fx<(FL), (RD), false><<<grid, FX_THREADS, 0, st>>>(a);                                             \
+    return true;                                                                                                    \
   }
   BRIDGE_FX_CASES(BRIDGE_FX_LAUNCH)
 #undef BRIDGE_FX_LAUNCH
@@ -59,32 +63,19 @@ void launch_field_to_fx(const CopyArgs& a, int block, cudaStream_t st) {
 }
 
 // nb blocks of n double2 entries (block_bytes apart; the padding between them
-// is not touched) of magnitude up to 2^e -> two limbs of each real times
-// 2^(60 - e); *top receives the largest high word met.
-__global__ void __launch_bounds__(256) k_to_fx(const char* src, char* dst, int nb, long n, long block_bytes, int e,
-                                               uint32_t* top) {
-  uint32_t m = 0;
+// is not touched) of magnitude up to 2^e -> two limbs of each real.
+__global__ void __launch_bounds__(256) k_to_fx(const char* src, char* dst, int nb, long n, long block_bytes, int e) {
   for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < nb * n; k += (long)gridDim.x * blockDim.x) {
     const long off = (k / n) * block_bytes + (k % n) * 16;
     const uint4 w = *reinterpret_cast<const uint4*>(src + off);
-    m = max(m, max(w.y & 0x7fffffffu, w.w & 0x7fffffffu));
-    // 2^e, exponent 1023 + e, becomes the integer 2^60; larger entries are refused by the caller
-    const int E = 1023 + e;
-    Fx2 r = fx_split(fx_from_bits<8>(w.x, w.y, max(E, (int)((w.y >> 20) & 0x7ffu)), 0));
-    Fx2 i = fx_split(fx_from_bits<8>(w.z, w.w, max(E, (int)((w.w >> 20) & 0x7ffu)), 0));
-    // the stencil negates limbs: keep the low one off -2^31 (by one unit, 2^(e - 60))
-    r.l = max(r.l, -0x7fffffff);
-    i.l = max(i.l, -0x7fffffff);
+    const Fx2 r = fx_limbs_of(w.x, w.y, 1023 + e), i = fx_limbs_of(w.z, w.w, 1023 + e);
     *reinterpret_cast<uint4*>(dst + off) = make_uint4((uint32_t)r.l, (uint32_t)r.h, (uint32_t)i.l, (uint32_t)i.h);
   }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
-  if ((threadIdx.x & 31) == 0) atomicMax(top, m);
 }
 
-void launch_to_fx(const char* src, char* dst, int nb, long n, long block_bytes, int e, uint32_t* top, cudaStream_t st) {
+void launch_to_fx(const char* src, char* dst, int nb, long n, long block_bytes, int e, cudaStream_t st) {
   const long grid = std::min<long>((nb * n + 255) / 256, 152L * 64);
-  k_to_fx<<<(unsigned)grid, 256, 0, st>>>(src, dst, nb, n, block_bytes, e, top);
+  k_to_fx<<<(unsigned)grid, 256, 0, st>>>(src, dst, nb, n, block_bytes, e);
 }
 
 }  // namespace bridge

@@ -47,7 +47,10 @@
 // is not finite, or within 2^128 of the ends of the FP64 range -- are computed
 // by the FP64 code (fx_site_fp64) too, so infinities and NaN propagate as there.
 // Links with an entry above 1 and clover blocks with one of 4 or more have no
-// fixed-point copy, and their lattice keeps the FP64 kernel.
+// fixed-point form, and their lattice keeps the FP64 kernel: which arithmetic
+// runs is a matter of the operator's entries alone.  The copies are a matter of
+// memory: where there is none for them the kernel converts as it reads
+// (FX_RAW), to the same integers and the same result.
 #pragma once
 
 #include "dslash.cuh"
@@ -61,7 +64,13 @@ constexpr uint32_t FX_LINK_TOP = 0x3ff00001u;  // links: at most 1 (+ rounding),
 constexpr int FX_NO_HOP = -2;                  // "exponent" of a hop with phase 0
 constexpr int FX_SELF = 6;                     // T x: |x| below 2^FX_SELF |beta| times the largest neighbour
 constexpr int FX_CLOV_EMAX = 2;                // clover entries: below 2^e, unit 2^(e - 60), e = 1 or 2
-BR_HD uint32_t fx_clov_top(int e) { return (uint32_t)(1023 + e) << 20; }  // high word of 2^e
+// The exponent e of clover blocks whose largest |entry| has the high word top
+// (entries below 2^e); 0: they have no fixed-point form.
+BR_HD int fx_clov_exponent(uint32_t top) {
+  for (int e = 1; e <= FX_CLOV_EMAX; ++e)
+    if (top < ((uint32_t)(1023 + e) << 20)) return e;
+  return 0;
+}
 
 // x as an integer with unit 2^(E - 1075 - SH), E >= the biased exponent of
 // x: |result| < 2^(53 + SH).  Rounds towards zero; neg = -1 changes the sign.
@@ -81,6 +90,21 @@ struct Fx2 {
 };
 BR_D Fx2 fx_split(long long x) { return {(int)(x >> 32) + (int)((uint32_t)x >> 31), (int)x}; }
 
+// The limbs of an operator entry, a double of magnitude up to 2^(e0 - 1023),
+// times 2^(60 + 1023 - e0).  The stencil negates limbs: the low one is kept
+// off -2^31 (by one unit).
+BR_D Fx2 fx_limbs_of(uint32_t lo, uint32_t hi, int e0) {
+  Fx2 r = fx_split(fx_from_bits<8>(lo, hi, max(e0, (int)((hi >> 20) & 0x7ffu)), 0));
+  r.l = max(r.l, -0x7fffffff);
+  return r;
+}
+// An operator entry as it is read: RAW a double, else its limbs.
+template <bool RAW>
+BR_D Fx2 fx_limbs(uint32_t w0, uint32_t w1, int e0) {
+  if constexpr (RAW) return fx_limbs_of(w0, w1, e0);
+  return {(int)w1, (int)w0};
+}
+
 // hh += a.h b.h, mid += a.h b.l + a.l b.h.
 BR_D void fx_mac(Fx2 a, Fx2 b, long long& hh, long long& mid) {
   asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(hh) : "r"(a.h), "r"(b.h));
@@ -99,6 +123,12 @@ BR_D uint32_t fx_max_word(const uint4 w[N]) {
   return m;
 }
 
+// What a site's exponent word says for the largest word of its components.
+BR_D int fx_site_exponent(uint32_t m) {
+  const int E = (int)(m >> 20);
+  return m == 0 ? 0 : (E < FX_EMIN || E > FX_EMAX) ? -1 : E;
+}
+
 // The fixed-point form of one FP64 spinor, stored at site ih of a block
 // (layout: fx_block_bytes).
 BR_D void fx_store(char* block, long vh, uint32_t ih, const cx<double> s[12]) {
@@ -115,7 +145,7 @@ BR_D void fx_store(char* block, long vh, uint32_t ih, const cx<double> s[12]) {
     const long long r = fx_from_bits<6>(w[k].x, w[k].y, E, 0), i = fx_from_bits<6>(w[k].z, w[k].w, E, 0);
     dst[k * vh] = make_uint4((uint32_t)r, (uint32_t)(r >> 32), (uint32_t)i, (uint32_t)(i >> 32));
   }
-  reinterpret_cast<int*>(block + 192 * vh)[ih] = m == 0 ? 0 : (E < FX_EMIN || E > FX_EMAX) ? -1 : E;
+  reinterpret_cast<int*>(block + 192 * vh)[ih] = fx_site_exponent(m);
 }
 
 BR_D long long fx_shift_round(long long x, int d) {  // x / 2^d to nearest, d in 0 .. 62
@@ -139,14 +169,24 @@ BR_D uint32_t fx_reaches(cx<long long> u) {
   return ((r ^ (r >> 31)) >= least ? 1u : 0u) | ((i ^ (i >> 31)) >= least ? 8u : 0u);
 }
 
-template <int MU>
-BR_D void fx_neighbours(const HopArgs& a, const int* ex, uint32_t ih, const int c[4], uint32_t xh, FxSlots& sh, int site,
+// The exponent word of site i of an FP64 block of N planes.
+template <int N>
+BR_D int fx_exponent(const char* block, long vh, uint32_t i) {
+  uint4 w[N];
+#pragma unroll
+  for (int k = 0; k < N; ++k) w[k] = __ldg(reinterpret_cast<const uint4*>(block) + k * vh + i);
+  return fx_site_exponent(fx_max_word<N>(w));
+}
+
+template <int MU, bool RAW>
+BR_D void fx_neighbours(const HopArgs& a, const char* in, uint32_t ih, const int c[4], uint32_t xh, FxSlots& sh, int site,
                         int& Ea, int& bad) {
   uint32_t f, b;
   bool wf, wb;
   neighbours<MU>(a.g, ih, c, xh, f, b, wf, wb);
   const float bc = a.bcf[MU];
-  int ef = __ldg(ex + f), eb = __ldg(ex + b);
+  const int* ex = reinterpret_cast<const int*>(in + 192 * a.g.vh);
+  int ef = RAW ? fx_exponent<12>(in, a.g.vh, f) : __ldg(ex + f), eb = RAW ? fx_exponent<12>(in, a.g.vh, b) : __ldg(ex + b);
   bad |= (ef < 0) | (eb < 0);
   if (wf && bc == 0.f) ef = FX_NO_HOP;
   if (wb && bc == 0.f) eb = FX_NO_HOP;
@@ -160,7 +200,14 @@ struct FxLoads {
   uint4 p, x, l[3];
 };
 
-BR_D cx<long long> fx_value(uint4 v) {
+// A spinor component of a site with exponent word E, as it is read: RAW two
+// doubles (E may be below them where the hop has phase 0: any value will do).
+template <bool RAW>
+BR_D cx<long long> fx_value(uint4 v, int E) {
+  if constexpr (RAW) {
+    auto one = [&](uint32_t lo, uint32_t hi) { return fx_from_bits<6>(lo, hi, max(E, (int)((hi >> 20) & 0x7ffu)), 0); };
+    return {one(v.x, v.y), one(v.z, v.w)};
+  }
   return {(long long)(((unsigned long long)v.y << 32) | v.x), (long long)(((unsigned long long)v.w << 32) | v.z)};
 }
 BR_D long long fx_sign(long long x, int m) { return (x ^ (long long)m) - (long long)m; }  // m = 0 or -1: x or -x
@@ -182,6 +229,7 @@ BR_D cx<long long> fx_shfl(cx<long long> v) {
 // issued while one is multiplied: unrolled over the directions the code
 // (115 KB) ran out of the instruction cache, and without the early loads the
 // kernel took 1.25 times as long.
+template <bool RAW>
 BR_D uint32_t fx_hops(const HopArgs& a, const char* in, const char* g_out, const char* g_in, long lbb, uint32_t ih, int Ea,
                   const FxSlots& sh, int site, int k, cx<long long> up[3], cx<long long> low[2][3]) {
   const long vs = 16 * a.g.vh;  // bytes of a plane
@@ -223,11 +271,12 @@ BR_D uint32_t fx_hops(const HopArgs& a, const char* in, const char* g_out, const
     const int s1 = fwd ? 1 : -1;
     long long rh[3] = {0, 0, 0}, rm[3] = {0, 0, 0}, jh[3] = {0, 0, 0}, jm[3] = {0, 0, 0};
     auto mac = [&](const FxLoads& f) {
-      const cx<long long> p = fx_value(f.p), x = fx_value(f.x);
+      const cx<long long> p = fx_value<RAW>(f.p, (int)w.y), x = fx_value<RAW>(f.x, (int)w.y);
       const Fx2 hr = fx_split(p.r + fx_sign(rot ? x.i : x.r, mr)), hi = fx_split(p.i + fx_sign(rot ? x.r : x.i, m));
 #pragma unroll
       for (int r = 0; r < 3; ++r) {
-        const Fx2 ur = {(int)f.l[r].y, (int)f.l[r].x}, ui = {s1 * (int)f.l[r].w, s1 * (int)f.l[r].z};
+        const Fx2 ur = fx_limbs<RAW>(f.l[r].x, f.l[r].y, 1023), li = fx_limbs<RAW>(f.l[r].z, f.l[r].w, 1023);
+        const Fx2 ui = {s1 * li.h, s1 * li.l};
         fx_mac(ur, hr, rh[r], rm[r]);
         fx_mac(fx_neg(ui), hi, rh[r], rm[r]);
         fx_mac(ur, hi, jh[r], jm[r]);
@@ -259,8 +308,9 @@ BR_D uint32_t fx_hops(const HopArgs& a, const char* in, const char* g_out, const
 
 // y = A x for one packed Hermitian 6x6 block in fixed point (entries below
 // 2^e times 2^(60 - e)) and |x| < 2^58 (twelve products then stay below
-// 2^63): y in units of 2^e times the unit of x.
-BR_D void fx_hermitian6(const char* base, long vh, uint32_t i, int b, const cx<long long> x[6], cx<long long> y[6]) {
+// 2^63): y in units of 2^e times the unit of x.  RAW: the block in FP64.
+template <bool RAW>
+BR_D void fx_hermitian6(const char* base, long vh, uint32_t i, int b, int e, const cx<long long> x[6], cx<long long> y[6]) {
   const uint4* p = reinterpret_cast<const uint4*>(base) + 18 * b * vh + i;
   Fx2 xr[6], xi[6];
   long long rh[6], rm[6], ih[6], im[6];
@@ -273,7 +323,7 @@ BR_D void fx_hermitian6(const char* base, long vh, uint32_t i, int b, const cx<l
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const uint4 w = ldg4<true>(p + k * vh);
-    const Fx2 d0 = {(int)w.y, (int)w.x}, d1 = {(int)w.w, (int)w.z};
+    const Fx2 d0 = fx_limbs<RAW>(w.x, w.y, 1023 + e), d1 = fx_limbs<RAW>(w.z, w.w, 1023 + e);
     fx_mac(d0, xr[2 * k], rh[2 * k], rm[2 * k]);
     fx_mac(d0, xi[2 * k], ih[2 * k], im[2 * k]);
     fx_mac(d1, xr[2 * k + 1], rh[2 * k + 1], rm[2 * k + 1]);
@@ -286,7 +336,7 @@ BR_D void fx_hermitian6(const char* base, long vh, uint32_t i, int b, const cx<l
     for (int c = 0; c < r; ++c) {
       const uint4 w = ldg4<true>(p + k * vh);
       ++k;
-      const Fx2 ar = {(int)w.y, (int)w.x}, ai = {(int)w.w, (int)w.z}, na = fx_neg(ai);
+      const Fx2 ar = fx_limbs<RAW>(w.x, w.y, 1023 + e), ai = fx_limbs<RAW>(w.z, w.w, 1023 + e), na = fx_neg(ai);
       fx_mac(ar, xr[c], rh[r], rm[r]);  // y_r += a x_c
       fx_mac(na, xi[c], rh[r], rm[r]);
       fx_mac(ar, xi[c], ih[r], im[r]);
@@ -439,8 +489,13 @@ __device__ __noinline__ void fx_site_fp64(const HopArgs& a, int rhs, uint32_t ih
 // (spins 2 k, 2 k + 1: one 6x6 clover block).  One lane a site needed 168
 // registers and left twelve warps on an SM, a third of the issue slots busy;
 // two need 128 (sixteen warps) and read each link as a broadcast.
-template <int FL, int RED>
-__global__ void __launch_bounds__(FX_THREADS, 4) hop_kernel_fx(const HopArgs a) {
+//
+// RAW (FX_RAW: no memory for the copies): operands converted as they are read,
+// every neighbour's exponent from its twelve components.  Full D on 24^3 x 48,
+// Wilson / clover: FP64 kernel 1421 / 1724 us, RAW 1023 / 1173, from copies 536
+// / 641 (staggered, stag.cuh: 528, 406, 238).
+template <int FL, int RED, bool RAW>
+__global__ void __launch_bounds__(FX_THREADS, RAW ? 2 : 4) hop_kernel_fx(const HopArgs a) {
   const int nrhs = a.nrhs;
   const int rhs = blockIdx.x % nrhs;
   const int sb = blockIdx.x / nrhs;
@@ -453,10 +508,9 @@ __global__ void __launch_bounds__(FX_THREADS, 4) hop_kernel_fx(const HopArgs a) 
   if (!skip) {
     const int p = a.out_parity, site = threadIdx.x >> 1, k = threadIdx.x & 1;
     const long lbb = link_block_bytes(P_F64, vh), cbb = clover_block_bytes(P_F64, vh);
-    const char* g_out = a.gauge_fx + (long)p * 4 * lbb;
-    const char* g_in = a.gauge_fx + (long)(1 - p) * 4 * lbb;
-    const char* in = a.in_fx + rhs * a.in_fx_rs;
-    const int* ex = reinterpret_cast<const int*>(in + 192 * vh);
+    const char* g_out = (RAW ? a.gauge : a.gauge_fx) + (long)p * 4 * lbb;
+    const char* g_in = (RAW ? a.gauge : a.gauge_fx) + (long)(1 - p) * 4 * lbb;
+    const char* in = RAW ? a.in + rhs * a.in_rs : a.in_fx + rhs * a.in_fx_rs;
     const uint32_t stride = (uint32_t)a.nblk * FX_SITES;
     // whole warps stay in the loop (shuffles): lanes past the end redo the last site
     for (uint32_t i0 = sb * FX_SITES + (site & ~15); i0 < (uint32_t)vh; i0 += stride) {
@@ -468,11 +522,11 @@ __global__ void __launch_bounds__(FX_THREADS, 4) hop_kernel_fx(const HopArgs a) 
         uint32_t xh;
         site_coords(a.g, ih, p, c, xh);
         if (k == 0) {
-          fx_neighbours<0>(a, ex, ih, c, xh, sh, site, Ea, bad);
-          fx_neighbours<1>(a, ex, ih, c, xh, sh, site, Ea, bad);
+          fx_neighbours<0, RAW>(a, in, ih, c, xh, sh, site, Ea, bad);
+          fx_neighbours<1, RAW>(a, in, ih, c, xh, sh, site, Ea, bad);
         } else {
-          fx_neighbours<2>(a, ex, ih, c, xh, sh, site, Ea, bad);
-          fx_neighbours<3>(a, ex, ih, c, xh, sh, site, Ea, bad);
+          fx_neighbours<2, RAW>(a, in, ih, c, xh, sh, site, Ea, bad);
+          fx_neighbours<3, RAW>(a, in, ih, c, xh, sh, site, Ea, bad);
         }
       }
       Ea = max(Ea, __shfl_xor_sync(0xffffffffu, Ea, 1));
@@ -480,7 +534,7 @@ __global__ void __launch_bounds__(FX_THREADS, 4) hop_kernel_fx(const HopArgs a) 
       cx<long long> q[6];
       {
         cx<long long> up[3], low[2][3];
-        const uint32_t mine = fx_hops(a, in, g_out, g_in, lbb, ih, Ea, sh, site, k, up, low);
+        const uint32_t mine = fx_hops<RAW>(a, in, g_out, g_in, lbb, ih, Ea, sh, site, k, up, low);
         // spin 0 or 1 from this lane's hops; spin 2 (lane 0) or 3 (lane 1) from both lanes'
         const uint32_t theirs = __shfl_xor_sync(0xffffffffu, mine, 1);
         if (Ea != 0 && ((mine & 0x3fu) != 0x3fu || (((mine >> 6) | (theirs >> 12)) & 0x3fu) != 0x3fu)) bad = 1;
@@ -503,7 +557,7 @@ __global__ void __launch_bounds__(FX_THREADS, 4) hop_kernel_fx(const HopArgs a) 
 #pragma unroll
         for (int j = 0; j < 6; ++j) q[j] = {fx_shift_round(q[j].r, d), fx_shift_round(q[j].i, d)};
         cx<long long> y[6];
-        fx_hermitian6(a.clovE_fx + p * cbb, vh, ih, k, q, y);
+        fx_hermitian6<RAW>((RAW ? a.clovE : a.clovE_fx) + p * cbb, vh, ih, k, a.eE_fx, q, y);
 #pragma unroll
         for (int j = 0; j < 6; ++j) q[j] = y[j];
         e += a.eE_fx + d;
@@ -550,7 +604,7 @@ __global__ void __launch_bounds__(FX_THREADS, 4) hop_kernel_fx(const HopArgs a) 
 #pragma unroll
           for (int j = 0; j < 6; ++j)
             q[j] = {fx_from_bits<5>(w[j].x, w[j].y, Es, 0), fx_from_bits<5>(w[j].z, w[j].w, Es, 0)};
-          fx_hermitian6(a.clovM_fx + p * cbb, vh, ih, k, q, y);
+          fx_hermitian6<RAW>((RAW ? a.clovM : a.clovM_fx) + p * cbb, vh, ih, k, a.eM_fx, q, y);
           // unit of q: 2^(Es - 1080); of y: 2^e times that
           const double fs = a.s1 * fx_pow2(Es - 57 + a.eM_fx);
 #pragma unroll

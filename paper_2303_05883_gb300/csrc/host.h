@@ -151,15 +151,6 @@ struct Stats {
   std::vector<cudaEvent_t> pool;
 };
 
-// The fixed-point copy of FP64 operator data (dslash_fx.cuh): built on first
-// use, or found unsuitable (an entry out of its range, no memory for it).
-struct FxCopy {
-  enum State { UNKNOWN, READY, UNSUITABLE };
-  State state = UNKNOWN;
-  int e = 0;  // entries are below 2^e (links: at most 1), their unit 2^(e - 60)
-  std::unique_ptr<DevBuf> buf;
-};
-
 // Clover term T = 1 - kcsw sum sigma F and its inverse for one value of
 // kcsw = kappa c_sw: FP64 masters plus lazily converted copies.  Shared by
 // the solves that use it, so a solve keeps its set alive even after the
@@ -167,7 +158,8 @@ struct FxCopy {
 struct CloverSet {
   double kcsw = 0.0;
   std::unique_ptr<DevBuf> T[4], Tinv[4];
-  FxCopy Tfx, Tinvfx;
+  uint32_t top[2] = {~0u, ~0u};  // largest high word of an |entry| of T and of T^-1
+  std::unique_ptr<DevBuf> fx[2];  // their fixed-point copies, where there was memory for them
   std::mutex mu;
 };
 
@@ -207,7 +199,9 @@ struct bridge_lattice_s {
   cudaStream_t stream = nullptr;
   // links per precision; [0] (F64, 18 reals) is the master copy
   std::unique_ptr<bridge::DevBuf> gauge[4];
-  bridge::FxCopy gauge_fx;  // the FP64 links in fixed point
+  uint32_t gauge_top = ~0u;  // largest high word of an |entry| of the FP64 links
+  std::unique_ptr<bridge::DevBuf> gauge_fx;  // their fixed-point copy, where there was memory for it;
+  bool gauge_fx_made = false;                // kept from one upload to the next, made again on first use
   std::mutex fx_mu;
   std::unique_ptr<bridge::DevBuf> fx_scratch;  // hop inputs in fixed point, for work on the lattice stream
   bool have_gauge = false;
@@ -256,21 +250,28 @@ const char* gauge_ptr(bridge_lattice_s* L, int prec);
 std::shared_ptr<CloverSet> clover_set(bridge_lattice_s* L, double kcsw);
 const char* clover_ptr(bridge_lattice_s* L, CloverSet& set, int prec, bool inverse);
 const char* clover_ptr(bridge_lattice_s* L, int prec, bool inverse, double kcsw);
-// The fixed-point copies of the FP64 links and clover blocks, or nullptr
-// where there is none and the FP64 kernels have to run: entries out of the
-// fixed-point range, no memory for the copy, or not built yet while st is
-// being captured into a graph.
-const char* gauge_fx_ptr(bridge_lattice_s* L, cudaStream_t st);
-const char* clover_fx_ptr(bridge_lattice_s* L, CloverSet& set, bool inverse, cudaStream_t st, int* e = nullptr);
-// Set the fixed-point pointers of an FP64 launch on stream st (set: the
-// clover set of the flags that need one; scratch as HopCall::fx_scratch) and
-// queue the conversion of its input; or leave them null.
-void set_fx_args(bridge_lattice_s* L, HopArgs& a, int flags, int red, CloverSet* set, char* scratch, cudaStream_t st);
+// Whether FP64 hops with these flags run in fixed point: a matter of the
+// entries of the links and clover blocks (set: of the flags that need one)
+// alone.  eE, eM: the exponents of T^-1 and T.
+bool fx_fits(bridge_lattice_s* L, const CloverSet* set, int flags, int* eE = nullptr, int* eM = nullptr);
+// The fixed-point copies of the operands, made on the lattice stream where
+// there is memory for them; null where there is none, or not made yet while the
+// lattice stream is being captured into a graph (the hops convert as they read).
+struct FxCopies {
+  const char *U = nullptr, *E = nullptr, *M = nullptr;
+};
+FxCopies fx_copies(bridge_lattice_s* L, CloverSet* set, int flags);
+// Set the fixed-point mode and pointers of an FP64 launch on stream st and
+// queue the conversion of its input where copies are used.  copies: what may
+// be read on st (null: fx_copies on the lattice stream, none on others);
+// scratch as HopCall::fx_scratch.
+void set_fx_args(bridge_lattice_s* L, HopArgs& a, int flags, int red, CloverSet* set, const FxCopies* copies,
+                 char* scratch, cudaStream_t st);
 // The lattice's scratch for hop inputs in fixed point (work on the lattice
 // stream), grown to `bytes`; null where there is no room or no growing now.
 char* fx_scratch(bridge_lattice_s* L, size_t bytes);
 // Where the FP64 application `which` (bridge_apply_op) of op on the lattice
-// stream runs in fixed point, room for nblocks half-lattice inputs; else null.
+// stream reads copies, room for nblocks half-lattice inputs; else null.
 char* fx_input(bridge_lattice_s* L, const bridge_op& op, int which, int nblocks);
 
 // ------------------------------------------------------- operators
@@ -292,8 +293,9 @@ struct HopCall {
   uint32_t n_map = 0;
   const char* in_fx = nullptr;  // FP64: `in` in fixed point, where the caller has it already
   long in_fx_rs = 0;
+  const FxCopies* fx = nullptr;  // FP64: the copies a launch on another stream than the lattice's may read
   char* fx_scratch = nullptr;  // FP64: room for nrhs blocks of fx_block_bytes (default: the lattice's, for
-                               // work on the lattice stream; elsewhere the launch stays on the FP64 kernel)
+                               // work on the lattice stream; elsewhere the launch converts as it reads)
   double work_fraction = 1.0;  // share of the sites the launch computes (for the byte and flop counts)
 };
 void run_hop(bridge_lattice_s* L, HopCall c, cudaStream_t st);

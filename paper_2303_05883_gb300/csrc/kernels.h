@@ -79,18 +79,20 @@ bool launch_clover_site(int prec, const CopyArgs& a, const char* clov, int block
 bool launch_g5_site(int prec, const CopyArgs& a, const char* clov, int block, cudaStream_t st);
 
 // ------------------------------------------------------- gauge, clover
-// Canonical FP64 links (4, V, 3, 3) -> internal F64 blocks [parity][mu].
-void launch_gauge_from_canon(const double* U, const Geom& g, char* g64, cudaStream_t st);
+// Canonical FP64 links (4, V, 3, 3) -> internal F64 blocks [parity][mu]; *top
+// (zero before) = the largest high word of an |entry|.
+void launch_gauge_from_canon(const double* U, const Geom& g, char* g64, uint32_t* top, cudaStream_t st);
 // Internal F64 links -> internal links of another precision.
 bool launch_gauge_convert(int prec, const Geom& g, const char* g64, char* gp, cudaStream_t st);
-// Clover term T = 1 - kcsw * sum sigma F and its inverse, packed FP64 [parity].
-void launch_clover_build(const Geom& g, const char* g64, double kcsw, char* T64, char* Tinv64, cudaStream_t st);
+// Clover term T = 1 - kcsw * sum sigma F and its inverse, packed FP64 [parity];
+// top[0], top[1] (zero before) = the largest high word of an |entry| of each.
+void launch_clover_build(const Geom& g, const char* g64, double kcsw, char* T64, char* Tinv64, uint32_t* top,
+                         cudaStream_t st);
 bool launch_clover_convert(int prec, const Geom& g, const char* c64, char* cp, cudaStream_t st);
 // FP64 half-lattice field src -> its fixed-point form dst (fx_block_bytes each).
 void launch_field_to_fx(const CopyArgs& a, int block, cudaStream_t st);
 // nb blocks, block_bytes apart, of n 16-byte entries (two doubles of magnitude
-// up to 2^e) -> the fixed-point form of dslash_fx.cuh, |entry| 2^(60 - e);
-// *top = the largest high word of an |entry|.
-void launch_to_fx(const char* src, char* dst, int nb, long n, long block_bytes, int e, uint32_t* top, cudaStream_t st);
+// up to 2^e) -> the fixed-point form of dslash_fx.cuh, |entry| 2^(60 - e).
+void launch_to_fx(const char* src, char* dst, int nb, long n, long block_bytes, int e, cudaStream_t st);
 
 }  // namespace bridge

@@ -468,10 +468,11 @@ bool launch_convert(int ps, int pd, const CopyArgs& a, int block, cudaStream_t s
 }
 
 // ----------------------------------------------------------- gauge field
-__global__ void __launch_bounds__(256) k_gauge_from_canon(const double* U, const Geom g, char* g64) {
+__global__ void __launch_bounds__(256) k_gauge_from_canon(const double* U, const Geom g, char* g64, uint32_t* top) {
   const long vh = g.vh, V = 2 * vh;
   const long lbb = link_block_bytes(P_F64, vh);
   const long n = 8 * vh;  // (parity, mu, ih)
+  uint32_t m = 0;
   for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (long)gridDim.x * blockDim.x) {
     const uint32_t ih = (uint32_t)(k % vh);
     const int mu = (int)((k / vh) % 4), p = (int)(k / (4 * vh));
@@ -482,15 +483,20 @@ __global__ void __launch_bounds__(256) k_gauge_from_canon(const double* U, const
     const double2* src = reinterpret_cast<const double2*>(U) + ((long)mu * V + lex) * 9;
     double2* dst = reinterpret_cast<double2*>(g64 + (long)(p * 4 + mu) * lbb);
 #pragma unroll
-    for (int e = 0; e < 9; ++e) dst[e * vh + ih] = __ldg(src + e);
+    for (int e = 0; e < 9; ++e) {
+      const double2 v = __ldg(src + e);
+      dst[e * vh + ih] = v;
+      m = max(m, high_word(v));
+    }
   }
+  warp_top(m, top);
 }
 
-void launch_gauge_from_canon(const double* U, const Geom& g, char* g64, cudaStream_t st) {
+void launch_gauge_from_canon(const double* U, const Geom& g, char* g64, uint32_t* top, cudaStream_t st) {
   const long n = 8L * g.vh;
   const int block = 256;
   const long grid = (n + block - 1) / block;
-  k_gauge_from_canon<<<(unsigned)(grid < 152 * 64 ? grid : 152 * 64), block, 0, st>>>(U, g, g64);
+  k_gauge_from_canon<<<(unsigned)(grid < 152 * 64 ? grid : 152 * 64), block, 0, st>>>(U, g, g64, top);
 }
 
 template <int P>

@@ -194,12 +194,16 @@ std::shared_ptr<CloverSet> clover_set(bridge_lattice_s* L, double kcsw) {
   auto s = std::make_shared<CloverSet>();
   s->kcsw = kcsw;
   const size_t n = (size_t)(2 * clover_block_bytes(P_F64, L->vh));
-  s->T[P_F64].reset(new DevBuf(n));
+  s->T[P_F64].reset(new DevBuf(n + 256));  // (behind T: the largest entries met)
   s->Tinv[P_F64].reset(new DevBuf(n));
+  uint32_t* top = reinterpret_cast<uint32_t*>(s->T[P_F64]->ptr + n);
+  BR_CUDA(cudaMemsetAsync(top, 0, sizeof(s->top), L->stream));
   note_launch(L, K_SETUP, 0, 0, L->stream, true);
-  launch_clover_build(L->g, L->gauge[P_F64]->ptr, kcsw, s->T[P_F64]->ptr, s->Tinv[P_F64]->ptr, L->stream);
+  launch_clover_build(L->g, L->gauge[P_F64]->ptr, kcsw, s->T[P_F64]->ptr, s->Tinv[P_F64]->ptr, top, L->stream);
   note_launch(L, K_SETUP, 0, 0, L->stream, false);
   BR_CUDA(cudaGetLastError());
+  BR_CUDA(cudaMemcpyAsync(s->top, top, sizeof(s->top), cudaMemcpyDeviceToHost, L->stream));
+  BR_CUDA(cudaStreamSynchronize(L->stream));
   L->clovers.insert(L->clovers.begin(), s);
   const size_t keep = 4;  // sets still used by a solve stay alive through its reference
   if (L->clovers.size() > keep) L->clovers.resize(keep);
@@ -232,107 +236,126 @@ static bool capturing(cudaStream_t st) {
   return !known || cap != cudaStreamCaptureStatusNone;
 }
 
-// The copy is made on the lattice stream, which orders it after the FP64
-// data, and waited for: other streams may read it next.  top(e): the high
-// word an entry must stay below for exponent e; e from `elo` to `ehi`.
-static const char* fx_copy(bridge_lattice_s* L, FxCopy& fx, const DevBuf& src, int nb, long block_bytes, long n, int elo,
-                           int ehi, const std::function<uint32_t(int)>& top, cudaStream_t st) {
-  if (fx.state == FxCopy::READY) return fx.buf->ptr;
-  if (fx.state == FxCopy::UNSUITABLE || capturing(st) || capturing(L->stream)) return nullptr;
-  fx.state = FxCopy::UNSUITABLE;
-  // leave the memory to the fields of a solve (up to 4 KB a site, seven link
-  // copies) where it is scarce
+bool fx_fits(bridge_lattice_s* L, const CloverSet* set, int flags, int* eE, int* eM) {
+  const int m = set ? fx_clov_exponent(set->top[0]) : 0, e = set ? fx_clov_exponent(set->top[1]) : 0;
+  if (eM) *eM = m;
+  if (eE) *eE = e;
+  return L->gauge_top < FX_LINK_TOP && (!(flags & F_SELF_CLOV) || m) && (!(flags & F_E_CLOV) || e);
+}
+
+// Whether `bytes` may go to data that only makes things faster: at most an
+// eighth of what is free, to leave the memory to the fields of a solve (up to
+// 4 KB a site, seven link copies) where it is scarce.  What the library's pool
+// holds unused is free.
+static bool fx_room(size_t bytes) {
+  int dev = 0;
+  cudaMemPool_t pool;
+  uint64_t held = 0, used = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
+    cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &held);
+    cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used);
+  }
+  cudaGetLastError();
+  const size_t idle = held > used ? (size_t)(held - used) : 0;
+  if (bytes <= idle / 8) return true;
   size_t free_b = 0, total_b = 0;
   BR_CUDA(cudaMemGetInfo(&free_b, &total_b));
-  if (src.bytes > free_b / 8) return nullptr;
-  std::unique_ptr<DevBuf> buf;
+  return bytes <= (free_b + idle) / 8;
+}
+
+// A buffer, from the pool in the order of the lattice stream if pooled, or null.
+static std::unique_ptr<DevBuf> fx_buffer(bridge_lattice_s* L, size_t bytes, bool pooled) {
+  if (capturing(L->stream) || !fx_room(bytes)) return nullptr;
   try {
-    buf.reset(new DevBuf(src.bytes + 256));  // (the last 256 bytes: the largest entry met)
+    return std::unique_ptr<DevBuf>(new DevBuf(bytes, L->stream, pooled));
   } catch (const Error&) {
     return nullptr;
   }
-  uint32_t* word = reinterpret_cast<uint32_t*>(buf->ptr + src.bytes);
-  for (int e = elo; e <= ehi; ++e) {
-    uint32_t seen = 0;
-    BR_CUDA(cudaMemsetAsync(word, 0, 256, L->stream));
-    note_launch(L, K_SETUP, 2.0 * src.bytes, 0, L->stream, true);
-    launch_to_fx(src.ptr, buf->ptr, nb, n, block_bytes, e, word, L->stream);
-    note_launch(L, K_SETUP, 0, 0, L->stream, false);
-    BR_CUDA(cudaGetLastError());
-    BR_CUDA(cudaMemcpyAsync(&seen, word, sizeof(seen), cudaMemcpyDeviceToHost, L->stream));
-    BR_CUDA(cudaStreamSynchronize(L->stream));
-    if (seen < top(e)) {
-      fx.buf = std::move(buf);
-      fx.e = e;
-      fx.state = FxCopy::READY;
-      return fx.buf->ptr;
-    }
-    if (seen >= top(ehi)) break;
+}
+
+// The copy is made on the lattice stream, which orders it after the FP64 data.
+static void fx_convert(bridge_lattice_s* L, const char* src, char* dst, int nb, long block_bytes, long n, int e) {
+  const double bytes = 2.0 * nb * block_bytes;
+  note_launch(L, K_SETUP, bytes, 0, L->stream, true);
+  launch_to_fx(src, dst, nb, n, block_bytes, e, L->stream);
+  note_launch(L, K_SETUP, bytes, 0, L->stream, false);
+  BR_CUDA(cudaGetLastError());
+}
+
+// (A clover set may outlive the stream of its lattice: its copies are not of
+// the pool.)
+static const char* fx_clover(bridge_lattice_s* L, CloverSet& set, bool inverse) {
+  std::unique_ptr<DevBuf>& buf = set.fx[inverse];
+  if (!buf) {
+    const long cbb = clover_block_bytes(P_F64, L->vh);
+    auto to = fx_buffer(L, (size_t)(2 * cbb), false);
+    if (!to) return nullptr;
+    fx_convert(L, (inverse ? set.Tinv : set.T)[P_F64]->ptr, to->ptr, 2, cbb, 36 * L->vh, fx_clov_exponent(set.top[inverse]));
+    buf = std::move(to);
   }
-  return nullptr;
+  return buf->ptr;
 }
 
-const char* gauge_fx_ptr(bridge_lattice_s* L, cudaStream_t st) {
-  std::lock_guard<std::mutex> lk(L->fx_mu);
-  return fx_copy(L, L->gauge_fx, *L->gauge[P_F64], 8, link_block_bytes(P_F64, L->vh), 9 * L->vh, 0, 0,
-                 [](int) { return FX_LINK_TOP; }, st);
-}
-
-const char* clover_fx_ptr(bridge_lattice_s* L, CloverSet& set, bool inverse, cudaStream_t st, int* e) {
-  std::lock_guard<std::mutex> lk(set.mu);
-  FxCopy& fx = inverse ? set.Tinvfx : set.Tfx;
-  const char* p = fx_copy(L, fx, inverse ? *set.Tinv[P_F64] : *set.T[P_F64], 2, clover_block_bytes(P_F64, L->vh),
-                          36 * L->vh, 1, FX_CLOV_EMAX, fx_clov_top, st);
-  if (e) *e = fx.e;
-  return p;
+FxCopies fx_copies(bridge_lattice_s* L, CloverSet* set, int flags) {
+  FxCopies c;
+  {
+    std::lock_guard<std::mutex> lk(L->fx_mu);
+    const long lbb = link_block_bytes(P_F64, L->vh);
+    if (!L->gauge_fx) L->gauge_fx = fx_buffer(L, (size_t)(8 * lbb), true);
+    if (L->gauge_fx && !L->gauge_fx_made && !capturing(L->stream)) {
+      fx_convert(L, L->gauge[P_F64]->ptr, L->gauge_fx->ptr, 8, lbb, 9 * L->vh, 0);
+      L->gauge_fx_made = true;
+    }
+    if (L->gauge_fx_made) c.U = L->gauge_fx->ptr;
+  }
+  if (!c.U || !(flags & (F_E_CLOV | F_SELF_CLOV))) return c;
+  std::lock_guard<std::mutex> lk(set->mu);
+  if (flags & F_SELF_CLOV) c.M = fx_clover(L, *set, false);
+  if (flags & F_E_CLOV) c.E = fx_clover(L, *set, true);
+  return c;
 }
 
 char* fx_scratch(bridge_lattice_s* L, size_t need) {
   if (!L->fx_scratch || L->fx_scratch->bytes < need) {
-    if (capturing(L->stream)) return nullptr;
-    L->fx_scratch.reset();
-    try {
-      L->fx_scratch.reset(new DevBuf(need));
-    } catch (const Error&) {
-      return nullptr;  // no room: the FP64 kernel needs none
-    }
+    auto grown = fx_buffer(L, need, true);
+    if (!grown) return nullptr;
+    L->fx_scratch = std::move(grown);
   }
   return L->fx_scratch->ptr;
 }
 
-void set_fx_args(bridge_lattice_s* L, HopArgs& a, int flags, int red, CloverSet* set, char* scratch, cudaStream_t st) {
-  a.gauge_fx = a.clovE_fx = a.clovM_fx = nullptr;
-  if (!fx_has(flags, red)) return;
-  if (!a.in_fx && !scratch && st != L->stream) return;
-  const char* E = (flags & F_E_CLOV) ? clover_fx_ptr(L, *set, true, st, &a.eE_fx) : nullptr;
-  const char* M = (flags & F_SELF_CLOV) ? clover_fx_ptr(L, *set, false, st, &a.eM_fx) : nullptr;
-  if (((flags & F_E_CLOV) && !E) || ((flags & F_SELF_CLOV) && !M)) return;
-  const char* U = gauge_fx_ptr(L, st);
-  if (!U) return;
+void set_fx_args(bridge_lattice_s* L, HopArgs& a, int flags, int red, CloverSet* set, const FxCopies* copies,
+                 char* scratch, cudaStream_t st) {
+  a.fx = FX_OFF;
+  if (!fx_has(flags, red) || !fx_fits(L, set, flags, &a.eE_fx, &a.eM_fx)) return;
+  a.eb_fx = a.beta != 0.0 && std::isfinite(a.beta) ? std::ilogb(a.beta) : -5000;
+  a.fx = FX_RAW;
+  const FxCopies c = copies ? *copies : st == L->stream ? fx_copies(L, set, flags) : FxCopies{};
+  if (!c.U || ((flags & F_E_CLOV) && !c.E) || ((flags & F_SELF_CLOV) && !c.M)) return;
   if (!a.in_fx) {
-    if (!scratch) scratch = fx_scratch(L, (size_t)a.nrhs * fx_block_bytes(L->vh));
+    if (!scratch && st == L->stream) scratch = fx_scratch(L, (size_t)a.nrhs * fx_block_bytes(L->vh));
     if (!scratch) return;
-    CopyArgs c;
-    std::memset(&c, 0, sizeof(c));
-    c.vh = (uint32_t)L->vh;
-    c.nrhs = a.nrhs;
-    c.nblk = (int)((L->vh + 255) / 256);
-    c.src = a.in;
-    c.src_rs = a.in_rs;
-    c.dst = scratch;
-    c.dst_rs = fx_block_bytes(L->vh);
-    c.red = a.red;  // right-hand sides whose solve has ended are skipped
+    CopyArgs v;
+    std::memset(&v, 0, sizeof(v));
+    v.vh = (uint32_t)L->vh;
+    v.nrhs = a.nrhs;
+    v.nblk = (int)((L->vh + 255) / 256);
+    v.src = a.in;
+    v.src_rs = a.in_rs;
+    v.dst = scratch;
+    v.dst_rs = fx_block_bytes(L->vh);
+    v.red = a.red;  // right-hand sides whose solve has ended are skipped
     const double bytes = (double)L->vh * a.nrhs * (192 + 196);
     note_launch(L, K_CONVERT, bytes, 0, st, true);
-    launch_field_to_fx(c, 256, st);
+    launch_field_to_fx(v, 256, st);
     note_launch(L, K_CONVERT, bytes, 0, st, false);
     a.in_fx = scratch;
-    a.in_fx_rs = c.dst_rs;
+    a.in_fx_rs = v.dst_rs;
   }
-  a.eb_fx = a.beta != 0.0 && std::isfinite(a.beta) ? std::ilogb(a.beta) : -5000;
-  a.gauge_fx = U;
-  a.clovE_fx = E;
-  a.clovM_fx = M;
+  a.fx = FX_COPIES;
+  a.gauge_fx = c.U;
+  a.clovE_fx = c.E;
+  a.clovM_fx = c.M;
 }
 
 // ------------------------------------------------------------ operators
@@ -399,7 +422,7 @@ void run_hop(bridge_lattice_s* L, HopCall c, cudaStream_t st) {
   a.red = c.redargs;
   a.in_fx = c.in_fx;
   a.in_fx_rs = c.in_fx_rs;
-  if (c.prec == P_F64 && !c.site_map) set_fx_args(L, a, c.flags, c.red, cs, c.fx_scratch, st);
+  if (c.prec == P_F64 && !c.site_map) set_fx_args(L, a, c.flags, c.red, cs, c.fx, c.fx_scratch, st);
   const std::string key = "hop/" + std::to_string(c.prec) + "/" + std::to_string(c.flags) + "/" +
                           std::to_string(c.red) + "/" + dims_key(L) + "/" + std::to_string(c.nrhs);
   const int variant = default_hop_variant(c.prec, c.flags, c.red, L->vh, c.nrhs, c.site_map != nullptr);
@@ -411,7 +434,7 @@ void run_hop(bridge_lattice_s* L, HopCall c, cudaStream_t st) {
   a.nblk = sh.nblk;
   if (c.red != R_NONE && a.red.partials == nullptr) {
     // a fixed-point launch takes up to one block for 64 sites
-    const long nb = a.gauge_fx ? std::max<long>(sh.nblk, (L->vh + 63) / 64) : sh.nblk;
+    const long nb = a.fx != FX_OFF ? std::max<long>(sh.nblk, (L->vh + 63) / 64) : sh.nblk;
     ensure_red_scratch(L, nb * c.nrhs, c.nrhs);
     a.red.partials = reinterpret_cast<double*>(L->red_partials->ptr);
     a.red.counter = reinterpret_cast<unsigned*>(L->red_counter->ptr);
@@ -431,14 +454,16 @@ void run_hop(bridge_lattice_s* L, HopCall c, cudaStream_t st) {
   BR_CUDA(cudaGetLastError());
 }
 
-// Whether the FP64 hops of op run in fixed point, and the scratch for the
-// fixed-point form of nblocks half-lattice inputs (null: they do not).
 char* fx_input(bridge_lattice_s* L, const bridge_op& op, int which, int nblocks) {
-  if (!gauge_fx_ptr(L, L->stream)) return nullptr;
-  if (op_is_clover(op) && which != BRIDGE_APPLY_DEO) {
-    auto set = clover_set(L, op_kcsw(op));
-    if (!clover_fx_ptr(L, *set, which == BRIDGE_APPLY_DHAT, L->stream)) return nullptr;
+  std::shared_ptr<CloverSet> set;
+  int flags = 0;
+  if (op_is_clover(op) && (which == BRIDGE_APPLY_D || which == BRIDGE_APPLY_DHAT)) {
+    set = clover_set(L, op_kcsw(op));
+    flags = which == BRIDGE_APPLY_D ? F_SELF_CLOV : F_E_CLOV;
   }
+  if (!fx_fits(L, set.get(), flags)) return nullptr;
+  const FxCopies c = fx_copies(L, set.get(), flags);
+  if (!c.U || ((flags & F_E_CLOV) && !c.E) || ((flags & F_SELF_CLOV) && !c.M)) return nullptr;
   return fx_scratch(L, (size_t)nblocks * fx_block_bytes(L->vh));
 }
 

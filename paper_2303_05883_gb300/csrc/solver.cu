@@ -169,10 +169,9 @@ SolveState::SolveState(bridge_lattice_s* L, const bridge_op& op, const bridge_so
     clov_ = clover_set(L_, kcsw_);
     clover_ptr(L_, *clov_, P_, true);
     clover_ptr(L_, *clov_, P_F64, false);
-    clover_fx_ptr(L_, *clov_, false, st_);
-    if (P_ == P_F64) clover_fx_ptr(L_, *clov_, true, st_);
   }
-  gauge_fx_ptr(L_, st_);
+  const int fl = clover_ ? F_SELF_CLOV | (P_ == P_F64 ? F_E_CLOV : 0) : 0;
+  if (fx_fits(L_, clov_.get(), fl)) fx_ = fx_copies(L_, clov_.get(), fl);
   if (st_ != L_->stream) BR_CUDA(cudaStreamSynchronize(L_->stream));
 }
 
@@ -208,6 +207,7 @@ void SolveState::enqueue_residual() {
   for (int q = 0; q < 2; ++q) {
     HopCall c;
     c.prec = P_F64;
+    c.fx = &fx_;
     c.fx_scratch = fx_scratch();
     c.flags = F_AUX | F_SELF | (clover_ ? F_SELF_CLOV : 0);
     c.red = R_NORM;
@@ -300,6 +300,7 @@ void SolveState::begin_inner() {
   // b^_e = T_ee^-1 (r_e + kappa H_eo T_oo^-1 r_o)
   HopCall c;
   c.prec = P_;
+  c.fx = &fx_;
   c.fx_scratch = fx_scratch();
   c.nrhs = nrhs_;
   c.kcsw = kcsw_;
@@ -358,6 +359,7 @@ void SolveState::enqueue_iteration() {
   const double S = P_ == P_F64 ? 192 : P_ == P_F32 ? 96 : 52, SX = PX_ == P_F64 ? 192 : PX_ == P_F32 ? 96 : 52;
   HopCall c;
   c.prec = P_;
+  c.fx = &fx_;
   c.fx_scratch = fx_scratch();
   c.nrhs = nrhs_;
   c.kcsw = kcsw_;
@@ -441,6 +443,7 @@ RedArgs SolveState::cg_red(int fin, bool check_done) {
 void SolveState::cg_dhat_norm(const Field& in, const Field& out) {
   HopCall c;
   c.prec = P_;
+  c.fx = &fx_;
   c.fx_scratch = fx_scratch();
   c.nrhs = nrhs_;
   c.kcsw = kcsw_;
@@ -494,6 +497,7 @@ void SolveState::cg_dhat_dag(const Field& in, const Field& out, bool check_done)
   BR_CUDA(cudaGetLastError());
   HopCall c;
   c.prec = P_;
+  c.fx = &fx_;
   c.fx_scratch = fx_scratch();
   c.nrhs = nrhs_;
   c.kcsw = kcsw_;
@@ -763,6 +767,7 @@ void SolveState::finish_inner() {
   }
   HopCall c;
   c.prec = P_;
+  c.fx = &fx_;
   c.fx_scratch = fx_scratch();
   c.nrhs = nrhs_;
   c.kcsw = kcsw_;

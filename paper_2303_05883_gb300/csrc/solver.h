@@ -92,6 +92,7 @@ class SolveState {
 
   Field b64_, x64_, r64_, rin_, bh_, r_, rhat_, p_, v_, s_, t_, xin_, xinp_, tmp_, eo_;
   std::unique_ptr<DevBuf> scal_, partials_, counter_, result_, mask_, fxs_;
+  FxCopies fx_;  // of the FP64 operands (null pointers: none, the hops convert as they read)
   char* fx_scratch() const { return fxs_ ? fxs_->ptr : v_.buf->ptr; }
   std::unique_ptr<PinnedBuf> h_sc_[2], h_result_, h_mask_, h_init_;
   cudaEvent_t ev_[2] = {nullptr, nullptr};

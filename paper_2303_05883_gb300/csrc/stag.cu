@@ -87,7 +87,7 @@ template <int RED>
 int fx_nblk(long vh, int nrhs) {
   static int n = 0;
   if (n == 0) {
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, stag_hop_fx_kernel<RED>, SFX_THREADS, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, stag_hop_fx_kernel<RED, false>, SFX_THREADS, 0);
     if (n <= 0) n = 1;
   }
   const long cover = (vh + SFX_THREADS - 1) / SFX_THREADS, persist = (long)sm_count() * n / std::max(1, nrhs);
@@ -97,11 +97,15 @@ int fx_nblk(long vh, int nrhs) {
 template <int RED>
 void launch_fx(StagArgs a, cudaStream_t st) {
   a.nblk = fx_nblk<RED>(a.g.vh, a.nrhs);
-  stag_hop_fx_kernel<RED><<<(unsigned)(a.nblk * a.nrhs), SFX_THREADS, 0, st>>>(a);
+  const unsigned grid = (unsigned)(a.nblk * a.nrhs);  // the same for both: the order of a reduction is
+  if (a.fx == FX_RAW)
+    stag_hop_fx_kernel<RED, true><<<grid, SFX_THREADS, 0, st>>>(a);
+  else
+    stag_hop_fx_kernel<RED, false><<<grid, SFX_THREADS, 0, st>>>(a);
 }
 
 void launch_stag_hop(int prec, int red, StagArgs a, cudaStream_t st) {
-  if (a.gauge_fx) {
+  if (a.fx != FX_OFF) {
     if (red == SR_NONE) launch_fx<SR_NONE>(a, st);
     else if (red == SR_NORM) launch_fx<SR_NORM>(a, st);
     else launch_fx<SR_DOT_SELF>(a, st);
@@ -187,12 +191,13 @@ void run_stag_hop(bridge_lattice_s* L, const bridge_op& op, const StagHop& c, cu
   a.aux_rs = c.aux_rs;
   a.gauge = gauge_ptr(L, c.prec);
   a.red = c.redargs;
-  if (c.prec == P_F64) {
-    // in fixed point, unless the links have no such copy or there is no room for the input's
-    const char* U = gauge_fx_ptr(L, st);
+  if (c.prec == P_F64 && fx_fits(L, nullptr, 0)) {
+    // in fixed point, from copies where the links and the input have one
+    const char* U = st == L->stream ? fx_copies(L, nullptr, 0).U : nullptr;
+    a.fx = FX_RAW;
     a.in_fx = c.in_fx;
     a.in_fx_rs = c.in_fx_rs;
-    if (U && !a.in_fx && st == L->stream) {
+    if (U && !a.in_fx) {
       char* to = fx_scratch(L, (size_t)c.nrhs * stag_fx_block_bytes(L->vh));
       if (to) {
         const int nb = vec_nblk(L->vh, c.nrhs);
@@ -205,7 +210,10 @@ void run_stag_hop(bridge_lattice_s* L, const bridge_op& op, const StagHop& c, cu
         note_launch(L, K_STAG_VEC, bytes, 0, st, false);
       }
     }
-    if (a.in_fx) a.gauge_fx = U;
+    if (U && a.in_fx) {
+      a.fx = FX_COPIES;
+      a.gauge_fx = U;
+    }
   }
   if (c.red != SR_NONE && a.red.partials == nullptr) {
     const long nb = std::max<long>(stag_nblk(c.prec, c.red, L->vh, c.nrhs), (L->vh + SFX_THREADS - 1) / SFX_THREADS);
@@ -272,7 +280,7 @@ void stag_canon(bridge_lattice_s* L, const Field& f, double* canon, bool full, c
 }  // namespace
 
 char* stag_fx_input(bridge_lattice_s* L, int nblocks) {
-  return gauge_fx_ptr(L, L->stream) ? fx_scratch(L, (size_t)nblocks * stag_fx_block_bytes(L->vh)) : nullptr;
+  return fx_fits(L, nullptr, 0) && fx_copies(L, nullptr, 0).U ? fx_scratch(L, (size_t)nblocks * stag_fx_block_bytes(L->vh)) : nullptr;
 }
 
 void stag_canon_to_field(bridge_lattice_s* L, const double* canon, const Field& f, bool canon_full, cudaStream_t st) {

@@ -96,7 +96,8 @@ struct StagArgs {
   const char* aux;   // may be null
   long aux_rs;
   const char* gauge;  // [parity][mu] link blocks
-  const char* gauge_fx;  // FP64 in fixed point: the links and the input
+  int fx;                // FP64: an FxMode, and for FX_COPIES the links and the input in fixed point
+  const char* gauge_fx;
   const char* in_fx;
   long in_fx_rs;
   RedArgs red;
@@ -228,19 +229,20 @@ BR_D void stag_fx_store(char* block, long vh, uint32_t ih, const cx<double> v[3]
     reinterpret_cast<uint4*>(block)[k * vh + ih] =
         make_uint4((uint32_t)r, (uint32_t)(r >> 32), (uint32_t)i, (uint32_t)(i >> 32));
   }
-  reinterpret_cast<int*>(block + 48 * vh)[ih] = m == 0 ? 0 : (E < FX_EMIN || E > FX_EMAX) ? -1 : E;
+  reinterpret_cast<int*>(block + 48 * vh)[ih] = fx_site_exponent(m);
 }
 
 // Slots of one site (direction 2 mu + backward): neighbour index, bit 31 the
 // sign of the hop (staggered and boundary phase, - for backward), exponent.
-template <int MU>
-BR_D void stag_fx_slots(const StagArgs& a, const int* ex, uint32_t ih, const int c[4], uint32_t xh, uint32_t eta_neg,
+template <int MU, bool RAW>
+BR_D void stag_fx_slots(const StagArgs& a, const char* in, uint32_t ih, const int c[4], uint32_t xh, uint32_t eta_neg,
                         uint2 (*w)[SFX_THREADS], int& Ea, bool& bad) {
   uint32_t f, b;
   bool wf, wb;
   neighbours<MU>(a.g, ih, c, xh, f, b, wf, wb);
   const uint32_t neg = a.bcf[MU] < 0.f;
-  const int ef = __ldg(ex + f), eb = __ldg(ex + b);
+  const int* ex = reinterpret_cast<const int*>(in + 48 * a.g.vh);
+  const int ef = RAW ? fx_exponent<3>(in, a.g.vh, f) : __ldg(ex + f), eb = RAW ? fx_exponent<3>(in, a.g.vh, b) : __ldg(ex + b);
   bad = bad || ef < 0 || eb < 0;
   Ea = max(Ea, max(ef, eb));
   w[2 * MU][threadIdx.x] = make_uint2(f | ((eta_neg ^ (wf & neg)) << 31), (uint32_t)ef);
@@ -258,17 +260,17 @@ BR_D void stag_fx_load(StagFxLoads& f, const char* in, const char* g, long vs, u
 }
 
 // The hop's result is added to acc; returned: the components it reaches (fx_reaches).
-template <bool FWD>
+template <bool FWD, bool RAW>
 BR_D uint32_t stag_fx_mac(const StagFxLoads& f, uint2 w, int Ea, cx<long long> acc[3]) {
   long long rh[3] = {0, 0, 0}, rm[3] = {0, 0, 0}, jh[3] = {0, 0, 0}, jm[3] = {0, 0, 0};
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const cx<long long> v = fx_value(f.v[c]);
+    const cx<long long> v = fx_value<RAW>(f.v[c], (int)w.y);
     const Fx2 hr = fx_split(v.r), hi = fx_split(v.i);
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
       const uint4 l = f.l[FWD ? 3 * r + c : 3 * c + r];
-      const Fx2 ur = {(int)l.y, (int)l.x}, ui = {(int)l.w, (int)l.z}, nui = fx_neg(ui);
+      const Fx2 ur = fx_limbs<RAW>(l.x, l.y, 1023), ui = fx_limbs<RAW>(l.z, l.w, 1023), nui = fx_neg(ui);
       fx_mac(ur, hr, rh[r], rm[r]);
       fx_mac(FWD ? nui : ui, hi, rh[r], rm[r]);
       fx_mac(ur, hi, jh[r], jm[r]);
@@ -297,8 +299,8 @@ __device__ __noinline__ inline void stag_fx_site_fp64(const StagArgs& a, int rhs
   for (int k = 0; k < 3; ++k) out[k] = make_double2(v[k].r, v[k].i);
 }
 
-template <int RED>
-__global__ void __launch_bounds__(SFX_THREADS, 4) stag_hop_fx_kernel(const StagArgs a) {
+template <int RED, bool RAW>
+__global__ void __launch_bounds__(SFX_THREADS, RAW ? 2 : 4) stag_hop_fx_kernel(const StagArgs a) {
   const int nrhs = a.nrhs;
   const int rhs = blockIdx.x % nrhs;
   const int sb = blockIdx.x / nrhs;
@@ -310,10 +312,9 @@ __global__ void __launch_bounds__(SFX_THREADS, 4) stag_hop_fx_kernel(const StagA
   if (!skip) {
     const int p = a.out_parity;
     const long lbb = link_block_bytes(P_F64, vh);
-    const char* g_out = a.gauge_fx + (long)p * 4 * lbb;
-    const char* g_in = a.gauge_fx + (long)(1 - p) * 4 * lbb;
-    const char* in = a.in_fx + rhs * a.in_fx_rs;
-    const int* ex = reinterpret_cast<const int*>(in + 48 * vh);
+    const char* g_out = (RAW ? a.gauge : a.gauge_fx) + (long)p * 4 * lbb;
+    const char* g_in = (RAW ? a.gauge : a.gauge_fx) + (long)(1 - p) * 4 * lbb;
+    const char* in = RAW ? a.in + rhs * a.in_rs : a.in_fx + rhs * a.in_fx_rs;
     const uint32_t stride = (uint32_t)a.nblk * SFX_THREADS;
     for (uint32_t ih = sb * SFX_THREADS + threadIdx.x; ih < (uint32_t)vh; ih += stride) {
       int Ea = 0;
@@ -322,10 +323,10 @@ __global__ void __launch_bounds__(SFX_THREADS, 4) stag_hop_fx_kernel(const StagA
         int c[4];
         uint32_t xh;
         site_coords(a.g, ih, p, c, xh);
-        stag_fx_slots<0>(a, ex, ih, c, xh, 0u, slot, Ea, bad);
-        stag_fx_slots<1>(a, ex, ih, c, xh, c[0] & 1, slot, Ea, bad);
-        stag_fx_slots<2>(a, ex, ih, c, xh, (c[0] + c[1]) & 1, slot, Ea, bad);
-        stag_fx_slots<3>(a, ex, ih, c, xh, (c[0] + c[1] + c[2]) & 1, slot, Ea, bad);
+        stag_fx_slots<0, RAW>(a, in, ih, c, xh, 0u, slot, Ea, bad);
+        stag_fx_slots<1, RAW>(a, in, ih, c, xh, c[0] & 1, slot, Ea, bad);
+        stag_fx_slots<2, RAW>(a, in, ih, c, xh, (c[0] + c[1]) & 1, slot, Ea, bad);
+        stag_fx_slots<3, RAW>(a, in, ih, c, xh, (c[0] + c[1] + c[2]) & 1, slot, Ea, bad);
       }
       cx<double> v[3], s[3];
       if (a.self != nullptr) load_cvec<P_F64>(a.self + rhs * a.self_rs, vh, ih, s);
@@ -339,8 +340,8 @@ __global__ void __launch_bounds__(SFX_THREADS, 4) stag_hop_fx_kernel(const StagA
           const uint32_t nf = wf.x & 0x7fffffffu, nb = wb.x & 0x7fffffffu;
           stag_fx_load(f, in, g_out + mu * lbb, vs, nf, ih);
           stag_fx_load(b, in, g_in + mu * lbb, vs, nb, nb);
-          reach |= stag_fx_mac<true>(f, wf, Ea, acc);
-          reach |= stag_fx_mac<false>(b, wb, Ea, acc);
+          reach |= stag_fx_mac<true, RAW>(f, wf, Ea, acc);
+          reach |= stag_fx_mac<false, RAW>(b, wb, Ea, acc);
         }
         bad = Ea != 0 && reach != 0x3fu;
       }

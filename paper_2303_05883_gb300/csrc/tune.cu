@@ -201,7 +201,7 @@ void tune_solver_kernels(bridge_lattice_s* L, const bridge_op& op, int prec, int
     if (v.flags & F_E_CLOV) a.clovE = clover_ptr(L, *cs, prec, true);
     if (v.flags & F_SELF_CLOV) a.clovM = clover_ptr(L, *cs, prec, false);
     if (v.flags & F_SELF_CLOV) a.s1 = -1.0;
-    if (prec == P_F64) set_fx_args(L, a, v.flags, v.red, cs.get(), nullptr, st);
+    if (prec == P_F64) set_fx_args(L, a, v.flags, v.red, cs.get(), nullptr, nullptr, st);
     a.red = red;
     a.red.fin = v.red == R_NONE ? FIN_NONE : FIN_STORE;
     const std::string key = "hop/" + std::to_string(prec) + "/" + std::to_string(v.flags) + "/" + std::to_string(v.red) +
