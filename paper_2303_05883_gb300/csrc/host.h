@@ -255,8 +255,9 @@ const char* clover_ptr(bridge_lattice_s* L, int prec, bool inverse, double kcsw)
 // alone.  eE, eM: the exponents of T^-1 and T.
 bool fx_fits(bridge_lattice_s* L, const CloverSet* set, int flags, int* eE = nullptr, int* eM = nullptr);
 // The fixed-point copies of the operands, made on the lattice stream where
-// there is memory for them; null where there is none, or not made yet while the
-// lattice stream is being captured into a graph (the hops convert as they read).
+// there is memory for them; null where there is none (the hops convert as they
+// read).  None either while the lattice stream is being captured: the graph may
+// be replayed when copies and scratch have moved.
 struct FxCopies {
   const char *U = nullptr, *E = nullptr, *M = nullptr;
 };
@@ -268,7 +269,7 @@ FxCopies fx_copies(bridge_lattice_s* L, CloverSet* set, int flags);
 void set_fx_args(bridge_lattice_s* L, HopArgs& a, int flags, int red, CloverSet* set, const FxCopies* copies,
                  char* scratch, cudaStream_t st);
 // The lattice's scratch for hop inputs in fixed point (work on the lattice
-// stream), grown to `bytes`; null where there is no room or no growing now.
+// stream), grown to `bytes`; null where there is no room, or in a capture.
 char* fx_scratch(bridge_lattice_s* L, size_t bytes);
 // Where the FP64 application `which` (bridge_apply_op) of op on the lattice
 // stream reads copies, room for nblocks half-lattice inputs; else null.

@@ -265,7 +265,7 @@ static bool fx_room(size_t bytes) {
 
 // A buffer, from the pool in the order of the lattice stream if pooled, or null.
 static std::unique_ptr<DevBuf> fx_buffer(bridge_lattice_s* L, size_t bytes, bool pooled) {
-  if (capturing(L->stream) || !fx_room(bytes)) return nullptr;
+  if (!fx_room(bytes)) return nullptr;
   try {
     return std::unique_ptr<DevBuf>(new DevBuf(bytes, L->stream, pooled));
   } catch (const Error&) {
@@ -298,11 +298,12 @@ static const char* fx_clover(bridge_lattice_s* L, CloverSet& set, bool inverse) 
 
 FxCopies fx_copies(bridge_lattice_s* L, CloverSet* set, int flags) {
   FxCopies c;
+  if (capturing(L->stream)) return c;
   {
     std::lock_guard<std::mutex> lk(L->fx_mu);
     const long lbb = link_block_bytes(P_F64, L->vh);
     if (!L->gauge_fx) L->gauge_fx = fx_buffer(L, (size_t)(8 * lbb), true);
-    if (L->gauge_fx && !L->gauge_fx_made && !capturing(L->stream)) {
+    if (L->gauge_fx && !L->gauge_fx_made) {
       fx_convert(L, L->gauge[P_F64]->ptr, L->gauge_fx->ptr, 8, lbb, 9 * L->vh, 0);
       L->gauge_fx_made = true;
     }
@@ -316,6 +317,7 @@ FxCopies fx_copies(bridge_lattice_s* L, CloverSet* set, int flags) {
 }
 
 char* fx_scratch(bridge_lattice_s* L, size_t need) {
+  if (capturing(L->stream)) return nullptr;
   if (!L->fx_scratch || L->fx_scratch->bytes < need) {
     auto grown = fx_buffer(L, need, true);
     if (!grown) return nullptr;
