@@ -2,6 +2,7 @@
 // host <-> device staging, and dispatch to the runtime and solver.
 #include <cmath>
 #include <cstring>
+#include <set>
 #include <string>
 
 #include "dwf.h"
@@ -20,6 +21,25 @@ extern std::atomic<long> g_dev_allocs;
 void tune_cache_load(bridge_lattice_s* L);
 int engine_submit(bridge_lattice_s* L, const bridge_op& op, const bridge_solver& s, const double* b, int nrhs,
                   bool borrow, bridge_request_h* out);
+
+// The lattices that exist, for release_idle.
+static std::mutex g_lattices_mu;
+static std::set<bridge_lattice_s*> g_lattices;
+
+bool release_idle(bridge_lattice_s* L, const std::vector<bridge_lattice_s*>& parts) {
+  std::lock_guard<std::mutex> lk(g_lattices_mu);
+  bool any = fx_release(L);
+  for (bridge_lattice_s* p : parts) any = fx_release(p) || any;
+  for (bridge_lattice_s* other : g_lattices) {
+    if (other == L || other->part || other->device != L->device) continue;
+    std::unique_lock<std::mutex> lo(other->api_mu, std::try_to_lock);
+    if (lo.owns_lock()) any = fx_release(other) || any;
+  }
+  cudaMemPool_t pool;
+  if (cudaDeviceGetDefaultMemPool(&pool, L->device) == cudaSuccess) cudaMemPoolTrimTo(pool, 0);
+  cudaGetLastError();
+  return any;
+}
 
 Field& workspace(bridge_lattice_s* L, const std::string& name, int prec, int subset, int nrhs) {
   const std::string key = name + "/" + std::to_string(prec) + "/" + std::to_string(subset) + "/" + std::to_string(nrhs);
@@ -166,16 +186,18 @@ static int mult_common(bridge_lattice L, const bridge_op* op, int prec, int whic
   std::lock_guard<std::mutex> lk(L->api_mu);
   const long sites = which == BRIDGE_APPLY_D ? L->V : L->vh;
   const size_t n = (size_t)nrhs * site_doubles(*op) * sites * sizeof(double);
-  if (host) {
-    double* din = reinterpret_cast<double*>(stage(L->stage_in, n));
-    double* dout = reinterpret_cast<double*>(stage(L->stage_out, n));
-    BR_CUDA(cudaMemcpyAsync(din, in, n, cudaMemcpyHostToDevice, L->stream));
-    mult_dev(L, *op, prec, which, out_parity, din, dout, nrhs);
-    BR_CUDA(cudaMemcpyAsync(out, dout, n, cudaMemcpyDeviceToHost, L->stream));
-    BR_CUDA(cudaStreamSynchronize(L->stream));
-  } else {
-    mult_dev(L, *op, prec, which, out_parity, in, out, nrhs);
-  }
+  with_room(L, [&] {
+    if (host) {
+      double* din = reinterpret_cast<double*>(stage(L->stage_in, n));
+      double* dout = reinterpret_cast<double*>(stage(L->stage_out, n));
+      BR_CUDA(cudaMemcpyAsync(din, in, n, cudaMemcpyHostToDevice, L->stream));
+      mult_dev(L, *op, prec, which, out_parity, din, dout, nrhs);
+      BR_CUDA(cudaMemcpyAsync(out, dout, n, cudaMemcpyDeviceToHost, L->stream));
+      BR_CUDA(cudaStreamSynchronize(L->stream));
+    } else {
+      mult_dev(L, *op, prec, which, out_parity, in, out, nrhs);
+    }
+  });
   BR_API_END
 }
 
@@ -195,24 +217,21 @@ static int solve_common(bridge_lattice L, const bridge_op* op, const bridge_solv
   const size_t n = (size_t)nrhs * site_doubles(*op) * L->V * sizeof(double);
   const double* db = b;
   double* dx = x;
-  if (host) {
-    db = reinterpret_cast<double*>(stage(L->stage_in, n));
-    dx = reinterpret_cast<double*>(stage(L->stage_out, n));
-    BR_CUDA(cudaMemcpyAsync(const_cast<double*>(db), b, n, cudaMemcpyHostToDevice, L->stream));
-    BR_CUDA(cudaMemcpyAsync(dx, x, n, cudaMemcpyHostToDevice, L->stream));
-  }
-  int status;
-  if (op_is_mobius(*op)) {
-    status = dwf_solve(L, *op, *s, db, dx, nrhs, info);
-  } else if (op_is_staggered(*op)) {
-    status = stag_solve(L, *op, *s, db, dx, nrhs, info);
-  } else {
+  const int status = with_room(L, [&] {
+    if (host) {
+      db = reinterpret_cast<double*>(stage(L->stage_in, n));
+      dx = reinterpret_cast<double*>(stage(L->stage_out, n));
+      BR_CUDA(cudaMemcpyAsync(const_cast<double*>(db), b, n, cudaMemcpyHostToDevice, L->stream));
+      BR_CUDA(cudaMemcpyAsync(dx, x, n, cudaMemcpyHostToDevice, L->stream));
+    }
+    if (op_is_mobius(*op)) return dwf_solve(L, *op, *s, db, dx, nrhs, info);
+    if (op_is_staggered(*op)) return stag_solve(L, *op, *s, db, dx, nrhs, info);
     SolveState S(L, *op, *s, nrhs, L->stream, db, dx);
     while (!S.advance()) BR_CUDA(cudaEventSynchronize(S.wait_event()));
     if (info)
       for (int r = 0; r < nrhs; ++r) info[r] = S.info()[r];
-    status = S.status();
-  }
+    return S.status();
+  });
   if (host) {
     BR_CUDA(cudaMemcpyAsync(x, dx, n, cudaMemcpyDeviceToHost, L->stream));
     BR_CUDA(cudaStreamSynchronize(L->stream));
@@ -259,6 +278,10 @@ int bridge_lattice_create(const int dims[4], bridge_lattice* out) {
     throw Error{BRIDGE_ECUDA, cudaGetErrorString(se)};
   }
   tune_cache_load(L);
+  {
+    std::lock_guard<std::mutex> lk(g_lattices_mu);
+    g_lattices.insert(L);
+  }
   *out = L;
   BR_API_END
 }
@@ -267,6 +290,10 @@ int bridge_lattice_destroy(bridge_lattice L) {
   BR_API_BEGIN
   if (!L) return BRIDGE_OK;
   BR_CHECK(L->in_flight.load() == 0, BRIDGE_ESTATE, "requests on this lattice are still running");
+  {
+    std::lock_guard<std::mutex> lk(g_lattices_mu);
+    g_lattices.erase(L);
+  }
   cudaStreamSynchronize(L->stream);
   {
     std::lock_guard<std::mutex> lk(L->stats.mu);
@@ -397,7 +424,13 @@ int bridge_field_create(bridge_lattice L, int prec, int subset, int nrhs, bridge
   auto* f = new bridge_field_s();
   f->L = L;
   try {
-    f->f = make_field(prec, subset, nrhs, L->vh);
+    try {
+      f->f = make_field(prec, subset, nrhs, L->vh);
+    } catch (const Error&) {
+      std::lock_guard<std::mutex> lk(L->api_mu);
+      if (!release_idle(L)) throw;
+      f->f = make_field(prec, subset, nrhs, L->vh);
+    }
   } catch (...) {
     delete f;
     throw;
@@ -503,7 +536,7 @@ int bridge_apply(bridge_lattice L, const bridge_op* op, int which, bridge_field 
       break;
     case BRIDGE_APPLY_DHAT: {
       BR_CHECK(in->f.subset != BRIDGE_ODD && out->f.subset != BRIDGE_ODD, BRIDGE_EINVAL, "D^ acts on even fields");
-      Field& tmp = workspace(L, "apply_tmp", in->f.prec, BRIDGE_ODD, in->f.nrhs);
+      Field& tmp = *with_room(L, [&] { return &workspace(L, "apply_tmp", in->f.prec, BRIDGE_ODD, in->f.nrhs); });
       apply_dhat(L, *op, out->f, in->f, tmp, L->stream);
       break;
     }

@@ -631,6 +631,7 @@ extern "C" int bridge_dd_create(bridge_lattice L, const bridge_op* op, int npart
     s.t0 = pl.t0;
     const int st = bridge_lattice_create(pl.local_dims, &s.L);
     if (st != BRIDGE_OK) throw Error{st, "slab lattice"};
+    s.L->part = true;
     BR_CUDA(cudaStreamCreateWithFlags(&s.comm, cudaStreamNonBlocking));
     BR_CUDA(cudaEventCreateWithFlags(&s.ev_in, cudaEventDisableTiming));
     BR_CUDA(cudaEventCreateWithFlags(&s.ev_sent, cudaEventDisableTiming));
@@ -687,6 +688,12 @@ extern "C" int bridge_dd_destroy(bridge_dd d) {
 }
 
 // which: 0 full D, 1 D_eo / D_oe (out_parity), 2 the Schur operator.
+static std::vector<bridge_lattice_s*> dd_parts(bridge_dd d) {
+  std::vector<bridge_lattice_s*> p;
+  for (auto& s : d->slabs) p.push_back(s.L);
+  return p;
+}
+
 static int dd_mult(bridge_dd d, int prec, int which, int out_parity, const double* in, double* out, int nrhs) {
   DD_BEGIN
   BR_CHECK(d != nullptr, BRIDGE_EINVAL, "NULL handle");
@@ -696,26 +703,28 @@ static int dd_mult(bridge_dd d, int prec, int which, int out_parity, const doubl
   BR_CHECK(in != nullptr && out != nullptr, BRIDGE_EINVAL, "in/out is NULL");
   BR_CHECK(out_parity == 0 || out_parity == 1, BRIDGE_EINVAL, "out_parity");
   std::lock_guard<std::mutex> lk(d->global->api_mu);
-  dd_fork(d);
-  if (which == 0) {
-    auto fin = dd_fields(d, "in", prec, BRIDGE_FULL, nrhs), fout = dd_fields(d, "out", prec, BRIDGE_FULL, nrhs);
-    dd_import(d, in, fin);
-    dd_d(d, prec, fout, fin);
-    dd_export(d, fout, out);
-  } else if (which == 1) {
-    const int q = out_parity;
-    auto fin = dd_fields(d, "hin", prec, 1 - q, nrhs), fout = dd_fields(d, "hout", prec, q, nrhs);
-    dd_import(d, in, fin);
-    dd_deo(d, prec, q, fout, fin);
-    dd_export(d, fout, out);
-  } else {
-    auto fin = dd_fields(d, "hin", prec, BRIDGE_EVEN, nrhs), fout = dd_fields(d, "hout", prec, BRIDGE_EVEN, nrhs),
-         ftmp = dd_fields(d, "htmp", prec, BRIDGE_ODD, nrhs);
-    dd_import(d, in, fin);
-    dd_dhat(d, prec, fout, fin, ftmp);
-    dd_export(d, fout, out);
-  }
-  dd_join(d);
+  with_room(d->global, [&] {
+    dd_fork(d);
+    if (which == 0) {
+      auto fin = dd_fields(d, "in", prec, BRIDGE_FULL, nrhs), fout = dd_fields(d, "out", prec, BRIDGE_FULL, nrhs);
+      dd_import(d, in, fin);
+      dd_d(d, prec, fout, fin);
+      dd_export(d, fout, out);
+    } else if (which == 1) {
+      const int q = out_parity;
+      auto fin = dd_fields(d, "hin", prec, 1 - q, nrhs), fout = dd_fields(d, "hout", prec, q, nrhs);
+      dd_import(d, in, fin);
+      dd_deo(d, prec, q, fout, fin);
+      dd_export(d, fout, out);
+    } else {
+      auto fin = dd_fields(d, "hin", prec, BRIDGE_EVEN, nrhs), fout = dd_fields(d, "hout", prec, BRIDGE_EVEN, nrhs),
+           ftmp = dd_fields(d, "htmp", prec, BRIDGE_ODD, nrhs);
+      dd_import(d, in, fin);
+      dd_dhat(d, prec, fout, fin, ftmp);
+      dd_export(d, fout, out);
+    }
+    dd_join(d);
+  }, dd_parts(d));
   BR_CUDA(cudaStreamSynchronize(d->global->stream));
   DD_END
 }
@@ -746,6 +755,11 @@ extern "C" int bridge_dd_solve_dev(bridge_dd d, const bridge_solver* prm, const 
   const bool clov = op_is_clover(d->op);
   const long V = d->global->V;
   const int max_iter = prm->max_iter > 0 ? prm->max_iter : 20000;
+  with_room(d->global, [&] {
+    for (const char* f : {"sB", "sX", "sR"}) dd_fields(d, f, P_F64, BRIDGE_FULL, 1);
+    dd_fields(d, "sTo", P_F64, BRIDGE_ODD, 1);
+    for (const char* f : {"sbh", "sr", "srh", "sp", "sv", "ss", "st", "sxe"}) dd_fields(d, f, P_F64, BRIDGE_EVEN, 1);
+  }, dd_parts(d));
   auto B = dd_fields(d, "sB", P_F64, BRIDGE_FULL, 1), X = dd_fields(d, "sX", P_F64, BRIDGE_FULL, 1),
        RF = dd_fields(d, "sR", P_F64, BRIDGE_FULL, 1), TO = dd_fields(d, "sTo", P_F64, BRIDGE_ODD, 1);
   auto bh = dd_fields(d, "sbh", P_F64, BRIDGE_EVEN, 1), r = dd_fields(d, "sr", P_F64, BRIDGE_EVEN, 1),

@@ -221,6 +221,7 @@ struct bridge_lattice_s {
   std::mutex tune_mu;
   std::map<std::string, bridge::Field> ws;  // reusable fields of the operator entry points
   bridge::Stats stats;
+  bool part = false;  // of a decomposed lattice, whose calls do not take api_mu
   std::mutex api_mu;  // serialises host entry points on one lattice
 };
 
@@ -261,7 +262,11 @@ bool fx_fits(bridge_lattice_s* L, const CloverSet* set, int flags, int* eE = nul
 struct FxCopies {
   const char *U = nullptr, *E = nullptr, *M = nullptr;
 };
-FxCopies fx_copies(bridge_lattice_s* L, CloverSet* set, int flags);
+// keep_free: bytes that are to stay free.
+FxCopies fx_copies(bridge_lattice_s* L, CloverSet* set, int flags, size_t keep_free = 0);
+// fx_release of L (whose api_mu the caller holds), its parts and every lattice
+// no call is running on; whether that freed anything.
+bool release_idle(bridge_lattice_s* L, const std::vector<bridge_lattice_s*>& parts = {});
 // Set the fixed-point mode and pointers of an FP64 launch on stream st and
 // queue the conversion of its input where copies are used.  copies: what may
 // be read on st (null: fx_copies on the lattice stream, none on others);
@@ -271,6 +276,22 @@ void set_fx_args(bridge_lattice_s* L, HopArgs& a, int flags, int red, CloverSet*
 // The lattice's scratch for hop inputs in fixed point (work on the lattice
 // stream), grown to `bytes`; null where there is no room, or in a capture.
 char* fx_scratch(bridge_lattice_s* L, size_t bytes);
+// Give the copies and the scratch of L back (the caller holds api_mu); whether
+// there were any.  Not while requests that may read them are in flight.
+bool fx_release(bridge_lattice_s* L);
+// f(), and once more after every idle lattice has given its copies back if
+// there was no memory for it: they only make things faster, and what would fit
+// without them has to fit.
+// (The caller holds api_mu of L; the parts of a decomposed one with it.)
+template <class F>
+auto with_room(bridge_lattice_s* L, F&& f, const std::vector<bridge_lattice_s*>& parts = {}) {
+  try {
+    return f();
+  } catch (const Error& e) {
+    if (e.code != BRIDGE_ENOMEM || !release_idle(L, parts)) throw;
+  }
+  return f();
+}
 // Where the FP64 application `which` (bridge_apply_op) of op on the lattice
 // stream reads copies, room for nblocks half-lattice inputs; else null.
 char* fx_input(bridge_lattice_s* L, const bridge_op& op, int which, int nblocks);

@@ -1071,7 +1071,7 @@ int bridge_mg_setup(bridge_lattice L, const bridge_op* op, const bridge_mg_param
   *out = nullptr;
   std::lock_guard<std::mutex> lk(L->api_mu);
   bridge_mg_s* g = nullptr;
-  mg_setup(L, *op, *prm, null_vectors, &g);
+  with_room(L, [&] { mg_setup(L, *op, *prm, null_vectors, &g); });
   *out = g;
   BR_MG_END
 }
@@ -1092,14 +1092,16 @@ int bridge_mg_solve(bridge_mg g, const bridge_solver* s, const double* b, double
   bridge_lattice_s* L = g->L;
   std::lock_guard<std::mutex> lk(L->api_mu);
   const size_t n = (size_t)L->V * 24;
-  DevBuf db(n * sizeof(double)), dx(n * sizeof(double));
   int status = BRIDGE_OK;
   for (int r = 0; r < nrhs; ++r) {
-    BR_CUDA(cudaMemcpyAsync(db.ptr, b + n * r, n * sizeof(double), cudaMemcpyHostToDevice, L->stream));
-    BR_CUDA(cudaMemcpyAsync(dx.ptr, x + n * r, n * sizeof(double), cudaMemcpyHostToDevice, L->stream));
     bridge_info inf;
-    mg_solve_one(g, reinterpret_cast<double*>(db.ptr), reinterpret_cast<double*>(dx.ptr), *s, inf);
-    BR_CUDA(cudaMemcpy(x + n * r, dx.ptr, n * sizeof(double), cudaMemcpyDeviceToHost));
+    with_room(L, [&] {
+      DevBuf db(n * sizeof(double)), dx(n * sizeof(double));
+      BR_CUDA(cudaMemcpyAsync(db.ptr, b + n * r, n * sizeof(double), cudaMemcpyHostToDevice, L->stream));
+      BR_CUDA(cudaMemcpyAsync(dx.ptr, x + n * r, n * sizeof(double), cudaMemcpyHostToDevice, L->stream));
+      mg_solve_one(g, reinterpret_cast<double*>(db.ptr), reinterpret_cast<double*>(dx.ptr), *s, inf);
+      BR_CUDA(cudaMemcpy(x + n * r, dx.ptr, n * sizeof(double), cudaMemcpyDeviceToHost));
+    });
     if (info) info[r] = inf;
     if (inf.status != BRIDGE_OK) status = inf.status;
   }
@@ -1119,7 +1121,7 @@ int bridge_mg_solve_dev(bridge_mg g, const bridge_solver* s, const double* b, do
   int status = BRIDGE_OK;
   for (int r = 0; r < nrhs; ++r) {
     bridge_info inf;
-    mg_solve_one(g, b + n * r, x + n * r, *s, inf);
+    with_room(L, [&] { mg_solve_one(g, b + n * r, x + n * r, *s, inf); });
     if (info) info[r] = inf;
     if (inf.status != BRIDGE_OK) status = inf.status;
   }
@@ -1137,10 +1139,12 @@ int bridge_mg_apply(bridge_mg g, int which, const double* in, double* out) {
   const bool fine_out = which == BRIDGE_MG_PROLONG || which == BRIDGE_MG_SAP || which == BRIDGE_MG_CYCLE;
   const size_t nf = (size_t)L->V * 24, ncd = (size_t)g->nc * 2;
   const size_t nin = fine_in ? nf : ncd, nout = fine_out ? nf : ncd;
-  DevBuf din(nin * sizeof(double)), dout(nout * sizeof(double));
-  BR_CUDA(cudaMemcpy(din.ptr, in, nin * sizeof(double), cudaMemcpyHostToDevice));
-  mg_apply(g, which, reinterpret_cast<double*>(din.ptr), reinterpret_cast<double*>(dout.ptr));
-  BR_CUDA(cudaMemcpy(out, dout.ptr, nout * sizeof(double), cudaMemcpyDeviceToHost));
+  with_room(L, [&] {
+    DevBuf din(nin * sizeof(double)), dout(nout * sizeof(double));
+    BR_CUDA(cudaMemcpy(din.ptr, in, nin * sizeof(double), cudaMemcpyHostToDevice));
+    mg_apply(g, which, reinterpret_cast<double*>(din.ptr), reinterpret_cast<double*>(dout.ptr));
+    BR_CUDA(cudaMemcpy(out, dout.ptr, nout * sizeof(double), cudaMemcpyDeviceToHost));
+  });
   BR_MG_END
 }
 

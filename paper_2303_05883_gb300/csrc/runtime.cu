@@ -247,7 +247,7 @@ bool fx_fits(bridge_lattice_s* L, const CloverSet* set, int flags, int* eE, int*
 // eighth of what is free, to leave the memory to the fields of a solve (up to
 // 4 KB a site, seven link copies) where it is scarce.  What the library's pool
 // holds unused is free.
-static bool fx_room(size_t bytes) {
+static bool fx_room(size_t bytes, size_t keep_free) {
   int dev = 0;
   cudaMemPool_t pool;
   uint64_t held = 0, used = 0;
@@ -257,15 +257,15 @@ static bool fx_room(size_t bytes) {
   }
   cudaGetLastError();
   const size_t idle = held > used ? (size_t)(held - used) : 0;
-  if (bytes <= idle / 8) return true;
+  if (bytes <= idle / 8 && bytes + keep_free <= idle) return true;
   size_t free_b = 0, total_b = 0;
   BR_CUDA(cudaMemGetInfo(&free_b, &total_b));
-  return bytes <= (free_b + idle) / 8;
+  return bytes <= (free_b + idle) / 8 && bytes + keep_free <= free_b + idle;
 }
 
 // A buffer, from the pool in the order of the lattice stream if pooled, or null.
-static std::unique_ptr<DevBuf> fx_buffer(bridge_lattice_s* L, size_t bytes, bool pooled) {
-  if (!fx_room(bytes)) return nullptr;
+static std::unique_ptr<DevBuf> fx_buffer(bridge_lattice_s* L, size_t bytes, bool pooled, size_t keep_free = 0) {
+  if (!fx_room(bytes, keep_free)) return nullptr;
   try {
     return std::unique_ptr<DevBuf>(new DevBuf(bytes, L->stream, pooled));
   } catch (const Error&) {
@@ -284,11 +284,11 @@ static void fx_convert(bridge_lattice_s* L, const char* src, char* dst, int nb, 
 
 // (A clover set may outlive the stream of its lattice: its copies are not of
 // the pool.)
-static const char* fx_clover(bridge_lattice_s* L, CloverSet& set, bool inverse) {
+static const char* fx_clover(bridge_lattice_s* L, CloverSet& set, bool inverse, size_t keep_free) {
   std::unique_ptr<DevBuf>& buf = set.fx[inverse];
   if (!buf) {
     const long cbb = clover_block_bytes(P_F64, L->vh);
-    auto to = fx_buffer(L, (size_t)(2 * cbb), false);
+    auto to = fx_buffer(L, (size_t)(2 * cbb), false, keep_free);
     if (!to) return nullptr;
     fx_convert(L, (inverse ? set.Tinv : set.T)[P_F64]->ptr, to->ptr, 2, cbb, 36 * L->vh, fx_clov_exponent(set.top[inverse]));
     buf = std::move(to);
@@ -296,13 +296,13 @@ static const char* fx_clover(bridge_lattice_s* L, CloverSet& set, bool inverse) 
   return buf->ptr;
 }
 
-FxCopies fx_copies(bridge_lattice_s* L, CloverSet* set, int flags) {
+FxCopies fx_copies(bridge_lattice_s* L, CloverSet* set, int flags, size_t keep_free) {
   FxCopies c;
   if (capturing(L->stream)) return c;
   {
     std::lock_guard<std::mutex> lk(L->fx_mu);
     const long lbb = link_block_bytes(P_F64, L->vh);
-    if (!L->gauge_fx) L->gauge_fx = fx_buffer(L, (size_t)(8 * lbb), true);
+    if (!L->gauge_fx) L->gauge_fx = fx_buffer(L, (size_t)(8 * lbb), true, keep_free);
     if (L->gauge_fx && !L->gauge_fx_made) {
       fx_convert(L, L->gauge[P_F64]->ptr, L->gauge_fx->ptr, 8, lbb, 9 * L->vh, 0);
       L->gauge_fx_made = true;
@@ -311,9 +311,31 @@ FxCopies fx_copies(bridge_lattice_s* L, CloverSet* set, int flags) {
   }
   if (!c.U || !(flags & (F_E_CLOV | F_SELF_CLOV))) return c;
   std::lock_guard<std::mutex> lk(set->mu);
-  if (flags & F_SELF_CLOV) c.M = fx_clover(L, *set, false);
-  if (flags & F_E_CLOV) c.E = fx_clover(L, *set, true);
+  if (flags & F_SELF_CLOV) c.M = fx_clover(L, *set, false, keep_free);
+  if (flags & F_E_CLOV) c.E = fx_clover(L, *set, true, keep_free);
   return c;
+}
+
+bool fx_release(bridge_lattice_s* L) {
+  if (L->in_flight.load() != 0) return false;
+  BR_CUDA(cudaStreamSynchronize(L->stream));
+  bool any = L->fx_scratch || L->gauge_fx;
+  L->fx_scratch.reset();
+  {
+    std::lock_guard<std::mutex> lk(L->fx_mu);
+    L->gauge_fx.reset();
+    L->gauge_fx_made = false;
+  }
+  std::lock_guard<std::mutex> lk(L->clover_mu);
+  for (auto& s : L->clovers) {
+    std::lock_guard<std::mutex> ls(s->mu);
+    for (auto& b : s->fx) {
+      any = any || b;
+      b.reset();
+    }
+  }
+  BR_CUDA(cudaStreamSynchronize(L->stream));
+  return any;
 }
 
 char* fx_scratch(bridge_lattice_s* L, size_t need) {

@@ -178,13 +178,20 @@ struct Engine {
     try {
       BR_CUDA(cudaStreamCreateWithPriority(&r->st, cudaStreamNonBlocking, priority_for(r)));
       const size_t n = r->nvals * sizeof(double);
-      r->b_dev.reset(new DevBuf(n, r->st, true));
-      r->x_dev.reset(new DevBuf(n, r->st, true));
-      BR_CUDA(cudaMemsetAsync(r->x_dev->ptr, 0, n, r->st));
+      size_t keep_free;  // what the budget may still admit
+      {
+        std::lock_guard<std::mutex> lk(mu);
+        keep_free = budget > used ? budget - used : 0;
+      }
       {
         std::lock_guard<std::mutex> lk(r->L->api_mu);
-        r->solve.reset(new SolveState(r->L, r->op, r->prm, r->nrhs, r->st, reinterpret_cast<double*>(r->b_dev->ptr),
-                                      reinterpret_cast<double*>(r->x_dev->ptr)));
+        with_room(r->L, [&] {
+          r->b_dev.reset(new DevBuf(n, r->st, true));
+          r->x_dev.reset(new DevBuf(n, r->st, true));
+          BR_CUDA(cudaMemsetAsync(r->x_dev->ptr, 0, n, r->st));
+          r->solve.reset(new SolveState(r->L, r->op, r->prm, r->nrhs, r->st, reinterpret_cast<double*>(r->b_dev->ptr),
+                                        reinterpret_cast<double*>(r->x_dev->ptr), keep_free));
+        });
       }
       r->t_admit = now_seconds();
       r->phase.store(PH_UPLOAD);

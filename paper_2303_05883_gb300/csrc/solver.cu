@@ -93,7 +93,7 @@ size_t solve_footprint(const bridge_lattice_s* L, const bridge_solver& prm, int 
 }
 
 SolveState::SolveState(bridge_lattice_s* L, const bridge_op& op, const bridge_solver& prm, int nrhs, cudaStream_t st,
-                       const double* b_dev, double* x_dev)
+                       const double* b_dev, double* x_dev, size_t keep_free)
     : L_(L), op_(op), prm_(prm), nrhs_(nrhs), st_(st), b_dev_(b_dev), x_dev_(x_dev) {
   t0_ = std::chrono::steady_clock::now();
   P_ = inner_prec(prm_);
@@ -171,7 +171,7 @@ SolveState::SolveState(bridge_lattice_s* L, const bridge_op& op, const bridge_so
     clover_ptr(L_, *clov_, P_F64, false);
   }
   const int fl = clover_ ? F_SELF_CLOV | (P_ == P_F64 ? F_E_CLOV : 0) : 0;
-  if (fx_fits(L_, clov_.get(), fl)) fx_ = fx_copies(L_, clov_.get(), fl);
+  if (fx_fits(L_, clov_.get(), fl)) fx_ = fx_copies(L_, clov_.get(), fl, keep_free);
   if (st_ != L_->stream) BR_CUDA(cudaStreamSynchronize(L_->stream));
 }
 

@@ -45,8 +45,9 @@ class SolveState {
  public:
   // b_dev / x_dev: canonical FP64 full-lattice fields on the device (nrhs of
   // each).  x_dev holds the initial guess and receives the solution.
+  // keep_free: bytes that copies of the operands leave free.
   SolveState(bridge_lattice_s* L, const bridge_op& op, const bridge_solver& prm, int nrhs, cudaStream_t st,
-             const double* b_dev, double* x_dev);
+             const double* b_dev, double* x_dev, size_t keep_free = 0);
   ~SolveState();
 
   // Queue whatever can be queued without blocking; true once finished.

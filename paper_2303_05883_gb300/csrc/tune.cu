@@ -299,9 +299,9 @@ extern "C" int bridge_tune(bridge_lattice L, const bridge_op* op, int prec, int 
     std::lock_guard<std::mutex> lk(L->api_mu);
     if (op->kind == BRIDGE_MOBIUS) {
       check_mobius(*op);
-      tune_dwf_kernels(L, *op, prec, nrhs);
+      with_room(L, [&] { tune_dwf_kernels(L, *op, prec, nrhs); });
     } else {
-      tune_solver_kernels(L, *op, prec, nrhs);
+      with_room(L, [&] { tune_solver_kernels(L, *op, prec, nrhs); });
     }
   } catch (const Error& e) {
     set_error(e.code, e.msg);

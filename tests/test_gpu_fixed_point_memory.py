@@ -77,3 +77,26 @@ def test_the_same_bits_without_memory_for_copies(api, kind):
         got = results(api, kind)
     for a, b in zip(got, want):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("spare", [8 << 20, -LINK_COPY // 2])
+@pytest.mark.parametrize("kind", ["wilson", "staggered"])
+def test_a_call_that_fits_without_copies_and_scratch_runs(api, kind, spare):
+    """Room for the input and output fields of a call and little else, not for scratch; then not even for them,
+    until the lattice gives back its link copy and the scratch of a smaller call."""
+    from paper_2303_05883_gb300 import _abi
+
+    U, nrhs = synth.gauge_field(DIMS, 0.3, 2), 24
+    site = (6 if kind == "staggered" else 24) * 8
+    op = api.make_staggered(0.2) if kind == "staggered" else api.make_op(kind, 0.11, 0.0)
+    f = torch.randn((nrhs, U.shape[1]) + ((3,) if kind == "staggered" else (4, 3)), dtype=torch.complex128, device="cuda")
+    L = api.Lattice(DIMS)
+    L.upload(U, op)
+    want = torch.cat([L.D(op, f[k : k + 1]) for k in range(nrhs)])
+    got = torch.empty_like(f)
+    with Scarce(2 * nrhs * U.shape[1] * site + spare):
+        _abi.check(_abi.load().bridge_mult_D_dev(L.handle, ctypes.byref(op), 0, ctypes.c_void_p(f.data_ptr()),
+                                                 ctypes.c_void_p(got.data_ptr()), nrhs), "bridge_mult_D_dev")
+        api.bridge_sync(L.handle)
+    assert torch.equal(got, want)
+    L.close()
