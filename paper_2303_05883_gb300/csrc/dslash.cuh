@@ -534,6 +534,7 @@ bool launch_hop<P_BF16>(int flags, int red, const HopArgs& a, int block, cudaStr
 #define BRIDGE_HOP_TILE_CASES(X)                                                        \
   X(F_SELF, R_NONE) X(F_SELF | F_E_CLOV, R_NONE) X(F_SELF | F_SELF_CLOV, R_NONE)        \
   X(F_AUX, R_NONE) X(F_AUX | F_E_CLOV, R_NONE) X(F_SELF, R_NORM) X(F_SELF | F_E_CLOV, R_NORM) X(F_SELF | F_G5, R_NONE)
+// (FP64: the kernel on the FP64 pipe; in fixed point there is one, for any variant.)
 bool hop_has_variant(int prec, int flags, int red, int variant);
 // Right-hand sides covered by one block group of a variant: 1 for v < 6, NR
 // for the NR-per-thread kernels (v = 6, 7, 8) and up to 12 for the

@@ -684,7 +684,7 @@ bool hop_has_variant(int prec, int flags, int red, int variant) {
   const bool shared = false BRIDGE_HOP_SHARED_CASES(BRIDGE_HOP_IS), tile = false BRIDGE_HOP_TILE_CASES(BRIDGE_HOP_IS);
 #undef BRIDGE_HOP_IS
   if (variant == 0) return true;
-  if (prec == P_F64) return false;
+  if (prec == P_F64) return variant < 6 && budget;
   if (variant < 6) return budget || (variant == 4 && apply);
   if (variant < 9) return shared;
   if (variant < 11) return shared || tile;
@@ -707,7 +707,7 @@ bool hop_has_variant(int prec, int flags, int red, int variant) {
 //     read-once operands past L1, 256-thread blocks (pass 2, 32^3 x 64: F32
 //     186 -> 175, 3 RHS 429 -> 360, F16 136 -> 130); on 16^3 x 32 it is slower.
 static int default_hop_variant(int prec, int flags, int red, long vh, int nrhs, bool mapped) {
-  if (mapped) return 0;
+  if (prec == P_F64 || mapped) return 0;
   const int per_block = (nrhs + (nrhs + 11) / 12 - 1) / ((nrhs + 11) / 12);  // right-hand sides of a tile block
   if (((per_block >= 4 && vh >= (1L << 18)) || (per_block >= 6 && vh >= (1L << 16))) &&
       hop_has_variant(prec, flags, red, 9))

@@ -123,8 +123,9 @@ static std::vector<Candidate> candidates(long vh, int nrhs, const std::vector<in
   return out;
 }
 
-static std::vector<int> hop_variants(int prec, int flags, int red, int nrhs) {
+static std::vector<int> hop_variants(int prec, int flags, int red, int nrhs, bool fixed_point) {
   std::vector<int> v = {0};
+  if (fixed_point) return v;
   for (int k = 1; k < HOP_NVARIANT; ++k)
     if (hop_has_variant(prec, flags, red, k) && (k < 6 || (k < 9 ? hop_variant_rpt(k) <= nrhs : nrhs >= 2))) v.push_back(k);
   return v;
@@ -213,7 +214,7 @@ void tune_solver_kernels(bridge_lattice_s* L, const bridge_op& op, int prec, int
     };
     float best = 1e30f;
     Candidate pick{128, 0, 0};
-    for (const auto& c : candidates(vh, nrhs, hop_variants(prec, v.flags, v.red, nrhs), occ)) {
+    for (const auto& c : candidates(vh, nrhs, hop_variants(prec, v.flags, v.red, nrhs, a.fx != FX_OFF), occ)) {
       a.nblk = c.nblk;
       const float ms =
           time_launches([&] { launch_hop_any(prec, v.flags, v.red, a, c.block, st, nullptr, c.variant); }, st, ea, eb, 5);

@@ -1,6 +1,7 @@
 """The launch table names kernels that exist: a recorded variant is one its
 (flags, reduction) pair is instantiated for."""
 
+import numpy as np
 import pytest
 
 import synth
@@ -41,3 +42,42 @@ def test_tuning_the_preparation_tries_its_own_kernels(api, nrhs):
     L, op, key = lattice(api, (8, 8, 8, 16))
     api.bridge_tune(L.handle, op, "f16", nrhs)
     assert api.bridge_tune_table(L.handle)[f"hop/2/12/0/{key}/{nrhs}"][2] in ((0,) if nrhs == 1 else (0, 9, 10))
+
+
+def tuned(api, capfd, monkeypatch, scale):
+    """The variants that tuning FP64 tries for D_eo on links scaled by `scale`."""
+    dims = (4, 4, 4, 8)
+    L = api.Lattice(dims)
+    op = api.make_op("wilson", 0.12 / scale, 0.0)
+    L.upload(scale * synth.gauge_field(dims, 0.2, 2), op)
+    monkeypatch.setenv("BRIDGE_TUNE_VERBOSE", "1")
+    capfd.readouterr()
+    api.bridge_tune(L.handle, op, "f64", 1)
+    lines = [x.split() for x in capfd.readouterr().err.splitlines() if x.startswith("tune hop/0/0/0/")]
+    return {int(x[x.index("variant") + 1].rstrip(":")) for x in lines}
+
+
+def test_tuning_fp64_arithmetic_tries_its_variants(api, capfd, monkeypatch):
+    """Links above 1 run on the FP64 pipe, which has the register-budget variants; in fixed point there is one kernel."""
+    assert tuned(api, capfd, monkeypatch, 2.0) == {0, 1, 2, 3, 4, 5}
+    assert tuned(api, capfd, monkeypatch, 1.0) == {0}
+
+
+@pytest.mark.parametrize("variant", [3, 5, 9])
+@pytest.mark.parametrize("scale", [1.0, 2.0])
+def test_fp64_entries_of_any_variant_run(api, variant, scale):
+    """Table lines of FP64 keys, whether their hops run in fixed point or not."""
+    dims = (4, 4, 4, 8)
+    psi = synth.gaussian_spinor(dims, 4)
+    got = []
+    for pin in (False, True):
+        L = api.Lattice(dims)
+        op = api.make_op("wilson", 0.12 / scale, 0.0)
+        L.upload(scale * synth.gauge_field(dims, 0.2, 2), op)
+        for key in ("0/0", "1/0", "1/2", "1/3", "8/0", "9/1"):
+            if pin:
+                api.bridge_tune_set(L.handle, f"hop/0/{key}/4x4x4x8/1", 64, 2, variant)
+        x, info = L.solve(op, psi, api.make_solver(tol=1e-10, mixed=0))
+        assert info[0]["status"] == 0
+        got.append((L.D(op, psi), L.Dhat(op, psi[:256])))
+    assert all(np.array_equal(a, b) for a, b in zip(*got))
