@@ -236,6 +236,9 @@ void note_launch(bridge_lattice_s* L, int cls, double bytes, double flops, cudaS
 LaunchShape shape_for(bridge_lattice_s* L, const std::string& key, long vh, int nrhs,
                       const std::function<int(int)>& occ, int variant = 0, bool cover_once = false);
 
+// What an untuned launch of a hop takes (nblk not capped at the lattice yet).
+LaunchShape default_hop_shape(int prec, int flags, int red, const HopArgs& a, bool mapped);
+
 // Algorithmic cost of one hop launch: bytes and flops per right-hand side
 // (spinors) and shared by all right-hand sides (links, clover blocks).
 struct HopCost {

@@ -54,9 +54,12 @@ char* scratch_on_current_device() {
   return g_scratch_ptr[dev];
 }
 
-// Launch shape without touching the lattice's shape table: the tuned entry
-// if one exists, else a persistent grid from the occupancy query.
-LaunchShape shape_readonly(bridge_lattice_s* L, const std::string& key, int nrhs, const std::function<int(int)>& occ) {
+// Launch shape of a hop without touching the lattice's shape table: the tuned
+// entry if one exists, else what an untuned launch takes.
+LaunchShape shape_readonly(bridge_lattice_s* L, int prec, int flags, const HopArgs& a) {
+  const std::string key = "hop/" + std::to_string(prec) + "/" + std::to_string(flags) + "/0/" +
+                          std::to_string(L->dims[0]) + "x" + std::to_string(L->dims[1]) + "x" +
+                          std::to_string(L->dims[2]) + "x" + std::to_string(L->dims[3]) + "/" + std::to_string(a.nrhs);
   LaunchShape s;
   bool found = false;
   {
@@ -67,24 +70,20 @@ LaunchShape shape_readonly(bridge_lattice_s* L, const std::string& key, int nrhs
       found = true;
     }
   }
-  if (!found) {
-    s.block = 128;
-    const int per_sm = occ(s.block);
-    s.nblk = std::max(1, sm_count() * (per_sm > 0 ? per_sm : 4) / std::max(1, nrhs));
-  }
+  if (!found) s = default_hop_shape(prec, flags, R_NONE, a, false);
   const long cover = (L->vh + s.block - 1) / s.block;
   if (s.nblk <= 0 || s.nblk > cover) s.nblk = (int)cover;
   return s;
 }
 
-// The clover inverse of this lattice for kcsw in precision prec, if it was
-// built before; nullptr otherwise (nothing is built here).
-const char* existing_clover_inverse(bridge_lattice_s* L, double kcsw, int prec) {
+// The clover set of this lattice for kcsw, if its inverse in precision prec
+// was built before; nullptr otherwise (nothing is built here).
+std::shared_ptr<CloverSet> existing_clover(bridge_lattice_s* L, double kcsw, int prec) {
   std::lock_guard<std::mutex> lk(L->clover_mu);
   for (auto& s : L->clovers)
     if (s->kcsw == kcsw) {
       std::lock_guard<std::mutex> lk2(s->mu);
-      return s->Tinv[prec] ? s->Tinv[prec]->ptr : nullptr;
+      return s->Tinv[prec] ? s : nullptr;
     }
   return nullptr;
 }
@@ -110,10 +109,10 @@ extern "C" int bridge_mult_Dhat_noalloc(bridge_lattice L, const bridge_op* op, i
     BR_CHECK(L->have_gauge && L->gauge[prec], BRIDGE_ESTATE,
              "links in this precision not built yet: apply the operator once with bridge_mult_Dhat first");
     const bool clov = op_is_clover(*op);
-    const char* tinv = nullptr;
+    std::shared_ptr<CloverSet> set;
     if (clov) {
-      tinv = existing_clover_inverse(L, op_kcsw(*op), prec);
-      BR_CHECK(tinv != nullptr, BRIDGE_ESTATE,
+      set = existing_clover(L, op_kcsw(*op), prec);
+      BR_CHECK(set != nullptr, BRIDGE_ESTATE,
                "clover term for this kappa*c_sw and precision not built yet: apply the operator once first");
     }
     char* scratch = scratch_on_current_device();
@@ -141,9 +140,8 @@ extern "C" int bridge_mult_Dhat_noalloc(bridge_lattice L, const bridge_op* op, i
     a.nrhs = nrhs;
     for (int k = 0; k < 4; ++k) a.bc[k] = op->bc[k];
     a.gauge = L->gauge[prec]->ptr;
-    a.clovE = tinv;
-    const std::string dims = std::to_string(L->dims[0]) + "x" + std::to_string(L->dims[1]) + "x" +
-                             std::to_string(L->dims[2]) + "x" + std::to_string(L->dims[3]);
+    a.clovE = set ? set->Tinv[prec]->ptr : nullptr;
+    const FxCopies none;  // FP64: without copies and scratch, to the same bits
     // pass 1: tmp_o = T_oo^-1 (-kappa H_oe in_e)
     const int f1 = clov ? F_E_CLOV : 0;
     a.out_parity = 1;
@@ -152,12 +150,8 @@ extern "C" int bridge_mult_Dhat_noalloc(bridge_lattice L, const bridge_op* op, i
     a.out_rs = block;
     a.in = f_in;
     a.in_rs = block;
-    LaunchShape s1 = shape_readonly(L, "hop/" + std::to_string(prec) + "/" + std::to_string(f1) + "/0/" + dims + "/" +
-                                           std::to_string(nrhs), nrhs, [&](int b) {
-      int n = 0;
-      launch_hop_any(prec, f1, R_NONE, a, b, st, &n);
-      return n;
-    });
+    if (prec == P_F64) set_fx_args(L, a, f1, R_NONE, set.get(), &none, nullptr, st);
+    const LaunchShape s1 = shape_readonly(L, prec, f1, a);
     a.nblk = s1.nblk;
     BR_CHECK(launch_hop_any(prec, f1, R_NONE, a, s1.block, st, nullptr, launch_variant(s1)), BRIDGE_EINVAL, "hop variant");
     // pass 2: out_e = in_e + kappa T_ee^-1 H_eo tmp_o
@@ -169,12 +163,8 @@ extern "C" int bridge_mult_Dhat_noalloc(bridge_lattice L, const bridge_op* op, i
     a.in = f_tmp;
     a.self = f_in;
     a.self_rs = block;
-    LaunchShape s2 = shape_readonly(L, "hop/" + std::to_string(prec) + "/" + std::to_string(f2) + "/0/" + dims + "/" +
-                                           std::to_string(nrhs), nrhs, [&](int b) {
-      int n = 0;
-      launch_hop_any(prec, f2, R_NONE, a, b, st, &n);
-      return n;
-    });
+    if (prec == P_F64) set_fx_args(L, a, f2, R_NONE, set.get(), &none, nullptr, st);
+    const LaunchShape s2 = shape_readonly(L, prec, f2, a);
     a.nblk = s2.nblk;
     BR_CHECK(launch_hop_any(prec, f2, R_NONE, a, s2.block, st, nullptr, launch_variant(s2)), BRIDGE_EINVAL, "hop variant");
 

@@ -131,6 +131,17 @@ void note_launch(bridge_lattice_s* L, int cls, double bytes, double flops, cudaS
   }
 }
 
+static LaunchShape default_shape(int nrhs, const std::function<int(int)>& occ, int variant, bool cover_once) {
+  LaunchShape s;
+  s.variant = variant;
+  s.block = variant == 4 && !cover_once ? 256 : 128;
+  const int per_sm = occ ? occ(s.block) : 0;
+  const long resident = (long)sm_count() * (per_sm > 0 ? per_sm : 4);
+  const int groups = (nrhs + hop_variant_rpt(variant) - 1) / hop_variant_rpt(variant);
+  s.nblk = variant == 4 && cover_once ? 0 : (int)std::max<long>(1, resident / std::max(1, groups));
+  return s;
+}
+
 LaunchShape shape_for(bridge_lattice_s* L, const std::string& key, long vh, int nrhs,
                       const std::function<int(int)>& occ, int variant, bool cover_once) {
   std::lock_guard<std::mutex> lk(L->tune_mu);
@@ -139,12 +150,7 @@ LaunchShape shape_for(bridge_lattice_s* L, const std::string& key, long vh, int 
   if (it != L->tuned.end()) {
     s = it->second;
   } else {
-    s.variant = variant;
-    s.block = variant == 4 && !cover_once ? 256 : 128;
-    const int per_sm = occ ? occ(s.block) : 0;
-    const long resident = (long)sm_count() * (per_sm > 0 ? per_sm : 4);
-    const int groups = (nrhs + hop_variant_rpt(variant) - 1) / hop_variant_rpt(variant);
-    s.nblk = variant == 4 && cover_once ? 0 : (int)std::max<long>(1, resident / std::max(1, groups));
+    s = default_shape(nrhs, occ, variant, cover_once);
     L->tuned[key] = s;
   }
   const long cover = (vh + s.block - 1) / s.block;
@@ -412,6 +418,20 @@ static std::string dims_key(const bridge_lattice_s* L) {
          std::to_string(L->dims[3]);
 }
 
+// Resident blocks per SM of an untuned launch, by its block size.
+static std::function<int(int)> hop_occupancy(int prec, int flags, int red, const HopArgs& a, int variant) {
+  return [=, &a](int block) {
+    int n = 0;
+    launch_hop_any(prec, flags, red, a, block, nullptr, &n, variant + (variant == 9 || variant == 10 ? HOP_TILE_WIDE : 0));
+    return n;
+  };
+}
+
+LaunchShape default_hop_shape(int prec, int flags, int red, const HopArgs& a, bool mapped) {
+  const int variant = default_hop_variant(prec, flags, red, a.g.vh, a.nrhs, mapped);
+  return default_shape(a.nrhs, hop_occupancy(prec, flags, red, a, variant), variant, red == R_NONE);
+}
+
 void run_hop(bridge_lattice_s* L, HopCall c, cudaStream_t st) {
   HopArgs a;
   std::memset(&a, 0, sizeof(a));
@@ -450,11 +470,8 @@ void run_hop(bridge_lattice_s* L, HopCall c, cudaStream_t st) {
   const std::string key = "hop/" + std::to_string(c.prec) + "/" + std::to_string(c.flags) + "/" +
                           std::to_string(c.red) + "/" + dims_key(L) + "/" + std::to_string(c.nrhs);
   const int variant = default_hop_variant(c.prec, c.flags, c.red, L->vh, c.nrhs, c.site_map != nullptr);
-  LaunchShape sh = shape_for(L, key, L->vh, c.nrhs, [&](int block) {
-    int n = 0;
-    launch_hop_any(c.prec, c.flags, c.red, a, block, st, &n, variant + (variant == 9 || variant == 10 ? HOP_TILE_WIDE : 0));
-    return n;
-  }, variant, c.red == R_NONE);
+  LaunchShape sh = shape_for(L, key, L->vh, c.nrhs, hop_occupancy(c.prec, c.flags, c.red, a, variant), variant,
+                             c.red == R_NONE);
   a.nblk = sh.nblk;
   if (c.red != R_NONE && a.red.partials == nullptr) {
     // a fixed-point launch takes up to one block for 64 sites

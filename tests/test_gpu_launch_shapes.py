@@ -81,3 +81,31 @@ def test_fp64_entries_of_any_variant_run(api, variant, scale):
         assert info[0]["status"] == 0
         got.append((L.D(op, psi), L.Dhat(op, psi[:256])))
     assert all(np.array_equal(a, b) for a, b in zip(*got))
+
+
+@pytest.mark.parametrize("kind", ["wilson", "clover"])
+@pytest.mark.parametrize("prec,nrhs", [("f64", 1), ("f32", 1), ("f16", 6)])
+def test_the_call_without_allocations_gives_the_same_bits(api, kind, prec, nrhs):
+    """bridge_mult_Dhat_noalloc against bridge_mult_Dhat, whichever came first."""
+    import torch
+
+    dims = (8, 8, 8, 16)
+    L, op, _ = lattice(api, dims, kind)
+    psi = torch.from_numpy(synth.gaussian_spinor(dims, 4, nrhs=nrhs)[:, :4096].copy()).cuda()
+    L.Dhat(op, psi[:1], prec)  # builds the operands
+    got = [torch.empty_like(psi) for _ in range(2)]
+    for out in got:
+        dhat_noalloc(api, L, op, prec, psi, out, nrhs)
+        want = L.Dhat(op, psi, prec)
+    assert torch.equal(got[0], want) and torch.equal(got[1], want)
+
+
+def dhat_noalloc(api, L, op, prec, psi, out, nrhs):
+    from ctypes import byref, c_void_p
+
+    from paper_2303_05883_gb300 import _abi
+
+    fn = _abi.load().bridge_mult_Dhat_noalloc
+    _abi.check(fn(L.handle, byref(op), {"f64": 0, "f32": 1, "f16": 2}[prec], c_void_p(psi.data_ptr()),
+                  c_void_p(out.data_ptr()), nrhs), "bridge_mult_Dhat_noalloc")
+    api.bridge_sync(L.handle)
