@@ -37,11 +37,12 @@
 // for Wilson, 1.8e-16 (1.9e-16) for clover.
 //
 // Measured (full clover D, one parity of 24^3 x 48, one right-hand side): FP64
-// kernel 780 us = 0.81 TFLOP/s, its pipe's limit; here 242 us = 3.2 TB/s plus
-// 26 us for the input's conversion; the FP64 residual of 32^3 x 64 2.46 ms ->
-// 0.81 ms a parity.  Bound by issue: 6800 instructions a warp of 16 sites at
-// 0.5 of the issue slots, sixteen warps an SM waiting on loads and on the
-// fixed latency of the integer chains; DRAM at 0.4 of its rate.
+// kernel 780 us = 0.81 TFLOP/s, its pipe's limit; here 248 us = 3.1 TB/s; the
+// FP64 residual of 32^3 x 64 2.46 ms -> 0.83 ms a parity.  Bound by latency: 7100
+// instructions a warp of 16 sites at half of the issue slots, because 128
+// registers (and 180-420 bytes of spills a thread, 2.6 % of the instructions)
+// leave sixteen warps an SM, which wait on loads and on the fixed latency of the
+// integer chains; DRAM at 0.42 of the copy rate.
 //
 // Other sites where fixed point does not apply -- a neighbour component that
 // is not finite, or within 2^128 of the ends of the FP64 range -- are computed

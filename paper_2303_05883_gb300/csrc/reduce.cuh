@@ -10,10 +10,10 @@
 // What bounds it is latency on the FP64 pipe (2 lanes a clock): a launch with
 // three dot products took 7.6 us where the same launch without took 2.4, 27 us
 // with twelve right-hand sides.  Hence the merged warp sums, one value a lane
-// over the partials, a warp for each right-hand side,
-// and nothing at all once every solve has ended.  Solves against the previous
-// tree: 8^4 4.94 -> 3.51 ms, 32^3 x 64 173 -> 167 ms, Moebius 16^3 x 32 x 16
-// 202 -> 198 ms, multigrid on 16^3 x 32 30.1 -> 26.6 ms.
+// over the partials, a warp for each right-hand side, and nothing at all once
+// every solve has ended.  Solves without and with these: 8^4 4.94 -> 3.51 ms
+// (one division a quotient; two, as the range of the quotients needs, add 0.05),
+// 32^3 x 64 173 -> 167 ms, Moebius 16^3 x 32 x 16 202 -> 198 ms.
 #pragma once
 
 #include "common.cuh"

@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(256) stag_hop_kernel(const StagArgs a) {
 // three IMAD.WIDE a hop; a site has nothing to project or reconstruct, so one
 // thread a site keeps its sum, a hop's rows and both hops' loads of a direction
 // in 128 registers.  Measured (one parity of 32^4): FP64 kernel 340 us, at the
-// FP64 pipe's limit (0.90 TFLOP/s); here 127 us = 5.3 TB/s, 0.79 of HBM.
+// FP64 pipe's limit (0.90 TFLOP/s); here 130 us = 5.2 TB/s, 0.77 of the copy rate.
 BR_HD long stag_fx_block_bytes(long vh) { return pad256(52 * vh); }
 constexpr int SFX_THREADS = 128;
 
