@@ -280,7 +280,8 @@ void set_fx_args(bridge_lattice_s* L, HopArgs& a, int flags, int red, CloverSet*
 // stream), grown to `bytes`; null where there is no room, or in a capture.
 char* fx_scratch(bridge_lattice_s* L, size_t bytes);
 // Give the copies and the scratch of L back (the caller holds api_mu); whether
-// there were any.  Not while requests that may read them are in flight.
+// there were any.  Not while requests that may read them are in flight, or its
+// stream is being captured.
 bool fx_release(bridge_lattice_s* L);
 // f(), and once more after every idle lattice has given its copies back if
 // there was no memory for it: they only make things faster, and what would fit

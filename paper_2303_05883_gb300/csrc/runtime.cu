@@ -323,7 +323,8 @@ FxCopies fx_copies(bridge_lattice_s* L, CloverSet* set, int flags, size_t keep_f
 }
 
 bool fx_release(bridge_lattice_s* L) {
-  if (L->in_flight.load() != 0) return false;
+  // (a stream in a capture cannot be waited for)
+  if (L->in_flight.load() != 0 || capturing(L->stream)) return false;
   BR_CUDA(cudaStreamSynchronize(L->stream));
   bool any = L->fx_scratch || L->gauge_fx;
   L->fx_scratch.reset();
